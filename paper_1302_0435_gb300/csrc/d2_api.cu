@@ -268,6 +268,7 @@ SolveCfg solve_cfg(const d2_ctx* c, int mode, int mmax) {
   s.sms = c->sms;
   s.start = start_default(c);
   s.certify = mode == 1 && c->cfg.certify == D2_CERTIFY_ALL;
+  s.lanes = c->cfg.start_rule == D2_START_AUTO;
   return s;
 }
 
@@ -420,34 +421,35 @@ unsigned blocks_for(long long n) {
 
 namespace {
 
-// Object bins by the nodes per lane their trees need (see d2k::bin_objects),
-// as a stable partition: order[start[b] .. start[b+1]) are bin b's objects
+// Objects sorted by support count (see d2k::bin_objects), as a stable
+// partition: order[start[b] .. start[b+1]) are the objects of b + 1 supports
 // in increasing index.  start stays on the device (the solver launches read
-// their bin's range there); the host copy hstart is read only when needed
+// their range there); the host copy hstart is read only when needed
 // (autotuning, tensor-core chunks), which waits.
 struct Bins {
   int* order = nullptr;
   const long long* start = nullptr;
-  long long hstart[5] = {0, 0, 0, 0, 0};
+  long long hstart[d2k::kSizeBins + 1] = {};
   bool binned = false;
   bool host = false;
 };
 
-int make_bins(d2_ctx* c, const ObjView& v, int nmax, Bins* b) {
+int make_bins(d2_ctx* c, const ObjView& v, Bins* b) {
   int rc = D2_OK;
   const long long N = v.count;
+  const int nb = d2k::kSizeBins;
   int* bins = static_cast<int*>(grow(c, kBins, (size_t)N * 4, &rc));
-  void* scr = grow(c, kBinSort, d2k::update_scratch_bytes(N, 4), &rc);
+  void* scr = grow(c, kBinSort, d2k::update_scratch_bytes(N, nb), &rc);
   if (rc != D2_OK) return rc;
-  CK(d2k::bin_objects(v, nmax, bins, c->stream));
+  CK(d2k::bin_objects(v, bins, c->stream));
   d2k::FlowOut none{nullptr, nullptr, 0};
-  ObjView flat = v;  // the bin sort is one group of 4 labels, whatever the segments
+  ObjView flat = v;  // the bin sort is one group of labels, whatever the segments
   flat.segof = nullptr;
-  CK(d2k::update_locations(flat, nullptr, bins, N, 4, none, 4, nullptr, v.d, 0, nullptr, nullptr, scr,
-                           c->stream));
+  CK(d2k::update_locations(flat, nullptr, bins, N, nb, none, nb, nullptr, v.d, 0, nullptr, nullptr,
+                           scr, c->stream));
   const long long* start;
   const int* order;
-  d2k::sorted_groups(scr, N, 4, &start, &order);
+  d2k::sorted_groups(scr, N, nb, &start, &order);
   b->start = start;
   b->order = const_cast<int*>(order);
   b->binned = true;
@@ -457,10 +459,28 @@ int make_bins(d2_ctx* c, const ObjView& v, int nmax, Bins* b) {
 
 int bins_to_host(d2_ctx* c, Bins* b) {
   if (b->host) return D2_OK;
-  CK(cudaMemcpyAsync(b->hstart, b->start, 5 * sizeof(long long), cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaMemcpyAsync(b->hstart, b->start, sizeof(b->hstart), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   b->host = true;
   return D2_OK;
+}
+
+// The support counts at which a binned batch is cut into launches, increasing,
+// the last one mmax.  The lane screen's shared memory and row loops follow
+// the launch's row bound, so its launches step by a third to a half of it;
+// the warp-per-pair kernels change with the nodes per lane only.
+int size_cuts(bool lanes, int mmax, int nmax, int* cut) {
+  static const int steps[] = {4, 8, 12, 16, 24, 32, 48};
+  int k = 0;
+  if (lanes) {
+    for (int s : steps)
+      if (s < mmax) cut[k++] = s;
+  } else {
+    for (int b = 1; b < 4; ++b)
+      if (32 * b - nmax >= 1 && 32 * b - nmax < mmax) cut[k++] = 32 * b - nmax;
+  }
+  cut[k++] = mmax;
+  return k;
 }
 
 // One assign over a batch, bin by bin (largest trees first), each bin with
@@ -512,14 +532,18 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
     CK(d2k::assign(v, cv, seg, K, base, om, lab, d2o, terms, fo, cand, c->d_err, c->stream, ws, tw));
     return D2_OK;
   }
-  const bool tuning = c->cfg.group_lanes == 0 && mode == 1 && v.count >= 8192;
-  const int lo_bin = (1 + nmax + 31) / 32 - 1;
-  const int hi_bin = std::min(3, (mmax + nmax + 31) / 32 - 1);
-  for (int b = hi_bin; b >= lo_bin; --b) {
+  // the lane screen has one launch shape per bound; the warp-per-pair screen
+  // is tuned
+  const bool lanes = base.lanes && mode == 1 && !ws;
+  const bool tuning = c->cfg.group_lanes == 0 && mode == 1 && v.count >= 8192 && !lanes;
+  int cut[8];
+  const int ncut = size_cuts(lanes, mmax, nmax, cut);
+  for (int b = ncut - 1; b >= 0; --b) {
+    const int lo = b > 0 ? cut[b - 1] : 0;  // support counts lo + 1 .. cut[b]
     SolveCfg cfg = base;
-    cfg.mmax = std::max(1, std::min(mmax, 32 * (b + 1) - nmax));
-    const auto key = std::make_tuple(b, (long long)K, cfg.mmax, nmax, v.d,
-                                     mode + (cfg.certify ? 2 : 0));
+    cfg.mmax = cut[b];
+    const auto key = std::make_tuple((cfg.mmax + nmax + 31) / 32 - 1, (long long)K, cfg.mmax, nmax,
+                                     v.d, mode + (cfg.certify ? 2 : 0));
     auto it = c->tuned.find(key);
     // the host needs the bin's count for tensor-core chunks and to tune a
     // new launch shape (a wait); otherwise the launches read it on the device
@@ -528,13 +552,14 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
     if (host) {
       int rc0 = bins_to_host(c, &bins);
       if (rc0 != D2_OK) return rc0;
-      cnt = bins.hstart[b + 1] - bins.hstart[b];
+      cnt = bins.hstart[cut[b]] - bins.hstart[lo];
       if (cnt <= 0) continue;
-      cfg.oidx = bins.order + bins.hstart[b];
+      cfg.oidx = bins.order + bins.hstart[lo];
       cfg.nobj = cnt;
     } else {
       cfg.oidx = bins.order;
-      cfg.dev_range = bins.start + b;
+      cfg.dev_lo = bins.start + lo;
+      cfg.dev_hi = bins.start + cut[b];
     }
     if (it == c->tuned.end() && tuning && cnt < 8192) {
       // too few objects to time: the default shape, kept for this key
@@ -594,7 +619,7 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
       ++c->tuning_runs;
       it = c->tuned.emplace(key, pick).first;
     }
-    if (it != c->tuned.end()) {
+    if (it != c->tuned.end() && !lanes) {
       cfg.tpb = std::get<0>(it->second);
       cfg.ipsm = std::get<1>(it->second);
       cfg.start = std::get<2>(it->second);
@@ -693,13 +718,14 @@ int segment_impl(d2_ctx* c, const ObjView& v, int mmax, const double* om, long l
   double* dd = static_cast<double*>(grow(c, kSgD2, (size_t)N * 8, &rc));
   int* fcell = static_cast<int*>(grow(c, kSgCell, (size_t)(N * stride) * 4, &rc));
   double* fw = static_cast<double*>(grow(c, kSgFw, (size_t)(N * stride) * 8, &rc));
-  int* cand = static_cast<int*>(grow(c, kSgCand, (size_t)d2k::assign_scratch_ints(N, 2, c->sms) * 4, &rc));
+  int* cand = static_cast<int*>(grow(c, kSgCand, (size_t)d2k::assign_scratch_ints(N, 2, c->sms, mmax, mmax) * 4, &rc));
   if (rc != D2_OK) return rc;
   SolveCfg cfg = solve_cfg(c, mode_for(c, v.ldt), mmax);
   cfg.nmax = mmax;  // the split centroids are bags of the data
   // the splits' centroids are FP64 (their FP32 copies are not exact), and
   // only their labels are used: no per-pair certificate
   cfg.certify = false;
+  cfg.lane_exact = false;
   cfg.start = c->cfg.start_rule == D2_START_VOGEL ? 1
             : c->cfg.start_rule == D2_START_RANKED ? 0 : (mmax >= 64 ? 1 : 0);
   const FlowOut fo{fcell, fw, stride};
@@ -870,18 +896,18 @@ int segment_impl(d2_ctx* c, const ObjView& v, int mmax, const double* om, long l
   return D2_OK;
 }
 
-// Bin only when the batch is large and its trees span more than one bin.
-bool want_bins(const d2_ctx* c, long long count, int mmax) {
-  const int nmax = std::max(c->nmax, 1);
-  const int lo_bin = (1 + nmax + 31) / 32 - 1;
-  const int hi_bin = (mmax + nmax + 31) / 32 - 1;
-  return count >= 4096 && hi_bin > lo_bin;
+// Bin only when the batch is large and its launches then differ.
+bool want_bins(const d2_ctx* c, const SolveCfg& cfg, long long count, int mmax, bool warm) {
+  int cut[8];
+  return count >= 4096 &&
+         size_cuts(cfg.lanes && cfg.mode == 1 && !warm, mmax, std::max(c->nmax, 1), cut) > 1;
 }
 
 }  // namespace
 
 namespace d2k {
 bool ctx_prune(const d2_ctx* c) { return c->cfg.no_prune == 0; }
+bool ctx_lanes(const d2_ctx* c) { return c->cfg.start_rule == D2_START_AUTO; }
 CentView ctx_centroids(const d2_ctx* c, int* nmax, int* d, int* device, int* mode, int* budget,
                        int* sms, long long* K, int* start) {
   *nmax = c->nmax;
@@ -944,7 +970,8 @@ int d2_ctx_create(d2_ctx** out, int32_t device, const d2_config* cfg) {
       cudaStreamCreateWithFlags(&c->own, cudaStreamDefault) != cudaSuccess ||
       cudaMalloc(&c->d_err, 4 * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&c->d_info, 4 * sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&c->h_pin, 16 * sizeof(int)) != cudaSuccess) {
+      cudaMallocHost(&c->h_pin, 16 * sizeof(int)) != cudaSuccess ||
+      cudaMemset(c->d_err, 0, 4 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     d2_ctx_destroy(c);
     return D2_ECUDA;
@@ -1240,12 +1267,13 @@ int assign_impl(d2_ctx* c, const d2_bags* objs, const double* omega, int32_t* la
     terms = static_cast<double*>(grow(c, kEpsTerms, (size_t)N * 8, &rc));
     if (rc != D2_OK) return rc;
   }
-  int* cand = static_cast<int*>(grow(c, kCand, (size_t)d2k::assign_scratch_ints(N, c->K, c->sms) * 4, &rc));
+  int* cand = static_cast<int*>(grow(c, kCand, (size_t)d2k::assign_scratch_ints(N, c->K, c->sms, mmax, c->nmax) * 4, &rc));
   if (rc != D2_OK) return rc;
   if ((rc = check_bag_symbols(c, v))) return rc;
-  Bins bins;
-  if (want_bins(c, N, mmax) && (rc = make_bins(c, v, c->nmax, &bins))) return rc;
   const int mode = mode_for(c, objs->loc_dtype);
+  Bins bins;
+  if (want_bins(c, solve_cfg(c, mode, mmax), N, mmax, false) && (rc = make_bins(c, v, &bins)))
+    return rc;
   d2k::TcWork tw;
   const bool tc = tc_wanted(c, objs, v, mode);
   if (tc && (rc = tc_work(c, N * (long long)mmax, mmax, &tw))) return rc;
@@ -1610,7 +1638,7 @@ int d2_assign_multi(d2_ctx* const* ctxs, int32_t B, const d2_bags* objs, int32_t
     if ((rc = stage_bags(cb, &objs[b], kObjOff, kObjLoc, kObjW, &v[b]))) return rc;
     if ((rc = bag_bound(cb, &objs[b], v[b], &mmax[b]))) return rc;
     float* pair = static_cast<float*>(grow(cb, kMbPair, (size_t)N * K * 2 * 4, &rc));
-    int* cand = static_cast<int*>(grow(cb, kCand, (size_t)d2k::assign_scratch_ints(N, K, cb->sms) * 4, &rc));
+    int* cand = static_cast<int*>(grow(cb, kCand, (size_t)d2k::assign_scratch_ints(N, K, cb->sms, mmax[b], cb->nmax) * 4, &rc));
     int* tl = static_cast<int*>(grow(cb, kMbTmpLab, (size_t)N * 4, &rc));
     double* td = static_cast<double*>(grow(cb, kMbTmpD2, (size_t)N * 8, &rc));
     if (rc != D2_OK) return rc;
@@ -1775,7 +1803,7 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     void* scr = grow(c, kUpd, d2k::update_scratch_bytes(n_l, KT), &rc);
     const size_t lpart_n = d2k::update_part_bytes(n_l, KT, d);
     double* lpart = static_cast<double*>(grow(c, kLvPart, lpart_n, &rc));
-    int* cand = static_cast<int*>(grow(c, kCand, (size_t)d2k::assign_scratch_ints(n_l, K, c->sms) * 4, &rc));
+    int* cand = static_cast<int*>(grow(c, kCand, (size_t)d2k::assign_scratch_ints(n_l, K, c->sms, cur_mmax, c->nmax) * 4, &rc));
     if (rc != D2_OK) return rc;
     k_replicate<<<blocks_for(M * Tc), 256, 0, c->stream>>>(c->c_loc32, c->c_loc64, c->c_Q, c->c_w64,
                                                            c->c_off, K, Tc, d, M, l32, l64, lQ, lw,
@@ -1811,7 +1839,8 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
                           0};
     }
     Bins bins;
-    if (want_bins(c, n_l, cur_mmax) && (rc = make_bins(c, cur, c->nmax, &bins))) return rc;
+    if (want_bins(c, cfg, n_l, cur_mmax, ws.par8 != nullptr) && (rc = make_bins(c, cur, &bins)))
+      return rc;
     // the pruning moments of this level's bags, once for all its rounds
     const bool moments = prunes(c, cfg, cv);
     if (moments && (rc = prune_moments(c, cur))) return rc;

@@ -118,8 +118,16 @@ struct SolveCfg {
   long long nobj = -1;        // entries of oidx (-1: all ob.count objects)
   long long obase = 0;        // first object when oidx is nullptr
   // device-side object range (bins whose counts stay on the device): the
-  // launch takes oidx[dev_range[0] .. dev_range[1]); overrides nobj
-  const long long* dev_range = nullptr;
+  // launch takes oidx[*dev_lo .. *dev_hi); overrides nobj
+  const long long* dev_lo = nullptr;
+  const long long* dev_hi = nullptr;
+  // the screen runs several pairs per warp (lane_screen) unless the caller
+  // fixed a cold-start rule or saved bases are in play; `screened`: it has
+  // run and the merged lists are in place
+  bool lanes = false;
+  bool screened = false;
+  bool lane_exact = true;  // the exact pass too (needs centroids whose FP32 copy is exact)
+  long long max_pairs = 1LL << 24;  // pairs of one lane_screen chunk
   int start = 0;              // cold start basis: 0 ranked northwest staircase, 1 Vogel
   // per-pair screen output (optional): pair_out[2*(i*K + j)] = FP32 value,
   // [..+1] = its error bound (+inf when the screen could not bound it, NaN
@@ -201,6 +209,104 @@ D2_NPL_DECL(2)
 D2_NPL_DECL(3)
 D2_NPL_DECL(4)
 #undef D2_NPL_DECL
+
+// ---- the screen with several pairs per warp (d2_lane.cuh, d2_lane.cu) ----
+// Screened pair: ends of its interval and, where certified, its FP64 value.
+struct alignas(16) PairRec {
+  float lo, hi;
+  double d64;
+};
+
+// One launch over the pairs of a chunk of objects.
+struct LaneArgs {
+  const int* oidx;            // object list (null: obase ..)
+  const long long* lo;        // device range of the list (null: t0 ..)
+  const long long* hi;
+  long long t0;               // chunk's first object, from *lo (or 0)
+  long long cap;              // most objects of the chunk
+  long long obase;
+  const uint2* list;          // kept pairs (chunk object, centroid); null: every pair
+  unsigned long long* ctr;    // [0] work queue, [1] pairs in the list, [2] fallbacks, [3] zero
+  const long long* omass;     // [count][mstride] object masses
+  const unsigned char* obad;  // [count] bags the solver rejects
+  int mstride;
+  PairRec* rec;               // [pairs of the chunk]
+  unsigned char* tree;        // saved bases of the chunk's pairs (parents)
+  int tstride;                // bytes a basis
+  int nb;                     // column blocks of 4 (set by the launch)
+  int warp_bytes;             // shared memory of a warp (set by the launch)
+};
+
+// Outputs of the exact pass (labels null: a launch of the screen).
+struct ExactOut {
+  const int* cand = nullptr;                     // merged records
+  const unsigned long long* ostart = nullptr;    // list starts of the chunk's objects
+  const double* omega = nullptr;
+  int* labels = nullptr;
+  double* dist2 = nullptr;
+  double* eps_terms = nullptr;
+  FlowOut fo{nullptr, nullptr, 0};
+  int* fb = nullptr;                             // objects left to k_exact
+  int* err = nullptr;
+};
+
+// Scratch of lane_screen behind the merged lists: byte offsets of the object
+// masses, flags and list starts, the pair list and the pair records, for
+// chunks of `objects` objects (about max_pairs pairs).
+struct LaneScratch {
+  long long objects;
+  size_t mass, bad, start, list, rec, tree, fb, bytes;
+  int tstride;
+};
+inline LaneScratch lane_scratch(long long count, long long K, int mmax, int nmax,
+                                long long max_pairs) {
+  auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  LaneScratch s;
+  const long long n = count > 0 ? count : 1, k = K > 0 ? K : 1;
+  s.objects = std::max<long long>(1, std::min(n, max_pairs / k));
+  const size_t pairs = (size_t)s.objects * (size_t)k;
+  size_t b = 256;  // work queue and list length
+  s.mass = b;
+  b += up((size_t)n * (size_t)mmax * 8);
+  s.bad = b;
+  b += up((size_t)n);
+  s.start = b;
+  b += up((size_t)s.objects * 8);
+  s.list = b;
+  b += up(pairs * 8);
+  s.rec = b;
+  b += up(pairs * 16);
+  s.tstride = mmax + nmax;
+  s.tree = b;
+  b += up(pairs * (size_t)s.tstride);
+  s.fb = b;
+  b += up((size_t)n * 4);
+  s.bytes = b;
+  return s;
+}
+// The merged lists come first: 4 ints, kMergedInts per object.
+size_t lane_scratch_offset(long long count);
+// Every pair of the launch's objects (or the kept ones) solved in FP32,
+// merged candidate lists at cand + 4 (not with cfg.screen_only).
+// With X.labels the exact pass as well (chunk by chunk); the objects it leaves
+// to k_exact are X's fb list, *fb_hi of them (lane_fallback).
+cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_size, int K,
+                        const SolveCfg& cfg, int* cand, int* d_err, cudaStream_t st,
+                        const TcWork* tw, ExactOut X);
+// Launch settings of k_exact over the fallback list of lane_screen.
+void lane_fallback(const ObjView& ob, int K, int* cand, SolveCfg* cfg);
+#define D2_LANE_DECL(U)                                                                          \
+  cudaError_t lane_screen_##U(const ObjView& ob, const CentView& cv, long long seg_size, int K,  \
+                              const SolveCfg& cfg, const LaneArgs& A, long long total_obj,       \
+                              long long work, const ExactOut& X, cudaStream_t st);               \
+  cudaError_t stats_lane_##U(long long out[6]);
+D2_LANE_DECL(a)
+D2_LANE_DECL(b)
+D2_LANE_DECL(c)
+D2_LANE_DECL(d)
+D2_LANE_DECL(e)
+D2_LANE_DECL(f)
+#undef D2_LANE_DECL
 
 // ---- pairs that cannot be the argmin (Alg. 2 Step 2 needs only it) ----
 // Under a pair's own marginals (the quantised masses the solver uses), for
@@ -292,9 +398,11 @@ constexpr int kCandCap = 16;
 // count, centroids, lower ends, best upper end, certified FP64 value of that centroid
 constexpr int kItemInts = 2 + 2 * kCandCap + 2;
 constexpr int kMergedInts = 1 + kCandCap + 2;  // count, centroids, certified FP64 value
-inline long long assign_scratch_ints(long long count, long long K, int sms = 160) {
-  (void)K;
-  return 4 + ((count * kMergedInts + 3) & ~3LL) + (count + (long long)sms * 256) * kItemInts + 4;
+inline long long assign_scratch_ints(long long count, long long K, int sms, int mmax, int nmax,
+                                     long long max_pairs = 1LL << 24) {
+  const long long items = (count + (long long)sms * 256) * kItemInts + 4;
+  const long long lanes = (long long)(lane_scratch(count, K, mmax, nmax, max_pairs).bytes + 256) / 4 + 1;
+  return 4 + ((count * kMergedInts + 3) & ~3LL) + std::max(items, lanes);
 }
 cudaError_t cost_matrix(const ObjView& ob, const CentView& cv, long long i, long long j, int mode,
                         double* C, cudaStream_t st);
@@ -338,10 +446,10 @@ void sorted_groups(void* scratch, long long N, long long KT, const long long** s
 cudaError_t group_weight_sum(const double* omega, long long N, long long KT, void* scratch,
                              double* out, cudaStream_t st);
 
-// Bin of each object by the lanes' node count its tree needs with centroid
-// supports up to nmax: bin b holds m + nmax <= 32*(b+1); -1 if m is out of
-// range.  labels_out: [count] ints.
-cudaError_t bin_objects(const ObjView& ob, int nmax, int* bins_out, cudaStream_t st);
+// Bin of each object: its support count less one, -1 if out of 1..kSizeBins.
+// labels_out: [count] ints.
+constexpr int kSizeBins = 64;
+cudaError_t bin_objects(const ObjView& ob, int* bins_out, cudaStream_t st);
 
 int device_sms(int dev);
 

@@ -66,12 +66,11 @@ __global__ void k_prep_centroids(const void* loc, int ldt, const void* w, int wd
   }
 }
 
-__global__ void k_bin_of(const long long* off, long long count, int nmax, int* bins) {
+__global__ void k_bin_of(const long long* off, long long count, int* bins) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
        i += (long long)gridDim.x * blockDim.x) {
     const long long m = off[i + 1] - off[i];
-    const long long nn = m + nmax;
-    bins[i] = (m < 1 || nn > 128) ? -1 : (int)((nn + 31) / 32 - 1);
+    bins[i] = (m < 1 || m > kSizeBins) ? -1 : (int)(m - 1);
   }
 }
 
@@ -251,7 +250,9 @@ long long launches() { return (long long)__atomic_load_n(&g_launches, __ATOMIC_R
 
 // Sum of the solver counters of the units that hold the solver kernels.
 cudaError_t solver_stats(long long out[6]) {
-  cudaError_t (*const units[4])(long long*) = {stats_npl1, stats_npl2, stats_npl3, stats_npl4};
+  cudaError_t (*const units[])(long long*) = {
+      stats_npl1,   stats_npl2,   stats_npl3,   stats_npl4,   stats_lane_a,
+      stats_lane_b, stats_lane_c, stats_lane_d, stats_lane_e, stats_lane_f};
   for (int i = 0; i < 6; ++i) out[i] = 0;
   for (auto f : units) {
     long long v[6];
@@ -328,10 +329,25 @@ cudaError_t mallows_pairs(const ObjView& ob, const CentView& cv, const long long
 }
 
 cudaError_t assign(const ObjView& ob, const CentView& cv, long long seg_size, int K,
-                   const SolveCfg& cfg, const double* omega, int* labels, double* dist2,
+                   const SolveCfg& cfg0, const double* omega, int* labels, double* dist2,
                    double* eps_terms, FlowOut fo, int* cand, int* d_err, cudaStream_t st,
                    const WarmStore* ws, const TcWork* tw) {
   if (ob.count <= 0) return cudaSuccess;
+  SolveCfg cfg = cfg0;
+  if (cfg.lanes && cfg.mode == 1 && cand && !ws) {
+    ExactOut X;
+    if (cfg.lane_exact && !cfg.screen_only) {
+      X.omega = omega;
+      X.labels = labels;
+      X.dist2 = dist2;
+      X.eps_terms = eps_terms;
+      X.fo = fo;
+    }
+    const cudaError_t e = lane_screen(ob, cv, seg_size, K, cfg, cand, d_err, st, tw, X);
+    if (e != cudaSuccess || cfg.screen_only) return e;
+    cfg.screened = true;
+    if (X.labels) lane_fallback(ob, K, cand, &cfg);  // the few objects k_exact still solves
+  }
   int G, NP;
   if (!pick_shape(cfg.mmax, cfg.nmax, &G, &NP)) return cudaErrorInvalidValue;
 #define X(g_, n_)                                                                            \
@@ -342,10 +358,10 @@ cudaError_t assign(const ObjView& ob, const CentView& cv, long long seg_size, in
   return cudaErrorInvalidValue;
 }
 
-cudaError_t bin_objects(const ObjView& ob, int nmax, int* bins_out, cudaStream_t st) {
+cudaError_t bin_objects(const ObjView& ob, int* bins_out, cudaStream_t st) {
   if (ob.count <= 0) return cudaSuccess;
   const unsigned b = (unsigned)std::min<long long>((ob.count + 255) / 256, 4096);
-  k_bin_of<<<b, 256, 0, st>>>(ob.off, ob.count, nmax, bins_out);
+  k_bin_of<<<b, 256, 0, st>>>(ob.off, ob.count, bins_out);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -1,0 +1,1597 @@
+// d2_lane.cuh -- the FP32 screen with several pairs per warp.
+//
+// A transportation LP of the sizes the framework meets (a few to 64 supports
+// a side) gives one warp too little parallel work: with a warp per pair most
+// of a pivot's warp instructions (reductions, path searches, preorder
+// bookkeeping) serve one pair, and a cold 16 x 16 pair took about 11,000 of
+// them.  Here a pair is solved by G lanes, 32/G pairs share a warp in lock
+// step, and the basis tree is kept in a form whose pivot touches only the
+// cycle:
+//   par[y]  parent, flow[y] int64 flow of the edge (y, par[y]), pot[y],
+//   D[y]    the set of nodes in the subtree of y, as a bit mask (32*MW bits).
+// The entering cell's cycle is the two walks up from its ends to the first
+// node whose mask holds the other end; the leaving node's mask is the cut-off
+// side S, whose potentials shift; and only the cycle's masks change: a node
+// of the re-hung path gets S less its old path child's set, the nodes above
+// it lose S, those of the other side gain it.  One lane walks each side.
+// The walks' loops are a few dozen instructions; the first form of this
+// kernel, which tested every node's mask against both ends in unrolled
+// per-lane loops, ran 13,000 instructions of code and stalled on instruction
+// fetch 4.2 of 9.5 cycles per issue (7,500 cycles per pivot with 12 warps on
+// an SM).
+//
+// Shared memory of a warp is laid out in 16-byte units, unit u of its pair p
+// at (u * PW + p) * 16 with PW = 32/G pairs, and lane g of pair p is warp lane
+// g * PW + p: the lanes of a quarter warp that touch a unit each (128-bit
+// accesses) then cover 128 consecutive bytes, as do a half warp's 64-bit and
+// a warp's 32-bit ones, and two pairs on different units never meet in a
+// bank.  (With the pairs' lanes side by side instead, half of all shared
+// wavefronts were bank conflicts.)  Nodes: row a is node a, column r is node
+// MP + r; both bounds and with them every own-node address are compile-time
+// constants.  Unused rows and columns hold +inf costs and empty masks.
+//
+// The pivot rule is the one of Simplex (d2_solver.cuh): the most negative
+// reduced cost enters (ties to the smallest cell), the smallest flow leaves
+// (ties to the smallest cell), Bland's rule after 2N degenerate pivots,
+// potentials shifted incrementally and refreshed every 64 pivots.
+#pragma once
+#include "d2_solve.cuh"
+
+namespace d2k {
+namespace {
+
+// G lanes per pair, L of them across the blocks of 4 columns (the other
+// factor G / L splits the rows), MW 32-bit words per node mask, NPL node
+// slots per lane: 4 L columns and G NPL - 4 L rows.
+template <int G_, int L_, int MW_, int NPL_>
+struct LaneShape {
+  static constexpr int G = G_, L = L_, MW = MW_, NPL = NPL_;
+  static constexpr int PW = 32 / G;           // pairs per warp
+  static constexpr int RS = G / L;            // row groups
+  static constexpr int PS = PW * 16;          // bytes between a pair's units
+  static constexpr int NS = G * NPL;          // node slots
+  static constexpr int MP = NS - 4 * L;       // row slots; columns are nodes MP ..
+  static constexpr int KR = MP / G;           // own slots that are rows
+  // blocks of two warps per SM the registers leave room for
+  static constexpr int kMinBlocks = G == 32 ? 5 : (G == 16 ? 8 : 10);
+  static_assert(MP > 0 && MP % G == 0 && NS <= 32 * MW, "lane shape");
+  // A node's record: its flow and mask in a 16-byte unit, with the parent in
+  // the fourth word where the mask is one word (one 128-bit access per step
+  // of a walk); masks of 4 words have a unit of their own.
+  static constexpr int kPot = 0;
+  static constexpr int kNode = kPot + NPL * 128;
+  static constexpr int kD4 = kNode + NPL * 512;               // MW = 4
+  static constexpr int kPar = kD4 + (MW == 4 ? NPL * 512 : 0);  // MW > 1
+  static constexpr int kCode = kPar + (MW > 1 ? (NS + 15) / 16 * PS : 0);
+  static constexpr int kTile = kCode + (NS + 15) / 16 * PS;
+};
+
+// Bytes of a warp with room for mmax rows of nb column blocks.
+template <class Sh>
+inline size_t lane_warp_bytes(int mmax, int nb) {
+  return (size_t)Sh::kTile + (size_t)((mmax + 3) & ~3) * nb * Sh::PS;
+}
+
+template <int MW>
+struct Mask {
+  unsigned w[MW];
+  __device__ __forceinline__ bool meets(const Mask& o) const {
+    unsigned x = w[0] & o.w[0];
+#pragma unroll
+    for (int i = 1; i < MW; ++i) x |= w[i] & o.w[i];
+    return x != 0u;
+  }
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < MW; ++i) w[i] = 0u;
+  }
+  __device__ __forceinline__ void set(int e) {
+#pragma unroll
+    for (int i = 0; i < MW; ++i)
+      if ((e >> 5) == i) w[i] |= 1u << (e & 31);
+  }
+  __device__ __forceinline__ Mask minus(const Mask& o) const {
+    Mask r;
+#pragma unroll
+    for (int i = 0; i < MW; ++i) r.w[i] = w[i] & ~o.w[i];
+    return r;
+  }
+  __device__ __forceinline__ Mask plus(const Mask& o) const {
+    Mask r;
+#pragma unroll
+    for (int i = 0; i < MW; ++i) r.w[i] = w[i] | o.w[i];
+    return r;
+  }
+};
+
+// One pair's view of its warp's shared memory and its solver state; every
+// lane of the warp runs the same code (a pair without work has live = false
+// and only joins the shuffles).
+template <class Sh>
+struct Lane {
+  static constexpr int G = Sh::G, L = Sh::L, MW = Sh::MW, NPL = Sh::NPL, RS = Sh::RS;
+  static constexpr int PW = Sh::PW, PS = Sh::PS, MP = Sh::MP, NS = Sh::NS, KR = Sh::KR;
+  static constexpr unsigned kAll = 0xffffffffu;
+  char* sp;         // the pair's first unit
+  int nb;           // column blocks of the tile
+  int g, gl, rg;    // lane in the pair, its column lane, its row group
+  int m, n, N, root;
+  bool live;
+
+  __device__ __forceinline__ Lane(char* warp_base, int nb_) : nb(nb_) {
+    const int lane = threadIdx.x & 31;
+    g = lane / PW;
+    gl = g & (L - 1);
+    rg = g / L;
+    sp = warp_base + (lane & (PW - 1)) * 16;
+    m = n = 1;
+    N = 2;
+    root = 0;
+    live = false;
+  }
+
+  // ---- shared memory: any node, and the own node of slot k (y = g + G k) ----
+  __device__ __forceinline__ float4& tile4(int a, int cb) const {
+    return *reinterpret_cast<float4*>(sp + Sh::kTile + (a * nb + cb) * PS);
+  }
+  __device__ __forceinline__ float& cell(int a, int r) const {
+    return *reinterpret_cast<float*>(sp + Sh::kTile + (a * nb + (r >> 2)) * PS + (r & 3) * 4);
+  }
+  __device__ __forceinline__ float4& pot4(int q) const {
+    return *reinterpret_cast<float4*>(sp + Sh::kPot + q * PS);
+  }
+  __device__ __forceinline__ float& pot(int y) const {
+    return *reinterpret_cast<float*>(sp + Sh::kPot + (y >> 2) * PS + (y & 3) * 4);
+  }
+  __device__ __forceinline__ float& potk(int k) const {
+    return *reinterpret_cast<float*>(sp + Sh::kPot + (g >> 2) * PS + (g & 3) * 4 + k * 128);
+  }
+  __device__ __forceinline__ char* rec(int y) const { return sp + Sh::kNode + y * PS; }
+  __device__ __forceinline__ long long& flow(int y) const {
+    return *reinterpret_cast<long long*>(rec(y));
+  }
+  __device__ __forceinline__ long long& flowk(int k) const { return flow(g + G * k); }
+  // a second float per node, in the mask's place (once the masks are done with)
+  __device__ __forceinline__ float& aux(int y) const {
+    return *reinterpret_cast<float*>(rec(y) + 8);
+  }
+  template <int SEC>
+  __device__ __forceinline__ unsigned char& u8at(int y) const {
+    return *reinterpret_cast<unsigned char*>(sp + SEC + (y >> 4) * PS + (y & 15));
+  }
+  template <int SEC>
+  __device__ __forceinline__ unsigned char& u8own(int k) const {
+    // y >> 4 and y & 15 of y = g + G k, split into a lane part and a slot part
+    if constexpr (G >= 16)
+      return *reinterpret_cast<unsigned char*>(sp + SEC + (g >> 4) * PS + (g & 15) +
+                                               k * (G / 16) * PS);
+    else
+      return *reinterpret_cast<unsigned char*>(sp + SEC + g + ((G * k) >> 4) * PS + ((G * k) & 15));
+  }
+  __device__ __forceinline__ unsigned par(int y) const {
+    if constexpr (MW == 1) return *reinterpret_cast<unsigned*>(rec(y) + 12);
+    else return u8at<Sh::kPar>(y);
+  }
+  __device__ __forceinline__ void put_par(int y, unsigned v) const {
+    if constexpr (MW == 1) *reinterpret_cast<unsigned*>(rec(y) + 12) = v;
+    else u8at<Sh::kPar>(y) = (unsigned char)v;
+  }
+  __device__ __forceinline__ Mask<MW> getD(int y) const {
+    Mask<MW> d;
+    if constexpr (MW == 1) {
+      d.w[0] = *reinterpret_cast<const unsigned*>(rec(y) + 8);
+    } else if constexpr (MW == 2) {
+      const uint2 v = *reinterpret_cast<const uint2*>(rec(y) + 8);
+      d.w[0] = v.x; d.w[1] = v.y;
+    } else {
+      const uint4 v = *reinterpret_cast<const uint4*>(sp + Sh::kD4 + y * PS);
+      d.w[0] = v.x; d.w[1] = v.y; d.w[2] = v.z; d.w[3] = v.w;
+    }
+    return d;
+  }
+  // the whole record
+  __device__ __forceinline__ void load(int y, long long& f, Mask<MW>& d, unsigned& p) const {
+    const uint4 v = *reinterpret_cast<const uint4*>(rec(y));
+    f = (long long)(((unsigned long long)v.y << 32) | v.x);
+    if constexpr (MW == 1) {
+      d.w[0] = v.z;
+      p = v.w;
+    } else if constexpr (MW == 2) {
+      d.w[0] = v.z; d.w[1] = v.w;
+      p = u8at<Sh::kPar>(y);
+    } else {
+      d = getD(y);
+      p = u8at<Sh::kPar>(y);
+    }
+  }
+  __device__ __forceinline__ void store(int y, long long f, const Mask<MW>& d, unsigned p) const {
+    const unsigned lo = (unsigned)(unsigned long long)f, hi = (unsigned)((unsigned long long)f >> 32);
+    if constexpr (MW == 1) {
+      *reinterpret_cast<uint4*>(rec(y)) = make_uint4(lo, hi, d.w[0], p);
+    } else {
+      if constexpr (MW == 2) {
+        *reinterpret_cast<uint4*>(rec(y)) = make_uint4(lo, hi, d.w[0], d.w[1]);
+      } else {
+        *reinterpret_cast<uint2*>(rec(y)) = make_uint2(lo, hi);
+        *reinterpret_cast<uint4*>(sp + Sh::kD4 + y * PS) =
+            make_uint4(d.w[0], d.w[1], d.w[2], d.w[3]);
+      }
+      u8at<Sh::kPar>(y) = (unsigned char)p;
+    }
+  }
+  __device__ __forceinline__ int node(int k) const { return g + G * k; }
+  // own slot k holds a node of the pair (rows first: a compile-time split)
+  __device__ __forceinline__ bool nodek(int k) const {
+    return k < KR ? g + G * k < m : g + G * k - MP < n;
+  }
+  __device__ __forceinline__ static bool is_row(int y) { return y < MP; }
+  // tile cell of the edge (y, p)
+  __device__ __forceinline__ float edge_cost(int y, int p) const {
+    return is_row(y) ? cell(y, p - MP) : cell(p, y - MP);
+  }
+  // own slot k's node in a set whose words were shifted right by g
+  // (G k + g: word (G k) >> 5 since G divides 32)
+  __device__ __forceinline__ static bool ink(const Mask<MW>& shifted, int k) {
+    return (shifted.w[(G * k) >> 5] >> ((G * k) & 31)) & 1u;
+  }
+
+  // ---- reductions over the pair's lanes (warp lanes g * PW + p) ----
+  template <typename V>
+  __device__ __forceinline__ static V sum(V v) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kAll, v, o * PW);
+    return v;
+  }
+  __device__ __forceinline__ static float maxf(float v) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kAll, v, o * PW));
+    return v;
+  }
+  __device__ __forceinline__ static unsigned maxu(unsigned v) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(kAll, v, o * PW));
+    return v;
+  }
+  __device__ __forceinline__ static unsigned oru(unsigned v) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v |= __shfl_xor_sync(kAll, v, o * PW);
+    return v;
+  }
+  // smallest (value, key) over W neighbouring lanes of the pair
+  template <int W>
+  __device__ __forceinline__ static void min_key(float& v, int& key) {
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(kAll, v, o * PW);
+      const int ok = __shfl_xor_sync(kAll, key, o * PW);
+      if (ov < v || (ov == v && ok < key)) { v = ov; key = ok; }
+    }
+  }
+
+  // Sum over the pair's nodes of the double in each node's flow slot, in an
+  // order that does not depend on the shape: slot y mod 32 (compact node
+  // index, rows then columns) over its nodes in order, then halves of the
+  // slots.
+  __device__ __forceinline__ double sum_nodes() {
+    __syncwarp();
+    double v[32 / G];
+#pragma unroll
+    for (int s = 0; s < 32 / G; ++s) {
+      v[s] = 0.0;
+#pragma unroll
+      for (int k = 0; k < MW; ++k) {
+        const int c = g + G * s + 32 * k;
+        if (live && c < N) {
+          const double x = *reinterpret_cast<double*>(&flow(c < m ? c : c - m + MP));
+          v[s] = k == 0 ? x : v[s] + x;
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 16 / G; h > 0; h >>= 1)
+#pragma unroll
+      for (int s = 0; s < h; ++s) v[s] += v[s + h];
+    __syncwarp();
+    return sum(v[0]);
+  }
+
+  // ---- start: rows in turn on centred costs ----
+  // Every remaining row in cyclic order sends as much mass as both ends hold
+  // to its cheapest remaining column, the cost of a column taken against its
+  // mean over the object (vm: sum_a p_a c_ar, the lane's 4 columns): two bags
+  // far apart cost nearly f(a) + g(r), and what tells the columns apart is
+  // the rest.  The end that runs out (the row on a tie) leaves and hangs from
+  // the other; the last line of either kind is the root and takes the rest.
+  // Flows are the int64 masses, so the basis is exactly feasible.  Dantzig
+  // pivots from there, against the other rules on the workload laws (CPU
+  // model, mean per pair): image 8.7 (ranked staircase 22.1, Vogel 13.7, the
+  // same rule on the plain costs 21.1), uneven 5.8 (18.7, 10.4, 18.7), serving
+  // 36 (117, 55, 84), high_dim 52 (217, 55, 76), sequences 11.2 (37, 9.8,
+  // 13.8).  A step reads one row of the tile, where Vogel's rule keeps the two
+  // best of every line.  flow holds the masses, D the singletons.
+  __device__ __forceinline__ void start_rows(const float4& vm) {
+    unsigned long long ra = m >= 64 ? ~0ull : ((1ull << m) - 1ull);
+    unsigned long long ca = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
+    int nr = m, nc = n, cur = -1;
+    for (;;) {
+      const bool act = live && nr > 1 && nc > 1;
+      if (!__any_sync(kAll, act)) break;
+      float best = INFINITY;
+      int key = INT_MAX;
+      int a = 0;
+      if (act) {
+        const unsigned long long later = ra & ~((2ull << (cur & 63)) - 1ull);
+        a = __ffsll((long long)((cur >= 0 && later) ? later : ra)) - 1;
+        if (gl < nb) {
+          const float4 c = tile4(a, gl);
+          const unsigned al = (unsigned)(ca >> (4 * gl)) & 15u;
+          const float d[4] = {c.x - vm.x, c.y - vm.y, c.z - vm.z, c.w - vm.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (((al >> i) & 1u) && d[i] < best) { best = d[i]; key = 4 * gl + i; }
+        }
+      }
+      min_key<L>(best, key);
+      long long ma = 0, mr = 0;
+      int r = 0;
+      if (act) {
+        r = key == INT_MAX ? __ffsll((long long)ca) - 1 : key;
+        ma = flow(a);
+        mr = flow(MP + r);
+      }
+      __syncwarp();
+      if (act) {
+        const bool row_leaves = ma <= mr;
+        if (g == 0) {
+          const int y = row_leaves ? a : MP + r, z = row_leaves ? MP + r : a;
+          put_par(y, (unsigned)z);
+          store(z, row_leaves ? mr - ma : ma - mr, getD(z).plus(getD(y)), 0xffu);
+        }
+        if (row_leaves) { ra &= ~(1ull << a); --nr; }
+        else { ca &= ~(1ull << r); --nc; }
+        cur = a;
+      }
+      __syncwarp();
+    }
+    // the last line takes the rest
+    const bool row_root = nr == 1;
+    root = row_root ? __ffsll((long long)ra) - 1 : MP + __ffsll((long long)ca) - 1;
+    Mask<MW> d;
+    d.clear();
+#pragma unroll 1
+    for (int k = 0; k < NPL; ++k) {
+      const int y = node(k);
+      if (live && nodek(k)) {
+        const bool row = k < KR;
+        const bool left = row ? (ra >> y) & 1ull : (ca >> (y - MP)) & 1ull;
+        if (left && row != row_root) {
+          put_par(y, (unsigned)root);
+          d = d.plus(getD(y));
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < MW; ++i) d.w[i] = oru(d.w[i]);
+    if (live && g == 0) store(root, 0, getD(root).plus(d), 0xffu);
+    __syncwarp();
+  }
+
+  // Accumulate the own nodes' edge terms acc over the path to the root by
+  // pointer jumping with alternating signs, acc(y) = acc(y) -+ acc(ancestor);
+  // at(y) is where node y's value lives meanwhile (and at the end).  Returns
+  // whether the tree is inconsistent.
+  template <typename T, typename At>
+  __device__ __forceinline__ bool jump(T (&acc)[NPL], At at) {
+    bool bad = false;
+    unsigned cd[NPL];  // ancestor | 128 * parity
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      cd[k] = (unsigned)root;
+      if (live && nodek(k) && node(k) != root) {
+        const unsigned p = par(node(k));
+        if (p >= (unsigned)NS || (k < KR) == is_row((int)p)) bad = true;
+        else cd[k] = p | 128u;
+      }
+    }
+    for (int round = 0; round < 9; ++round) {  // depth < 128: at most 8
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < NPL; ++k) {
+        if (live) {
+          u8own<Sh::kCode>(k) = (unsigned char)cd[k];
+          at(node(k)) = acc[k];
+        }
+      }
+      __syncwarp();
+      bool moved = false;
+#pragma unroll
+      for (int k = 0; k < NPL; ++k) {
+        const int an = (int)(cd[k] & 127u);
+        const unsigned c2 = u8at<Sh::kCode>(an);
+        const T v = at(an);
+        const bool mv = live && an != root;
+        const T nx = (cd[k] & 128u) ? acc[k] - v : acc[k] + v;
+        acc[k] = mv ? nx : acc[k];
+        cd[k] = mv ? ((c2 & 127u) | ((cd[k] ^ c2) & 128u)) : cd[k];
+        moved |= mv;
+      }
+      if (!__any_sync(kAll, moved)) break;
+    }
+    __syncwarp();
+    return bad;
+  }
+
+  // Potentials from the tree: pot(root) = 0, pot(y) = c(y, par y) - pot(par y).
+  __device__ __forceinline__ bool refresh() {
+    float acc[NPL];
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      acc[k] = 0.f;
+      if (live && nodek(k) && node(k) != root) {
+        const int p = (int)par(node(k));
+        if (p < NS && (k < KR) != is_row(p))
+          acc[k] = k < KR ? cell(node(k), p - MP) : cell(p, node(k) - MP);
+      }
+    }
+    return jump(acc, [&](int y) -> float& { return pot(y); });
+  }
+
+  // Most negative reduced cost of the tile (ties to the smallest cell
+  // key (a << 8) | r); key INT_MAX if none is negative.
+  __device__ __forceinline__ void price(bool act, float& best, int& key) {
+    best = 0.f;
+    key = INT_MAX;
+    if (act && gl < nb) {
+      int brow = -1;
+      const float4 v = pot4((MP >> 2) + gl);
+      const float2 nv0 = make_float2(-v.x, -v.y), nv1 = make_float2(-v.z, -v.w);
+      const char* tp = sp + Sh::kTile + (4 * rg * nb + gl) * PS;
+      const int step = nb * PS;
+      for (int a = 4 * rg; a < m; a += 4 * RS) {
+        const float4 u = pot4(a >> 2);
+        const float uu[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 c = *reinterpret_cast<const float4*>(tp + i * step);
+          const float2 nu = make_float2(-uu[i], -uu[i]);
+          const float2 d0 = __fadd2_rn(__fadd2_rn(make_float2(c.x, c.y), nu), nv0);
+          const float2 d1 = __fadd2_rn(__fadd2_rn(make_float2(c.z, c.w), nu), nv1);
+          const float lo = fminf(fminf(d0.x, d0.y), fminf(d1.x, d1.y));
+          if (lo < best) { best = lo; brow = a + i; }
+        }
+        tp += 4 * RS * step;
+      }
+      if (brow >= 0) {
+        const float4 c = tile4(brow, gl);
+        const float u = pot(brow);
+        int r = 3;
+        if (c.z - u - v.z == best) r = 2;
+        if (c.y - u - v.y == best) r = 1;
+        if (c.x - u - v.x == best) r = 0;
+        key = (brow << 8) | (4 * gl + r);
+      }
+    }
+    min_key<G>(best, key);
+  }
+
+  // Bland's rule: the smallest cell with reduced cost below -tol.
+  __device__ void price_bland(bool act, float tol, float& best, int& key) {
+    best = 0.f;
+    key = INT_MAX;
+    if (act && gl < nb) {
+      for (int a = 0; a < m && key == INT_MAX; ++a) {
+        if ((a >> 2) % RS != rg) continue;
+        for (int i = 0; i < 4 && key == INT_MAX; ++i) {
+          const int r = 4 * gl + i;
+          const float d = cell(a, r) - pot(a) - pot(MP + r);
+          if (d < -tol) { best = d; key = (a << 8) | r; }
+        }
+      }
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(kAll, best, o * PW);
+      const int ok = __shfl_xor_sync(kAll, key, o * PW);
+      if (ok < key) { best = ov; key = ok; }
+    }
+  }
+
+  // Group minimum of a 64-bit value that is never negative.
+  __device__ __forceinline__ static long long min64(long long v) {
+    if constexpr (G == 32) {
+      const unsigned hi = (unsigned)((unsigned long long)v >> 32), lo = (unsigned)v;
+      const unsigned mh = __reduce_min_sync(kAll, hi);
+      const unsigned ml = __reduce_min_sync(kAll, hi == mh ? lo : 0xffffffffu);
+      return (long long)(((unsigned long long)mh << 32) | ml);
+    } else {
+#pragma unroll
+      for (int o = G / 2; o > 0; o >>= 1) {
+        const long long w = __shfl_xor_sync(kAll, v, o * PW);
+        v = w < v ? w : v;
+      }
+      return v;
+    }
+  }
+
+  // The pivot of the wide shapes (16 or 32 lanes a pair): no walk, every lane
+  // tests its own nodes' masks against both ends (a node is on the cycle iff
+  // its subtree holds exactly one), and a node of the cut path hands its old
+  // parent the edge between them.  At 64 x 64 a side's walk is about 11 steps
+  // of dependent loads: 6.0 k cycles a pivot against 3.6 k for this form.
+  __device__ __forceinline__ int pivot_scan(bool act, int key, float dE) {
+    const int ea = act ? key >> 8 : 0;
+    const int eB = act ? MP + (key & 0xff) : MP;
+    Mask<MW> mA, mB;
+    mA.clear();
+    mB.clear();
+    if (act) {
+      mA.set(ea);
+      mB.set(eB);
+    }
+    unsigned aS = 0u, bS = 0u;  // own nodes on the row / column side
+    long long th = LLONG_MAX;
+    unsigned tk = 0u;  // own slots holding the smallest flow
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const Mask<MW> D = getD(node(k));
+      const long long f = flowk(k);
+      const bool a = D.meets(mA), b = D.meets(mB);
+      aS |= (a && !b) ? 1u << k : 0u;
+      bS |= (b && !a) ? 1u << k : 0u;
+      if (k < KR ? (a && !b) : (b && !a)) {
+        tk = f < th ? 1u << k : (f == th ? tk | (1u << k) : tk);
+        th = f < th ? f : th;
+      }
+    }
+    const long long own = th;
+    if (th < 0) th = LLONG_MAX;  // inconsistent: no leaving edge
+    th = min64(th);
+    int tkey = INT_MAX;
+    if (own == th && th != LLONG_MAX) {
+      for (unsigned t = tk; t; t &= t - 1) {
+        const int y = node(__ffs((int)t) - 1), p = (int)par(y);
+        const int kk = ((is_row(y) ? (y << 8) | (p - MP) : (p << 8) | (y - MP)) << 7) | y;
+        tkey = min(tkey, kk);
+      }
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) tkey = min(tkey, __shfl_xor_sync(kAll, tkey, o * PW));
+    const bool good = act && tkey != INT_MAX;
+    const int zL = good ? tkey & 0x7f : 0;
+    Mask<MW> S;
+    S.clear();
+    if (good) S = getD(zL);
+    const bool aside = S.meets(mA);  // the leaving side holds the row end
+    const int enode = aside ? ea : eB, onode = aside ? eB : ea;
+    Mask<MW> Sg;  // S seen from the own slots
+#pragma unroll
+    for (int i = 0; i < MW; ++i) Sg.w[i] = S.w[i] >> g;
+    const unsigned on = good ? (aS | bS) : 0u;
+    const unsigned minus = (aS & ((1u << KR) - 1u)) | (bS & ~((1u << KR) - 1u));
+    const unsigned lbits = aside ? aS : bS;
+    // read everything, then write
+    Mask<MW> Dn[NPL];
+    long long nf[NPL];
+    unsigned op[NPL];
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      op[k] = 0u;
+      if ((on >> k) & 1u) {
+        const bool inS = ink(Sg, k);
+        Mask<MW> D;
+        load(node(k), nf[k], D, op[k]);
+        nf[k] += ((minus >> k) & 1u) ? -th : th;
+        Dn[k] = inS ? S.minus(D) : (((lbits >> k) & 1u) ? D.minus(S) : D.plus(S));
+      }
+    }
+    __syncwarp();
+    const float se = is_row(enode) ? dE : -dE;  // shift of a row's potential
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const bool inS = ink(Sg, k);
+      if ((on >> k) & 1u) {
+        const int y = node(k);
+        if (!inS) store(y, nf[k], Dn[k], op[k]);
+        else if (y != zL) store((int)op[k], nf[k], Dn[k], (unsigned)y);
+        if (inS && y == enode) store(y, th, S, (unsigned)onode);
+      }
+      if (inS) potk(k) += k < KR ? se : -se;
+    }
+    __syncwarp();
+    return good ? (th > 0 ? 1 : 0) : -1;
+  }
+
+  // One pivot on entering cell `key` with reduced cost dE < 0.  Returns 1 if
+  // flow moved, 0 if none did, -1 if the tree is inconsistent.  Lane 0 of the pair walks
+  // the row side of the cycle, lane 1 the column side.
+  __device__ __forceinline__ int pivot(bool act, int key, float dE) {
+    const int ea = key >> 8, eB = MP + (key & 0xff);
+    const bool walker = act && g < 2;
+    const bool colside = (g & 1) != 0;
+    const int x0 = colside ? eB : ea, x1 = colside ? ea : eB;
+    Mask<MW> far;  // the other end
+    far.clear();
+    if (act) far.set(x1);
+    // 1. up to the first node above both ends; the edges that lose flow hang
+    // from rows on the row side and from columns on the column side
+    long long th = LLONG_MAX;
+    int tkey = INT_MAX;  // (row, column, node) of the smallest flow
+    bool lost = false;
+    if (walker) {
+      int x = x0;
+      lost = true;
+      for (int it = 0; it < NS; ++it) {
+        long long f;
+        Mask<MW> D;
+        unsigned p;
+        load(x, f, D, p);
+        if (D.meets(far)) { lost = false; break; }
+        if (p >= (unsigned)NS) break;
+        const bool row = is_row(x);
+        if (row != colside && f <= th) {
+          const int kk = ((row ? (x << 8) | ((int)p - MP) : ((int)p << 8) | (x - MP)) << 7) | x;
+          if (f < th || kk < tkey) { th = f; tkey = kk; }
+        }
+        x = (int)p;
+      }
+    }
+    // the smaller of the two sides (ties to the smaller cell)
+    const long long oth = __shfl_xor_sync(kAll, th, PW);
+    const int okey = __shfl_xor_sync(kAll, tkey, PW);
+    const bool mine = th < oth || (th == oth && tkey < okey);  // this side leaves
+    th = mine ? th : oth;
+    tkey = mine ? tkey : okey;
+    const int src = threadIdx.x & (PW - 1);  // lane 0 of the pair
+    const int olost = __shfl_xor_sync(kAll, (int)lost, PW);
+    int z = (tkey == INT_MAX || th < 0 || lost || olost) ? -1 : tkey & 0x7f;
+    // to the pair's other lanes: node, whether flow moves, which side leaves
+    z = __shfl_sync(kAll, z * 4 + (th > 0 ? 2 : 0) + (mine ? 0 : 1), src);
+    const int zL = z >> 2;
+    const bool good = act && zL >= 0;
+    const int enode = (z & 1) ? eB : ea;
+    Mask<MW> S;
+    S.clear();
+    if (good) S = getD(zL);
+    __syncwarp();
+    // 2. potentials of the cut-off side
+    const float se = is_row(enode) ? dE : -dE;
+    Mask<MW> Sg;  // S seen from the own slots
+#pragma unroll
+    for (int i = 0; i < MW; ++i) Sg.w[i] = S.w[i] >> g;
+#pragma unroll
+    for (int k = 0; k < NPL; ++k)
+      if (ink(Sg, k)) potk(k) += k < KR ? se : -se;
+    // 3. the walks again: flows, masses of the subtrees, the re-hung path
+    if (walker && good) {
+      int x = x0;
+      bool path = mine;  // still below the leaving edge: the edge turns round
+      unsigned prev = (unsigned)x1;
+      long long carry = th;
+      Mask<MW> dprev;
+      dprev.clear();
+      for (int it = 0; it < NS; ++it) {
+        long long f;
+        Mask<MW> D;
+        unsigned p;
+        load(x, f, D, p);
+        if (D.meets(far)) break;
+        const long long nf = is_row(x) != colside ? f - th : f + th;
+        const Mask<MW> nd = path ? S.minus(dprev) : (mine ? D.minus(S) : D.plus(S));
+        store(x, path ? carry : nf, nd, path ? prev : p);
+        carry = nf;
+        dprev = D;
+        prev = (unsigned)x;
+        path = path && x != zL;
+        x = (int)p;
+      }
+    }
+    __syncwarp();
+    return good ? (z >> 1) & 1 : -1;
+  }
+
+  // Pivot until no reduced cost is below -tol.  Optimality is accepted on the
+  // incrementally shifted potentials (the screen's error bound covers their
+  // drift).  Returns kStOk, kStNotConverged or kStInvalid.
+  __device__ __forceinline__ int run(int max_pivots, float tol, int* pivots) {
+    int st = kStOk;
+    int done = 0, degen = 0, since = 64;
+    bool bland = false, open = live;
+    for (;;) {
+      const bool due = open && since >= 64;
+      if (__any_sync(kAll, due)) {  // the first round, then every 64 pivots
+        const bool was = live;
+        live = due;
+        const bool b = refresh();
+        live = was;
+        if (due) since = 0;
+        if (maxu(due && b ? 1u : 0u)) { st = kStInvalid; open = false; }
+      }
+      float dE;
+      int key;
+      price(open && !bland, dE, key);
+      if (__any_sync(kAll, open && bland)) {
+        float d2;
+        int k2;
+        price_bland(open && bland, tol, d2, k2);
+        if (bland) { dE = d2; key = k2; }
+      }
+      if (open && !(dE < -tol && key != INT_MAX)) open = false;
+      if (open && done >= max_pivots) { st = kStNotConverged; open = false; }
+      if (!__any_sync(kAll, open)) break;
+      int moved;
+      if constexpr (G >= 16) moved = pivot_scan(open, key, dE);
+      else moved = pivot(open, key, dE);
+      if (open) {
+        if (moved < 0) {
+          st = kStInvalid;
+          open = false;
+        } else {
+          ++done;
+          ++since;
+          if (moved) { degen = 0; bland = false; }
+          else if (++degen >= 2 * N) bland = true;
+        }
+      }
+    }
+    *pivots += done;
+    return st;
+  }
+};
+
+// ---- ground-cost tiles -------------------------------------------------
+
+// Tile of FP32 bags with a small compile-time dimension: the lane keeps its 4
+// centroid supports in registers (each read once per pair) and takes the
+// object's rows one by one.  Same operations in the same order as cost_cells.
+template <class Sh, int D>
+__device__ __forceinline__ float lane_cost_small(const Lane<Sh>& P, const float* __restrict__ x,
+                                                 const float* __restrict__ y) {
+  float cmax = 0.f;
+  if (!P.live || P.gl >= P.nb) return cmax;
+  float yv[4][D];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int r = min(4 * P.gl + j, P.n - 1);
+#pragma unroll
+    for (int k = 0; k < D; ++k) yv[j][k] = __ldg(y + r * D + k);
+  }
+  const int mq = (P.m + 3) >> 2;
+  for (int q = P.rg; q < mq; q += Sh::RS) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int a = 4 * q + i;
+      float c[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+      if (a < P.m) {
+        float xv[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) xv[k] = __ldg(x + a * D + k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float acc = 0.f;
+#pragma unroll
+          for (int k = 0; k < D; ++k) {
+            const float df = xv[k] - yv[j][k];
+            acc = fmaf(df, df, acc);
+          }
+          if (4 * P.gl + j < P.n) {
+            c[j] = acc;
+            cmax = acc > cmax ? acc : cmax;
+          }
+        }
+      }
+      P.tile4(a, P.gl) = make_float4(c[0], c[1], c[2], c[3]);
+    }
+  }
+  return cmax;
+}
+
+// Any dimension: 4 x 4 cells at a time, the coordinates in steps of V
+// (V = 4: vector loads, d a multiple of 4 and 16-byte aligned rows).
+template <class Sh, typename X, int V>
+__device__ __forceinline__ float lane_cost_any(const Lane<Sh>& P, const X* __restrict__ x,
+                                               const float* __restrict__ y, int d) {
+  float cmax = 0.f;
+  if (!P.live || P.gl >= P.nb) return cmax;
+  const int mq = (P.m + 3) >> 2;
+  const float* yp[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) yp[j] = y + (long long)min(4 * P.gl + j, P.n - 1) * d;
+  for (int q = P.rg; q < mq; q += Sh::RS) {
+    const X* xp[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) xp[i] = x + (long long)min(4 * q + i, P.m - 1) * d;
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int k = 0; k < d; k += V) {
+      float xv[4][V], yv[4][V];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if constexpr (V == 4) {
+          const float4 t = __ldg(reinterpret_cast<const float4*>(xp[i] + k));
+          xv[i][0] = t.x; xv[i][1] = t.y; xv[i][2] = t.z; xv[i][3] = t.w;
+          const float4 s = __ldg(reinterpret_cast<const float4*>(yp[i] + k));
+          yv[i][0] = s.x; yv[i][1] = s.y; yv[i][2] = s.z; yv[i][3] = s.w;
+        } else {
+          xv[i][0] = cvt<float>(xp[i][k]);
+          yv[i][0] = __ldg(yp[i] + k);
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < V; ++t)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float df = xv[i][t] - yv[j][t];
+            acc[i][j] = fmaf(df, df, acc[i][j]);
+          }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float c[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool in = 4 * q + i < P.m && 4 * P.gl + j < P.n;
+        c[j] = in ? acc[i][j] : INFINITY;
+        if (in && acc[i][j] > cmax) cmax = acc[i][j];
+      }
+      P.tile4(4 * q + i, P.gl) = make_float4(c[0], c[1], c[2], c[3]);
+    }
+  }
+  return cmax;
+}
+
+// One value per cell from `f(a, r)`: symbol tables and ready-made tiles.
+template <class Sh, typename F>
+__device__ __forceinline__ float lane_cost_from(const Lane<Sh>& P, F f) {
+  float cmax = 0.f;
+  if (!P.live || P.gl >= P.nb) return cmax;
+  const int mq = (P.m + 3) >> 2;
+  for (int q = P.rg; q < mq; q += Sh::RS) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int a = 4 * q + i;
+      float c[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = 4 * P.gl + j;
+        if (a < P.m && r < P.n) {
+          c[j] = f(a, r);
+          cmax = c[j] > cmax ? c[j] : cmax;
+        }
+      }
+      P.tile4(a, P.gl) = make_float4(c[0], c[1], c[2], c[3]);
+    }
+  }
+  return cmax;
+}
+
+// Mean of each column over the object, sum_a p_a c_ar (the lane's 4 columns).
+template <class Sh>
+__device__ __forceinline__ float4 lane_col_means(const Lane<Sh>& P) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (P.live && P.gl < P.nb) {
+    for (int a = 4 * P.rg; a < P.m; a += 4 * Sh::RS) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (a + i < P.m) {
+          const float p = (float)P.flow(a + i) * (float)kInvMass;
+          const float4 c = P.tile4(a + i, P.gl);
+          v.x = fmaf(p, c.x, v.x);
+          v.y = fmaf(p, c.y, v.y);
+          v.z = fmaf(p, c.z, v.z);
+          v.w = fmaf(p, c.w, v.w);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int o = Sh::G / 2; o >= Sh::L; o >>= 1) {  // the row groups
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o * Sh::PW);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o * Sh::PW);
+    v.z += __shfl_xor_sync(0xffffffffu, v.z, o * Sh::PW);
+    v.w += __shfl_xor_sync(0xffffffffu, v.w, o * Sh::PW);
+  }
+  return v;
+}
+
+// The pair's FP32 tile, its largest cost and its column means.
+template <class Sh>
+__device__ __forceinline__ float lane_tile(const Lane<Sh>& P, const ObjView& ob, long long o0,
+                                           const CentView& cv, long long c0, const float* tile_g,
+                                           long long ldc, float4& vm) {
+  float cmax;
+  if (tile_g) {  // made ahead by the tensor cores: rows of 16 B where aligned
+    if (((reinterpret_cast<uintptr_t>(tile_g) | (uintptr_t)(ldc * 4)) & 15) == 0 &&
+        (P.n & 3) == 0) {
+      cmax = 0.f;
+      if (P.live && P.gl < P.nb && 4 * P.gl < P.n) {
+        const int mq = (P.m + 3) >> 2;
+        for (int q = P.rg; q < mq; q += Sh::RS) {
+          float4 c[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            c[i] = 4 * q + i < P.m
+                       ? __ldg(reinterpret_cast<const float4*>(tile_g + (4 * q + i) * ldc + 4 * P.gl))
+                       : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            P.tile4(4 * q + i, P.gl) = c[i];
+            if (4 * q + i < P.m)
+              cmax = fmaxf(cmax, fmaxf(fmaxf(c[i].x, c[i].y), fmaxf(c[i].z, c[i].w)));
+          }
+        }
+      } else if (P.live && P.gl < P.nb) {
+        const int mq = (P.m + 3) >> 2;
+        for (int q = P.rg; q < mq; q += Sh::RS)
+          for (int i = 0; i < 4; ++i)
+            P.tile4(4 * q + i, P.gl) = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+      }
+    } else {
+      cmax = lane_cost_from(P, [&](int a, int r) { return __ldg(tile_g + a * ldc + r); });
+    }
+  } else if (cv.A) {
+    const float* ys = cv.loc32 + c0;
+    cmax = lane_cost_from(P, [&](int a, int r) {
+      int xs = (int)ldx<float>(ob.loc, ob.ldt, o0 + a);
+      int yy = (int)ys[r];
+      xs = xs < 0 ? 0 : (xs >= cv.A ? cv.A - 1 : xs);
+      yy = yy < 0 ? 0 : (yy >= cv.A ? cv.A - 1 : yy);
+      return __ldg(cv.tab32 + xs * cv.A + yy);
+    });
+  } else {
+    const int d = cv.d;
+    const float* y = cv.loc32 + c0 * d;
+    const long long o = o0 * d;
+    if (ob.ldt == 1) {
+      const float* x = static_cast<const float*>(ob.loc) + o;
+      if (d == 6) cmax = lane_cost_small<Sh, 6>(P, x, y);
+      else if (d == 3) cmax = lane_cost_small<Sh, 3>(P, x, y);
+      else if ((d & 3) == 0 && ((reinterpret_cast<uintptr_t>(ob.loc) |
+                                 reinterpret_cast<uintptr_t>(cv.loc32)) & 15) == 0)
+        cmax = lane_cost_any<Sh, float, 4>(P, x, y, d);
+      else cmax = lane_cost_any<Sh, float, 1>(P, x, y, d);
+    } else if (ob.ldt == 2) {
+      cmax = lane_cost_any<Sh, __nv_bfloat16, 1>(
+          P, static_cast<const __nv_bfloat16*>(ob.loc) + o, y, d);
+    } else {
+      cmax = lane_cost_any<Sh, double, 1>(P, static_cast<const double*>(ob.loc) + o, y, d);
+    }
+  }
+  cmax = Lane<Sh>::maxf(cmax);
+  vm = lane_col_means(P);  // the lane's own cells
+  __syncwarp();
+  return cmax;
+}
+
+// ---- certificate ---------------------------------------------------------
+
+// certify_fp64 (d2_solve.cuh) on a lane pair: the same arithmetic, bounds and
+// tests; only the order of the objective's FP64 sum differs.  Overwrites the
+// tile's basic cells, the flows and the masks (kept: par).
+template <class Sh>
+__device__ __forceinline__ bool lane_certify(Lane<Sh>& P, bool go, const ObjView& ob, long long o0,
+                             const CentView& cv, long long c0, float cmax, float ecost,
+                             double* D64, float* tau_out, int* nchk) {
+  constexpr int NPL = Sh::NPL;
+  constexpr unsigned kAll = 0xffffffffu;
+  const bool keep_live = P.live;
+  P.live = go;
+  constexpr int MP = Sh::MP, NS = Sh::NS;
+  const int xt = (cv.A == 0 && ob.ldt != 0) ? ob.ldt : 0;
+  // basic cells in double-float: objective terms into the flow slots (the
+  // flows are done with), residuals of the FP32 potentials into aux
+  bool bad = false;
+#pragma unroll 1
+  for (int k = 0; k < NPL; ++k) {
+    const int y = P.node(k);
+    if (!go || !(k < Sh::KR ? y < P.m : y - MP < P.n)) continue;
+    double term = 0.0;
+    float res = 0.f;
+    if (y != P.root) {
+      const int p = (int)P.par(y);
+      const bool row = y < MP;
+      if (p >= NS || row == (p < MP)) {
+        bad = true;
+      } else {
+        const int a = row ? y : p;
+        const int r = (row ? p : y) - MP;
+        float ch, cl;
+        cost_dd(xt, ob, o0, cv, c0, a, r, ch, cl);
+        const double w = (double)P.flow(y) * kInvMass;
+        term = fma(w, (double)cl, w * (double)ch);
+        float s1, e1;
+        two_sum(ch, -P.pot(y), s1, e1);
+        e1 = __fadd_rn(e1, cl);
+        float s2, e2;
+        two_sum(s1, -P.pot(p), s2, e2);
+        res = __fadd_rn(s2, __fadd_rn(e2, e1));
+      }
+    }
+    *reinterpret_cast<double*>(&P.flow(y)) = term;
+    P.aux(y) = res;
+  }
+  const double D = P.sum_nodes();
+  *D64 = D;
+  float delta[NPL];
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) delta[k] = go && P.nodek(k) ? P.aux(P.node(k)) : 0.f;
+  bad |= P.jump(delta, [&](int y) -> float& { return P.aux(y); });  // corrections
+  unsigned pm = 0u, dm = 0u;
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) {
+    const int y = P.node(k);
+    if (go && P.nodek(k)) {
+      const float b = P.potk(k);
+      *reinterpret_cast<float2*>(&P.flowk(k)) = make_float2(b, delta[k]);
+      const float u = b + delta[k];
+      P.potk(k) = u;
+      pm = max(pm, __float_as_uint(fabsf(u)));
+      dm = max(dm, __float_as_uint(fabsf(delta[k])));
+      if (y != P.root && !bad) {
+        const int p = (int)P.par(y);
+        if (k < Sh::KR) P.cell(y, p - MP) = INFINITY;
+        else P.cell(p, y - MP) = INFINITY;
+      }
+    }
+  }
+  const float pmax = __uint_as_float(Lane<Sh>::maxu(pm));
+  const float dmax = __uint_as_float(Lane<Sh>::maxu(dm));
+  __syncwarp();
+  if (Lane<Sh>::oru(bad ? 1u : 0u)) { *D64 = NAN; go = false; }
+  if (!isfinite(D) || !isfinite(pmax) || !isfinite(dmax) || !(cmax < FLT_MAX)) go = false;
+  const float tau = fmaxf(__fmul_rd(__double2float_rd(D), 0x1p-24f), __fmul_rd(cmax, 0x1p-43f));
+  if (go) *tau_out = tau;
+  const float err = __fmul_ru((float)(P.N + 1),
+                              __fmaf_ru((float)(6 * cv.d + 32) * 0x1p-48f, cmax,
+                                        __fmul_ru(dmax, 0x1p-24f)));
+  const float E = __fmul_ru(__fadd_ru(ecost, __fmul_ru(__fmaf_ru(5.f, pmax, 2.f * cmax), 0x1p-24f)),
+                            1.f + 0x1p-10f);
+  const float thr = __fsub_ru(__fadd_ru(E, err), tau);
+  const float thr_dd = __fsub_ru(err, tau);
+  // pass 1: the FP32 test of every cell (a NaN reduced cost is flagged)
+  bool flagged = false;
+  const bool col = go && P.gl < P.nb;
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int mq = (P.m + 3) >> 2;
+  if (col) {
+    v = P.pot4((MP >> 2) + P.gl);
+    for (int q = P.rg; q < mq; q += Sh::RS) {
+      const float4 u4 = P.pot4(q);
+      const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float u = uu[i];
+        const float4 c = P.tile4(4 * q + i, P.gl);
+        flagged |= !(c.x - u - v.x >= thr) | !(c.y - u - v.y >= thr) | !(c.z - u - v.z >= thr) |
+                   !(c.w - u - v.w >= thr);
+      }
+    }
+  }
+  bool fail = false;
+  if (__any_sync(kAll, flagged)) {
+    // pass 2 (few pairs): the flagged cells re-priced in double-float
+    int cnt = 0;
+    if (flagged) {
+      for (int q = P.rg; q < mq; q += Sh::RS) {
+        for (int t = 0; t < 16; ++t) {
+          const int a = 4 * q + (t >> 2), r = 4 * P.gl + (t & 3);
+          if (a >= P.m || r >= P.n) continue;
+          if (!(P.cell(a, r) - P.pot(a) - P.pot(MP + r) >= thr)) {
+            ++cnt;
+            float ch, cl;
+            cost_dd(xt, ob, o0, cv, c0, a, r, ch, cl);
+            const float2 pu = *reinterpret_cast<float2*>(&P.flow(a));
+            const float2 pv = *reinterpret_cast<float2*>(&P.flow(MP + r));
+            dd_add(ch, cl, -pu.x, -pu.y);
+            dd_add(ch, cl, -pv.x, -pv.y);
+            fail |= !((double)ch + (double)cl >= (double)thr_dd);
+          }
+        }
+      }
+    }
+    *nchk += cnt;
+  }
+  fail = Lane<Sh>::oru(fail ? 1u : 0u) != 0u;
+  P.live = keep_live;
+  __syncwarp();
+  return go && !fail;
+}
+
+// ---- the screen ------------------------------------------------------------
+
+// Objects of the chunk: first list entry and count.
+__device__ __forceinline__ void lane_chunk(const LaneArgs& A, long long total, long long* first,
+                                           long long* cnt) {
+  long long b = A.t0, e = total;
+  if (A.lo) {
+    b += *A.lo;
+    e = *A.hi;
+  }
+  *first = b;
+  const long long c = e - b;
+  *cnt = c < 0 ? 0 : (c < A.cap ? c : A.cap);
+}
+
+template <class Sh, bool CERT>
+__global__ void __launch_bounds__(64, Sh::kMinBlocks)
+    k_lane_screen(ObjView ob, CentView cv, long long seg_size, int K, SolveCfg cfg, LaneArgs A,
+                  long long total_obj) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int NPL = Sh::NPL, PW = Sh::PW;
+  Lane<Sh> P(reinterpret_cast<char*>(smem) + (threadIdx.x >> 5) * A.warp_bytes, A.nb);
+  const int lane = threadIdx.x & 31;
+  long long first, cnt;
+  lane_chunk(A, total_obj, &first, &cnt);
+  const unsigned long long total = A.list ? A.ctr[1] : (unsigned long long)cnt * (unsigned)K;
+  const float rel = (float)(cv.d + 3) * 0x1p-24f + 0x1p-17f;
+  int n_scr = 0, p_scr = 0, n_cert = 0, n_chk = 0;
+  for (;;) {
+    unsigned long long q0 = 0;
+    if (lane == 0) q0 = atomicAdd(A.ctr, (unsigned long long)PW);
+    q0 = __shfl_sync(kAll, q0, 0);
+    if (q0 >= total) break;
+    const unsigned long long q = q0 + (lane & (PW - 1));
+    P.live = q < total;
+    long long tt = 0, i = 0, o0 = 0, c0 = 0, cb = 0;
+    int j = 0;
+    if (P.live) {
+      if (A.list) {
+        const uint2 e = A.list[q];
+        tt = e.x;
+        j = (int)e.y;
+      } else {
+        tt = (long long)(q / (unsigned)K);
+        j = (int)(q - (unsigned long long)tt * (unsigned)K);
+      }
+      i = A.oidx ? (long long)A.oidx[first + tt] : A.obase + first + tt;
+      o0 = ob.off[i];
+      const long long mm = ob.off[i + 1] - o0;
+      cb = seg_of(ob, i, seg_size) * (long long)K;
+      P.live = mm >= 1 && mm <= cfg.mmax && cb + K <= cv.K && !A.obad[i];
+      if (P.live) {
+        c0 = cv.off[cb + j];
+        const long long nn = cv.off[cb + j + 1] - c0;
+        P.live = nn >= 1 && nn <= cfg.nmax;
+        P.m = (int)mm;
+        P.n = (int)nn;
+      }
+    }
+    if (!P.live) P.m = P.n = 1;
+    P.N = P.m + P.n;
+    // masses, singleton masks, potentials of the unused slots
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const int y = P.node(k);
+      long long w = 0;
+      Mask<Sh::MW> d;
+      d.clear();
+      if (P.live && P.nodek(k)) {
+        d.set(y);
+        if (k < Sh::KR) {
+          w = A.omass[i * A.mstride + y];
+        } else {
+          const int r = y - Sh::MP;
+          w = cv.Qpre[c0 + r] - (r > 0 ? cv.Qpre[c0 + r - 1] : 0LL);
+        }
+      }
+      P.store(y, w, d, 0xffu);
+      P.potk(k) = 0.f;
+    }
+    __syncwarp();
+    const float* tile_g = nullptr;
+    float nxm = 0.f;
+    if (cfg.tile.C) {
+      if (P.live) {
+        const long long trow0 = cfg.tile.trow[tt];
+        tile_g = cfg.tile.C + trow0 * cfg.tile.ldc + (c0 - cfg.tile.col0);
+        for (int a = P.g; a < P.m; a += Sh::G) nxm = fmaxf(nxm, cfg.tile.nx[trow0 + a]);
+      } else {
+        tile_g = cfg.tile.C;
+      }
+      nxm = Lane<Sh>::maxf(nxm);
+    }
+    float4 vm;
+    const float cmax = lane_tile<Sh>(P, ob, o0, cv, c0, tile_g, cfg.tile.ldc, vm);
+    P.start_rows(vm);
+    int piv = 0;
+    int st = P.run(cfg.budget * P.N, tol32(cmax), &piv);
+    if (P.live && P.g == 0) {
+      ++n_scr;
+      p_scr += piv;
+    }
+    if (A.tree && P.live) {  // the basis, for the exact pass (parents, compact node numbers)
+      unsigned char* tr = A.tree + q * (unsigned)A.tstride;
+#pragma unroll
+      for (int k = 0; k < NPL; ++k) {
+        if (P.nodek(k)) {
+          const int y = P.node(k);
+          const unsigned p = P.par(y);
+          tr[k < Sh::KR ? y : y - Sh::MP + P.m] =
+              (unsigned char)(y == P.root || st == kStInvalid
+                                  ? 0xffu
+                                  : (p < (unsigned)Sh::MP ? p : p - Sh::MP + P.m));
+        }
+      }
+    }
+    float tc_e = 0.f;
+    if (cfg.tile.C && P.live) tc_e = tc_bound(cv.d, nxm, cfg.tile.cn[cb + j], cfg.tile.cd[cb + j]);
+    PairRec rec;
+    rec.d64 = NAN;
+    if constexpr (CERT) {
+      double D64 = NAN;
+      float tau = 0.f;
+      const float ecost = cfg.tile.C ? tc_e : (cv.A ? 0x1p-23f : (float)(cv.d + 3) * 0x1p-24f) * cmax;
+      const bool cert = lane_certify<Sh>(P, P.live && st == kStOk, ob, o0, cv, c0, cmax, ecost, &D64,
+                                         &tau, &n_chk);
+      const float dhi = __double2float_ru(D64);
+      if (cert) {
+        if (P.g == 0) ++n_cert;
+        rec.lo = __fsub_rd(__fmul_rd(__double2float_rd(D64), 1.f - 0x1p-22f), tau);
+        rec.hi = __fmul_ru(dhi, 1.f + 0x1p-22f);
+        rec.d64 = D64;
+      } else {
+        rec.lo = -FLT_MAX;
+        rec.hi = st == kStOk && isfinite(D64) ? __fmul_ru(dhi, 1.f + 0x1p-22f) : FLT_MAX;
+      }
+      if (P.live && P.g == 0 && cfg.pair64) cfg.pair64[i * (long long)K + j] = rec.d64;
+    } else {
+      // FP32 objective and its error bound
+      float acc = 0.f;
+#pragma unroll
+      for (int k = 0; k < NPL; ++k) {
+        const int y = P.node(k);
+        if (P.live && P.nodek(k) && y != P.root) {
+          const int p = (int)P.par(y);
+          if (p < Sh::NS) acc += ((float)P.flowk(k) * (float)kInvMass) * P.edge_cost(y, p);
+        }
+      }
+      const float D = Lane<Sh>::sum(acc);
+      const float e = D * rel + cmax * 0x1p-14f + tc_e;
+      const bool good = st == kStOk && !isnan(D) && !isnan(e);
+      if (P.live && P.g == 0 && cfg.pair_out) {
+        float* po = cfg.pair_out + 2 * (i * (long long)K + j);
+        po[0] = D;
+        po[1] = st != kStOk ? INFINITY : e;
+      }
+      rec.lo = good ? D - e : -FLT_MAX;
+      rec.hi = good ? D + e : FLT_MAX;
+    }
+    if (q < total && P.g == 0) {
+      if (!P.live) {
+        rec.lo = -FLT_MAX;
+        rec.hi = FLT_MAX;
+        rec.d64 = NAN;
+        if (cfg.pair_out) cfg.pair_out[2 * (i * (long long)K + j)] = NAN;
+        if (cfg.pair64) cfg.pair64[i * (long long)K + j] = NAN;
+      }
+      A.rec[q] = rec;
+    }
+    __syncwarp();
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    n_scr += __shfl_xor_sync(kAll, n_scr, o);
+    p_scr += __shfl_xor_sync(kAll, p_scr, o);
+    n_cert += __shfl_xor_sync(kAll, n_cert, o);
+    n_chk += __shfl_xor_sync(kAll, n_chk, o);
+  }
+  if (lane == 0) add_stats(n_scr, p_scr, 0, 0, n_cert, n_chk);
+}
+
+// ---- the exact pass --------------------------------------------------------
+
+// Exact value of one pair from the basis the screen saved: the basic cells'
+// costs, the objective and the potentials in FP64, and the optimality test of
+// k_exact (no FP64 reduced cost below -2^-43 c_max) with the FP32 tile as its
+// filter: a cell whose FP32 reduced cost clears the rounding bound E of
+// lane_certify has a non-negative FP64 one, the few others are priced in FP64.
+// Returns false when the tree is inconsistent or not optimal (the object then
+// goes to k_exact).  `value`: only the flows are wanted (certified pairs).
+template <class Sh>
+__device__ __forceinline__ bool lane_verify(Lane<Sh>& P, bool go, bool value, char* pot64,
+                                            const ObjView& ob, long long o0, const CentView& cv,
+                                            long long c0, double* D64) {
+  constexpr int NPL = Sh::NPL, MP = Sh::MP, NS = Sh::NS, PS = Sh::PS;
+  constexpr unsigned kAll = 0xffffffffu;
+  P.live = go;
+  auto u64 = [&](int y) -> double& {
+    return *reinterpret_cast<double*>(pot64 + (y >> 1) * PS + (y & 1) * 8);
+  };
+  // flows: the edge above a node carries the net mass of its subtree, summed
+  // by walking every node's mass up to the root (exact integers)
+  bool bad = false;
+  long long b[NPL];
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) {
+    b[k] = P.flowk(k);
+    if (k >= Sh::KR) b[k] = -b[k];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) P.flowk(k) = 0;
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) {
+    if (go && P.nodek(k)) {
+      int x = P.node(k);
+      for (int it = 0; it < NS && x != P.root; ++it) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(&P.flow(x)), (unsigned long long)b[k]);
+        const unsigned p = P.par(x);
+        if (p >= (unsigned)NS || (x < MP) == (p < (unsigned)MP)) { bad = true; break; }
+        x = (int)p;
+      }
+      if (x != P.root) bad = true;  // no way to the root
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = Sh::KR; k < NPL; ++k) P.flowk(k) = -P.flowk(k);
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) bad |= go && P.nodek(k) && P.flowk(k) < 0;
+  bad = Lane<Sh>::oru(bad ? 1u : 0u) != 0u;
+  const bool full = go && value && !bad;
+  if (!__any_sync(kAll, full)) return go && !bad;
+  P.live = full;
+  float4 vm;
+  const float cmax = lane_tile<Sh>(P, ob, o0, cv, c0, nullptr, 0, vm);
+  // basic cells in FP64
+  double edge[NPL];
+#pragma unroll 1
+  for (int k = 0; k < NPL; ++k) {
+    const int y = P.node(k);
+    double c = 0.0;
+    if (full && (k < Sh::KR ? y < P.m : y - MP < P.n) && y != P.root) {
+      const int p = (int)P.par(y);
+      c = y < MP ? cost64_cell(ob, o0, cv, c0, y, p - MP) : cost64_cell(ob, o0, cv, c0, p, y - MP);
+    }
+    u64(y) = c;
+  }
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) edge[k] = u64(P.node(k));
+  __syncwarp();
+  double pot[NPL];
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) pot[k] = edge[k];
+  bool fail = P.jump(pot, u64);
+  float pm = 0.f;
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) {
+    const int y = P.node(k);
+    if (full && P.nodek(k)) {
+      const float u = __double2float_rn(pot[k]);
+      P.pot(y) = u;
+      pm = fmaxf(pm, fabsf(u));
+      fail |= !isfinite(u);
+      if (y != P.root) {  // a basic cell's reduced cost is zero
+        const int p = (int)P.par(y);
+        if (k < Sh::KR) P.cell(y, p - MP) = INFINITY;
+        else P.cell(p, y - MP) = INFINITY;
+      }
+    }
+  }
+  const float pmax = Lane<Sh>::maxf(pm);
+  __syncwarp();
+  const float ecost = (cv.A ? 0x1p-23f : (float)(cv.d + 3) * 0x1p-24f) * cmax;
+  const float E = __fmul_ru(__fadd_ru(ecost, __fmul_ru(__fmaf_ru(5.f, pmax, 2.f * cmax), 0x1p-24f)),
+                            1.f + 0x1p-10f);
+  if (!(cmax < FLT_MAX) || !isfinite(E)) fail = true;
+  const double tol = (double)cmax * (0x1p-43 * (1.0 - 0x1p-12));
+  const int mq = (P.m + 3) >> 2;
+  if (full && P.gl < P.nb) {
+    const float4 v = P.pot4((MP >> 2) + P.gl);
+    const float vv[4] = {v.x, v.y, v.z, v.w};
+    for (int a = 4 * P.rg; a < 4 * mq; a += (a & 3) == 3 ? 4 * Sh::RS - 3 : 1) {
+      const float u = P.pot(a);
+      const float4 c = P.tile4(a, P.gl);
+      const float cc[4] = {c.x, c.y, c.z, c.w};
+      unsigned flag = 0u;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) flag |= !(cc[t] - u - vv[t] >= E) ? 1u << t : 0u;
+      for (; flag; flag &= flag - 1) {
+        const int r = 4 * P.gl + __ffs((int)flag) - 1;
+        if (a < P.m && r < P.n)
+          fail |= !(cost64_cell(ob, o0, cv, c0, a, r) - u64(a) - u64(MP + r) >= -tol);
+      }
+    }
+  }
+  // objective (the flow slots become its terms; kept for the flow records)
+  long long fl[NPL];
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) {
+    fl[k] = P.flowk(k);
+    if (full && P.nodek(k))
+      *reinterpret_cast<double*>(&P.flowk(k)) = ((double)fl[k] * kInvMass) * edge[k];
+  }
+  const double D = P.sum_nodes();
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) P.flowk(k) = fl[k];
+  __syncwarp();
+  if (full) *D64 = D;
+  fail |= full && !isfinite(D);
+  fail = Lane<Sh>::oru(fail ? 1u : 0u) != 0u;
+  return go && !bad && !(full && fail);
+}
+
+// The candidates of the chunk's objects (k_lane_merge's records) to their
+// labels and exact distances, as k_exact; an object with a candidate that
+// does not verify is listed for k_exact (fb, counted in ctr[2]).
+template <class Sh>
+__global__ void __launch_bounds__(64, Sh::kMinBlocks)
+    k_lane_exact(ObjView ob, CentView cv, long long seg_size, int K, SolveCfg cfg, LaneArgs A,
+                 long long total_obj, ExactOut X) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int NPL = Sh::NPL, PW = Sh::PW, MP = Sh::MP;
+  char* warp_base = reinterpret_cast<char*>(smem) + (threadIdx.x >> 5) * A.warp_bytes;
+  Lane<Sh> P(warp_base, A.nb);
+  char* pot64 = warp_base + A.warp_bytes - (Sh::NS / 2) * Sh::PS + (P.sp - warp_base);
+  const int lane = threadIdx.x & 31;
+  long long first, cnt;
+  lane_chunk(A, total_obj, &first, &cnt);
+  int n_ex = 0;
+  const long long step = (long long)gridDim.x * (blockDim.x >> 5) * PW;
+  for (long long t0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PW; t0 < cnt;
+       t0 += step) {
+    const long long t = t0 + (lane & (PW - 1));
+    const bool have = t < cnt;
+    long long i = 0, o0 = 0, cb = 0;
+    const int* mr = X.cand;
+    int nc = 0;
+    if (have) {
+      i = A.oidx ? (long long)A.oidx[first + t] : A.obase + first + t;
+      mr = X.cand + i * kMergedInts;
+      nc = mr[0];
+      o0 = ob.off[i];
+      P.m = (int)(ob.off[i + 1] - o0);
+      cb = seg_of(ob, i, seg_size) * (long long)K;
+    }
+    const bool invalid = have && nc == -2;
+    bool fallback = have && (nc == -1 || nc == 0);
+    if (!have || nc < 1) { nc = 0; P.m = 1; }
+    double d64c = NAN;
+    if (cfg.certify && nc == 1)
+      d64c = __longlong_as_double(((long long)mr[2 + kCandCap] << 32) |
+                                  (long long)(unsigned)mr[1 + kCandCap]);
+    const bool known = !isnan(d64c);
+    double best = NAN;
+    int best_j = -1;
+    for (int c = 0; __any_sync(kAll, c < nc); ++c) {
+      const bool go = c < nc && !fallback && (!known || X.fo.cell);
+      int j = 0;
+      long long c0 = 0;
+      P.n = 1;
+      unsigned long long q = 0;
+      if (go) {
+        j = mr[1 + c];
+        c0 = cv.off[cb + j];
+        P.n = (int)(cv.off[cb + j + 1] - c0);
+        if (A.list) {  // the pair's place in the list: kept centroids before j
+          const unsigned* kb = cfg.keep + i * cfg.keep_words;
+          q = X.ostart[t] + __popc(kb[j >> 5] & ((1u << (j & 31)) - 1u));
+          for (int w = 0; w < (j >> 5); ++w) q += __popc(kb[w]);
+        } else {
+          q = (unsigned long long)t * (unsigned)K + (unsigned)j;
+        }
+      }
+      P.N = P.m + P.n;
+      P.live = go;
+      // masses and the saved tree
+      const unsigned char* tr = A.tree + q * (unsigned)A.tstride;
+      int root = INT_MAX;
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < NPL; ++k) {
+        const int y = P.node(k);
+        long long w = 0;
+        unsigned p = 0xffu;
+        if (go && P.nodek(k)) {
+          if (k < Sh::KR) {
+            w = A.omass[i * A.mstride + y];
+          } else {
+            const int r = y - MP;
+            w = cv.Qpre[c0 + r] - (r > 0 ? cv.Qpre[c0 + r - 1] : 0LL);
+          }
+          p = tr[k < Sh::KR ? y : y - MP + P.m];
+          if (p == 0xffu) root = min(root, y);
+          else if (p >= (unsigned)P.m) p = p - P.m + MP;
+        }
+        Mask<Sh::MW> none;
+        none.clear();
+        P.store(y, w, none, p);
+        P.potk(k) = 0.f;
+      }
+#pragma unroll
+      for (int o = Sh::G / 2; o > 0; o >>= 1)
+        root = min(root, __shfl_xor_sync(kAll, root, o * PW));
+      P.root = root == INT_MAX ? 0 : root;
+      __syncwarp();
+      double D = d64c;
+      const bool ok = lane_verify<Sh>(P, go, !known, pot64, ob, o0, cv, c0, &D);
+      if (go && !ok) fallback = true;
+      if (go && ok && !known && P.g == 0) {
+        ++n_ex;
+        if (cfg.pair64) cfg.pair64[i * (long long)K + j] = D;
+      }
+      const bool better = c < nc && !fallback && (best_j < 0 || D < best);
+      if (better) {
+        best = D;
+        best_j = mr[1 + c];
+        if (X.fo.cell) {  // basis flows: one entry per node but the root
+          int* fc = X.fo.cell + i * X.fo.stride;
+          double* fw = X.fo.w + i * X.fo.stride;
+          const int rc = P.root < MP ? P.root : P.root - MP + P.m;
+#pragma unroll
+          for (int k = 0; k < NPL; ++k) {
+            const int y = P.node(k);
+            if (P.nodek(k) && y != P.root) {
+              const int p = (int)P.par(y);
+              const int e = k < Sh::KR ? y : y - MP + P.m;
+              fc[e < rc ? e : e - 1] = k < Sh::KR ? (y << 16) | (p - MP) : (p << 16) | (y - MP);
+              fw[e < rc ? e : e - 1] = (double)P.flowk(k) * kInvMass;
+            }
+          }
+          for (long long e = P.N - 1 + P.g; e < X.fo.stride; e += Sh::G) {
+            fc[e] = -1;
+            fw[e] = 0.0;
+          }
+        }
+      }
+      __syncwarp();
+    }
+    if (have && P.g == 0) {
+      if (fallback) {
+        X.fb[atomicAdd(A.ctr + 2, 1ull)] = (int)i;
+      } else {
+        X.labels[i] = invalid ? -1 : best_j;
+        const double dd = invalid ? NAN : best;
+        X.dist2[i] = dd;
+        if (X.eps_terms) X.eps_terms[i] = (X.omega ? X.omega[i] : 1.0) * dd;
+        if (invalid) atomicOr(X.err, kErrInvalid);
+      }
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) n_ex += __shfl_xor_sync(kAll, n_ex, o);
+  if (lane == 0) add_stats(0, 0, n_ex, 0);
+}
+
+// Blocks of two warps where they fit, one otherwise.
+template <typename Kern, typename... Args>
+cudaError_t lane_blocks(Kern kern, int warp_bytes, int sms, long long warps_of_work,
+                        cudaStream_t st, const Args&... args) {
+  const int warps = 2 * warp_bytes <= 113 * 1024 ? 2 : 1;
+  const size_t smem = (size_t)warp_bytes * warps;
+  unsigned grid = 1;
+  const cudaError_t e = launch_cfg(kern, smem, 32 * warps, sms, warps_of_work, warps, &grid);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, 32 * warps, smem, st>>>(args...);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+// One launch of the shape: the screen (X.labels null) or the exact pass.
+template <class Sh>
+cudaError_t lane_launch(const ObjView& ob, const CentView& cv, long long seg_size, int K,
+                        const SolveCfg& cfg, LaneArgs A, long long total_obj, long long work,
+                        const ExactOut& X, cudaStream_t st) {
+  A.nb = (cfg.nmax + 3) / 4;
+  if (cfg.mmax > Sh::MP || A.nb > Sh::L) return cudaErrorInvalidConfiguration;
+  A.warp_bytes = (int)lane_warp_bytes<Sh>(cfg.mmax, A.nb);
+  const long long warps = (work + Sh::PW - 1) / Sh::PW;
+  if (X.labels) {
+    A.warp_bytes += Sh::NS / 2 * Sh::PS;  // FP64 potentials
+    return lane_blocks(k_lane_exact<Sh>, A.warp_bytes, cfg.sms, warps, st, ob, cv, seg_size, K, cfg,
+                       A, total_obj, X);
+  }
+  if (cfg.certify)
+    return lane_blocks(k_lane_screen<Sh, true>, A.warp_bytes, cfg.sms, warps, st, ob, cv, seg_size,
+                       K, cfg, A, total_obj);
+  return lane_blocks(k_lane_screen<Sh, false>, A.warp_bytes, cfg.sms, warps, st, ob, cv, seg_size, K,
+                     cfg, A, total_obj);
+}
+
+}  // namespace
+}  // namespace d2k

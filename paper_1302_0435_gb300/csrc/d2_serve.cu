@@ -126,6 +126,7 @@ struct d2_server {
   d2k::CentView cv{};
   int nmax = 0, d = 0, mode = 1, budget_pivots = 64, sms = 1, start = 0;
   long long K = 0;
+  bool lanes = false;  // the lane screen (no cold-start rule fixed by the caller)
   // means and spreads of the resident centroids (pruning; null: off)
   double* d_cmu = nullptr;
   double* d_cvar = nullptr;
@@ -140,6 +141,12 @@ struct d2_server {
   long long next_ticket = 1;
   long long admitted = 0, completed = 0, peak_inflight = 0;
 
+  long long chunk_objects() const {
+    return std::max<long long>(1, kChunkPairs / std::max<long long>(K, 1));
+  }
+  long long scratch_ints(const std::shared_ptr<Request>& r) const {
+    return d2k::assign_scratch_ints(r->count, K, sms, r->mmax, nmax, chunk_objects() * K);
+  }
   bool launch(Slot& s, const std::shared_ptr<Request>& r);
   void run();
 };
@@ -160,7 +167,7 @@ bool d2_server::launch(Slot& s, const std::shared_ptr<Request>& r) {
       !grow_dev(&s.d_off, &s.n_off, b_off) || !grow_dev(&s.d_order, &s.n_order, b_ord + 16) ||
       !grow_dev(&s.d_lab, &s.n_lab, (size_t)N * 4 + 16) ||
       !grow_dev(&s.d_d2, &s.n_d2, (size_t)N * 8 + 16) ||
-      !grow_dev(&s.d_cand, &s.n_cand, (size_t)d2k::assign_scratch_ints(N, K, sms) * 4 + 16) ||
+      !grow_dev(&s.d_cand, &s.n_cand, (size_t)scratch_ints(r) * 4 + 16) ||
       (d_cmu && (!grow_dev(&s.d_mu, &s.n_mu, (size_t)N * r->dim * 8 + 16) ||
                  !grow_dev(&s.d_var, &s.n_var, (size_t)N * 8 + 16) ||
                  !grow_dev(&s.d_keep, &s.n_keep, (size_t)N * ((K + 31) / 32) * 4 + 16))) ||
@@ -193,6 +200,8 @@ bool d2_server::launch(Slot& s, const std::shared_ptr<Request>& r) {
   cfg.budget = budget_pivots;
   cfg.sms = sms;
   cfg.start = start;
+  cfg.lanes = lanes;
+  cfg.max_pairs = chunk_objects() * K;
   d2k::FlowOut fo{nullptr, nullptr, 0};
   if (d_cmu && cfg.mode == 1) {
     // skip the pairs that cannot be an object's argmin (d2k::prune_keep)
@@ -208,7 +217,7 @@ bool d2_server::launch(Slot& s, const std::shared_ptr<Request>& r) {
   }
   // bounded chunks, bin by bin (largest trees first); one stream, so the
   // chunks of a request run in order and share its scratch
-  const long long per = std::max<long long>(1, kChunkPairs / std::max<long long>(K, 1));
+  const long long per = chunk_objects();
   for (int b = 3; b >= 0; --b) {
     const long long b0 = r->bstart[b], b1 = r->bstart[b + 1];
     for (long long t0 = b0; t0 < b1; t0 += per) {
@@ -331,6 +340,7 @@ namespace d2k {
 CentView ctx_centroids(const d2_ctx* c, int* nmax, int* d, int* device, int* mode, int* budget,
                        int* sms, long long* K, int* start);
 bool ctx_prune(const d2_ctx* c);
+bool ctx_lanes(const d2_ctx* c);
 }
 
 extern "C" int d2_server_create(d2_server** out, d2_ctx* ctx, int32_t nslots, int64_t mem_budget) {
@@ -343,6 +353,7 @@ extern "C" int d2_server_create(d2_server** out, d2_ctx* ctx, int32_t nslots, in
   sv->cv = d2k::ctx_centroids(ctx, &sv->nmax, &sv->d, &sv->device, &mode, &sv->budget_pivots, &sv->sms,
                               &sv->K, &sv->start);
   sv->mode = mode;
+  sv->lanes = d2k::ctx_lanes(ctx);
   if (sv->K == 0) {
     delete sv;
     return D2_ENOCENTROIDS;
@@ -439,7 +450,7 @@ extern "C" int d2_server_submit(d2_server* sv, const d2_bags* objs, int64_t* tic
     const int m = (int)(objs->off[i + 1] - objs->off[i]);
     r->order[fill[(m + sv->nmax + 31) / 32 - 1]++] = (int)i;
   }
-  const long long per = std::max<long long>(1, kChunkPairs / std::max<long long>(sv->K, 1));
+  const long long per = sv->chunk_objects();
   for (int b = 0; b < 4; ++b) r->chunks += (cnt[b] + per - 1) / per;
   r->count = N;
   r->dim = objs->dim;
@@ -452,7 +463,7 @@ extern "C" int d2_server_submit(d2_server* sv, const d2_bags* objs, int64_t* tic
   r->w.assign(static_cast<const unsigned char*>(objs->w), static_cast<const unsigned char*>(objs->w) + b_w);
   r->off.assign(objs->off, objs->off + N + 1);
   r->bytes = b_loc + b_w + (size_t)(N + 1) * 8 + (size_t)N * (4 + 4 + 8) +
-             (size_t)d2k::assign_scratch_ints(N, sv->K, sv->sms) * 4;
+             (size_t)sv->scratch_ints(r) * 4;
   r->t_submit = std::chrono::steady_clock::now();
   {
     std::lock_guard<std::mutex> lk(sv->mu);

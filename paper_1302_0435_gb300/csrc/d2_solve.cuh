@@ -640,13 +640,13 @@ __global__ void __launch_bounds__(128) k_pairs64(ObjView ob, CentView cv, const 
 // bits), and the block's smallest upper end (float bits).
 
 // Objects of a launch: their count and list (oidx, or obase.. when null);
-// with a device-side range the count is read here (SolveCfg::dev_range).
+// with a device-side range the count is read here (SolveCfg::dev_lo).
 __device__ __forceinline__ long long launch_objects(const SolveCfg& cfg, long long count,
                                                     const int** oidx) {
-  if (cfg.dev_range) {
-    const long long lo = cfg.dev_range[0];
+  if (cfg.dev_lo) {
+    const long long lo = *cfg.dev_lo;
     *oidx = cfg.oidx + lo;
-    return cfg.dev_range[1] - lo;
+    return *cfg.dev_hi - lo;
   }
   *oidx = cfg.oidx;
   return cfg.nobj >= 0 ? cfg.nobj : count;
@@ -744,17 +744,40 @@ __device__ __forceinline__ void dd_sq_acc(float xv, float yv, float& H, float& L
   H = t;
 }
 
+// The same step on two coordinates at once (even and odd, each lane of the
+// pair rounded on its own): the packed FP32 operations take one issue slot
+// for both.
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+  s = __fadd2_rn(a, b);
+  const float2 bb = __fadd2_rn(s, neg2(a));
+  e = __fadd2_rn(__fadd2_rn(a, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(b, neg2(bb)));
+}
+__device__ __forceinline__ void dd_sq_acc2(float2 xv, float2 yv, float2& H, float2& L) {
+  float2 s, e;
+  two_sum2(xv, neg2(yv), s, e);
+  const float2 p = __fmul2_rn(s, s);
+  const float2 q = __ffma2_rn(s, s, neg2(p));
+  const float2 rr = __ffma2_rn(__fadd2_rn(s, s), e, q);
+  float2 t, z;
+  two_sum2(H, p, t, z);
+  L = __fadd2_rn(L, __fadd2_rn(z, rr));
+  H = t;
+}
+
 // Two independent running sums (even and odd coordinates) shorten the
 // dependent chain; they are added exactly at the end (two-sum).
 template <typename X>
 __device__ __forceinline__ void cost_dd_x(const X* __restrict__ x, const float* __restrict__ y,
                                           int d, float& hi, float& lo) {
-  float H0 = 0.f, L0 = 0.f, H1 = 0.f, L1 = 0.f;
+  float2 H = make_float2(0.f, 0.f), Lo = make_float2(0.f, 0.f);
   int k = 0;
-  for (; k + 1 < d; k += 2) {
-    dd_sq_acc(cvt<float>(x[k]), y[k], H0, L0);
-    dd_sq_acc(cvt<float>(x[k + 1]), y[k + 1], H1, L1);
-  }
+#pragma unroll 1
+  for (; k + 1 < d; k += 2)
+    dd_sq_acc2(make_float2(cvt<float>(x[k]), cvt<float>(x[k + 1])), make_float2(y[k], y[k + 1]), H,
+               Lo);
+  float H0 = H.x, L0 = Lo.x;
+  const float H1 = H.y, L1 = Lo.y;
   if (k < d) dd_sq_acc(cvt<float>(x[k]), y[k], H0, L0);
   float t, z;
   two_sum(H0, H1, t, z);
@@ -1495,9 +1518,9 @@ static cudaError_t assign_g(const ObjView& ob, const CentView& cv, long long seg
   const bool screen = cfg.mode == 1 && cand != nullptr;
   // with a device-side range the count is not known here: persistent
   // grids, sized by the batch
-  const long long nobj = cfg.dev_range ? ob.count : (cfg.nobj >= 0 ? cfg.nobj : ob.count);
+  const long long nobj = cfg.dev_lo ? ob.count : (cfg.nobj >= 0 ? cfg.nobj : ob.count);
   if (nobj <= 0) return cudaSuccess;
-  if (screen) {
+  if (screen && !cfg.screened) {
     // scratch layout: [queue counter: 4 ints][merged lists: count*kMergedInts][items]
     unsigned long long* queue = reinterpret_cast<unsigned long long*>(cand);
     int* merged = cand + 4;
@@ -1511,7 +1534,7 @@ static cudaError_t assign_g(const ObjView& ob, const CentView& cv, long long seg
       // (centroid_blocks) from the launch's object count
       int NB, KB;
       centroid_blocks(sc, cnt, K, &NB, &KB);
-      const long long work = sc.dev_range ? (1LL << 40) : cnt * (long long)NB;
+      const long long work = sc.dev_lo ? (1LL << 40) : cnt * (long long)NB;
       cudaError_t e2 = cudaMemsetAsync(queue, 0, sizeof(unsigned long long), st);
       if (e2 != cudaSuccess) return e2;
       const size_t sl = sc.tile.C ? slice_tc : slice32;
@@ -1536,7 +1559,7 @@ static cudaError_t assign_g(const ObjView& ob, const CentView& cv, long long seg
       return cudaGetLastError();
     };
     if (tw && tw->C && cfg.mmax <= 64) {
-      if (cfg.dev_range) return cudaErrorInvalidValue;  // chunks are cut on the host
+      if (cfg.dev_lo) return cudaErrorInvalidValue;  // chunks are cut on the host
       // tensor-core tiles, chunk by chunk within the tile buffer
       const long long per = std::max<long long>(1, tw->rows_cap / cfg.mmax);
       for (long long t0 = 0; t0 < nobj; t0 += per) {
@@ -1564,7 +1587,7 @@ static cudaError_t assign_g(const ObjView& ob, const CentView& cv, long long seg
   }
   if (screen && cfg.screen_only) return cudaGetLastError();
   e = launch_cfg(k_exact<G, NPL, ST>, smem, gpb * G, cfg.sms,
-                 cfg.dev_range ? (1LL << 40) : nobj, gpb, &grid);
+                 cfg.dev_lo ? (1LL << 40) : nobj, gpb, &grid);
   if (e != cudaSuccess) return e;
   WarmStore wx = ws;
   if (!screen) wx.par8 = nullptr;

@@ -1,0 +1,95 @@
+"""The screen that runs several pairs per warp, at the edges of its shapes.
+
+A launch's row bound picks the lanes per pair and the node slots per lane, the
+centroid bound the column lanes, so the sizes are the bounds of every shape and
+their neighbours, in one launch (small batch) and cut into bins (large batch).
+Every D^2 is certified within 2^-24 D^2 + 2^-43 c_max of the optimum, so the
+oracle's values may differ by 1e-7 relative plus 1e-12 of the largest cost.
+"""
+import numpy as np
+import pytest
+
+from paper_1302_0435_gb300.synth import Bags
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [1, 2, 4, 5, 8, 9, 12, 13, 16, 17, 24, 25, 32, 33, 48, 49, 63, 64]
+
+
+@pytest.fixture(scope="module")
+def d2():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1302_0435_gb300 import build, d2 as mod
+    build.build()
+    mod.load()
+    return mod
+
+
+def bags(rng, sizes, d, law):
+    """normal: scattered supports; lattice: integer supports and weights
+    (equal costs, zero and equal masses); far: bags far apart."""
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    T = int(off[-1])
+    if law == "lattice":
+        loc = rng.integers(0, 3, size=(T, d)).astype(np.float32)
+        w = rng.integers(0, 3, size=T).astype(np.float32)
+        w[off[:-1]] += 1.0
+    else:
+        loc = rng.normal(size=(T, d)).astype(np.float32)
+        if law == "far":
+            loc += np.repeat(rng.normal(0, 20, size=(len(sizes), d)), sizes, axis=0).astype(np.float32)
+        w = rng.exponential(size=T).astype(np.float32)
+    return Bags(loc, w, off, "f32", "f32")
+
+
+def run_all(d2, objs, cents):
+    import torch
+    ctx = d2.Context(0)
+    d2.d2_set_centroids(ctx, d2.bags_from_synth(cents, device="cuda:0"))
+    ob = d2.bags_from_synth(objs, device="cuda:0")
+    N, K = objs.count, cents.count
+    every = torch.empty((N, K), dtype=torch.float64, device="cuda:0")
+    lab = torch.empty(N, dtype=torch.int32, device="cuda:0")
+    dist = torch.empty(N, dtype=torch.float64, device="cuda:0")
+    assert d2.d2_mallows_all(ctx, ob, every, lab, dist) == d2.D2_OK
+    d2.d2_sync(ctx)
+    lab2, dist2 = torch.empty_like(lab), torch.empty_like(dist)
+    assert d2.d2_assign(ctx, ob, lab2, dist2) == d2.D2_OK
+    d2.d2_sync(ctx)
+    ctx.close()
+    return [t.cpu().numpy() for t in (every, lab, dist, lab2, dist2)]
+
+
+def check(oracle_mod, objs, cents, out, rows):
+    every, lab, dist, lab2, dist2 = out
+    sub = objs.subset(rows)
+    _, _, ref = oracle_mod.assign(sub, cents, nthreads=8, return_all=True)
+    big = float(np.max(np.abs(objs.loc))) + float(np.max(np.abs(cents.loc)))
+    floor = 1e-12 * objs.dim * big * big
+    assert np.all(np.abs(every[rows] - ref) <= 1e-7 * ref + floor)
+    for l, dd in ((lab, dist), (lab2, dist2)):
+        at = ref[np.arange(len(rows)), l[rows]]
+        assert np.all(at <= ref.min(axis=1) * (1 + 1e-9) + floor)
+        assert np.all(np.abs(dd[rows] - at) <= 1e-7 * at + floor)
+
+
+@pytest.mark.parametrize("law", ["normal", "lattice", "far"])
+@pytest.mark.parametrize("n,d", [(1, 3), (4, 6), (15, 6), (16, 16), (17, 5), (20, 1), (32, 32),
+                                 (33, 3), (64, 8)])
+def test_shapes(d2, oracle_mod, n, d, law):
+    rng = np.random.default_rng(1000 * n + d + len(law))
+    objs = bags(rng, np.asarray(EDGES * 2), d, law)
+    cents = bags(rng, np.asarray([n, max(1, n - 1), n, max(1, n // 2)]), d, law)
+    check(oracle_mod, objs, cents, run_all(d2, objs, cents), np.arange(objs.count))
+
+
+@pytest.mark.parametrize("n", [16, 32, 64])
+def test_bins(d2, oracle_mod, n):
+    """A batch large enough to be sorted by size and cut into launches."""
+    rng = np.random.default_rng(n)
+    objs = bags(rng, rng.choice(EDGES, size=4500), 4, "far")
+    cents = bags(rng, np.full(6, n), 4, "far")
+    rows = np.sort(rng.choice(objs.count, size=120, replace=False))
+    check(oracle_mod, objs, cents, run_all(d2, objs, cents), rows)
