@@ -46,7 +46,7 @@ enum Slot {
   // d2_mallows_all
   kAllLab, kAllD2, kAllPair,
   // pruning of pairs that cannot be the argmin
-  kPrMuO, kPrVarO, kPrMuC, kPrVarC, kPrKeep,
+  kPrMuO, kPrVarO, kPrMuC, kPrVarC, kPrKeep, kPrMuT, kPrCn, kPrVb, kPrMass, kPrBad,
   kSlots
 };
 
@@ -490,14 +490,19 @@ bool prunes(const d2_ctx* c, const SolveCfg& base, const CentView& cv) {
   return base.mode == 1 && !base.certify && !base.pair64 && cv.A == 0 && !c->cfg.no_prune;
 }
 
-// The bags' means and spreads into the slots run_assign reads (the rounds
-// of a level reuse them: the bags do not change).
-int prune_moments(d2_ctx* c, const ObjView& v) {
+// The bags' masses, and with `moments` their means and spreads, into the slots
+// run_assign reads (the rounds of a level reuse them: the bags do not change).
+int prep_bags(d2_ctx* c, const ObjView& v, int mmax, bool moments) {
   int rc = D2_OK;
-  double* mu_o = static_cast<double*>(grow(c, kPrMuO, (size_t)v.count * v.d * 8, &rc));
-  double* var_o = static_cast<double*>(grow(c, kPrVarO, (size_t)v.count * 8, &rc));
+  long long* mass = static_cast<long long*>(grow(c, kPrMass, (size_t)v.count * mmax * 8, &rc));
+  unsigned char* bad = static_cast<unsigned char*>(grow(c, kPrBad, (size_t)v.count, &rc));
+  double *mu = nullptr, *var = nullptr;
+  if (moments) {
+    mu = static_cast<double*>(grow(c, kPrMuO, (size_t)v.count * v.d * 8, &rc));
+    var = static_cast<double*>(grow(c, kPrVarO, (size_t)v.count * 8, &rc));
+  }
   if (rc != D2_OK) return rc;
-  CK(d2k::bag_moments(v, mu_o, var_o, c->stream));
+  CK(d2k::bag_prep(v, nullptr, mmax, mass, bad, mmax, mu, var, c->stream));
   return D2_OK;
 }
 
@@ -505,26 +510,37 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
                int mmax, const double* om, int* lab, double* d2o, double* terms, FlowOut fo,
                int* cand, const d2k::WarmStore* ws, Bins& bins,
                const d2k::TcWork* tw = nullptr, bool certify_all = false,
-               double* pair64 = nullptr, bool obj_moments_ready = false) {
+               double* pair64 = nullptr, bool bags_ready = false) {
   const int nmax = std::max(c->nmax, 1);
   SolveCfg base = solve_cfg(c, mode, mmax);
   if (certify_all && mode == 1) base.certify = true;
   base.pair64 = pair64;
-  if (prunes(c, base, cv)) {
+  const bool prune = prunes(c, base, cv);
+  if (base.mode == 1 && (prune || base.lanes)) {
+    // (a level prepares its bags once: prep_bags)
+    int rc = D2_OK;
+    if (!bags_ready && (rc = prep_bags(c, v, mmax, prune))) return rc;
+    base.mass = static_cast<const long long*>(c->slot[kPrMass].p);
+    base.bad = static_cast<const unsigned char*>(c->slot[kPrBad].p);
+    base.mstride = mmax;
+  }
+  if (prune) {
     // pairs whose lower bound is above their object's upper bound cannot be
     // the argmin: bounds from the bags' means and spreads, keep bits per object
     int rc = D2_OK;
     const int kw = (K + 31) / 32;
-    double* mu_o = static_cast<double*>(grow(c, kPrMuO, (size_t)v.count * v.d * 8, &rc));
-    double* var_o = static_cast<double*>(grow(c, kPrVarO, (size_t)v.count * 8, &rc));
-    double* mu_c = static_cast<double*>(grow(c, kPrMuC, (size_t)cv.K * cv.d * 8, &rc));
-    double* var_c = static_cast<double*>(grow(c, kPrVarC, (size_t)cv.K * 8, &rc));
+    d2k::CentMoments cm;
+    cm.mu = static_cast<double*>(grow(c, kPrMuC, (size_t)cv.K * cv.d * 8, &rc));
+    cm.var = static_cast<double*>(grow(c, kPrVarC, (size_t)cv.K * 8, &rc));
+    cm.muT32 = static_cast<float*>(grow(c, kPrMuT, (size_t)cv.K * cv.d * 4, &rc));
+    cm.cn = static_cast<float*>(grow(c, kPrCn, (size_t)cv.K * 4, &rc));
+    cm.vb = static_cast<float2*>(grow(c, kPrVb, (size_t)cv.K * 8, &rc));
     unsigned* keep = static_cast<unsigned*>(grow(c, kPrKeep, (size_t)v.count * kw * 4, &rc));
     if (rc != D2_OK) return rc;
-    // (a level computes its bags' moments once: prune_moments)
-    if (!obj_moments_ready) CK(d2k::bag_moments(v, mu_o, var_o, c->stream));
-    CK(d2k::cent_moments(cv, mu_c, var_c, c->stream));
-    CK(d2k::prune_keep(v, seg, K, cv.K, v.d, mu_o, var_o, mu_c, var_c, keep, kw, c->stream));
+    CK(d2k::cent_moments(cv, cm, c->stream));
+    CK(d2k::prune_keep(v, seg, K, cv.K, v.d, static_cast<const double*>(c->slot[kPrMuO].p),
+                       static_cast<const double*>(c->slot[kPrVarO].p), cm, keep, kw, nullptr,
+                       c->stream));
     base.keep = keep;
     base.keep_words = kw;
   }
@@ -1841,9 +1857,8 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     Bins bins;
     if (want_bins(c, cfg, n_l, cur_mmax, ws.par8 != nullptr) && (rc = make_bins(c, cur, &bins)))
       return rc;
-    // the pruning moments of this level's bags, once for all its rounds
-    const bool moments = prunes(c, cfg, cv);
-    if (moments && (rc = prune_moments(c, cur))) return rc;
+    // this level's bags (masses, pruning moments), once for all its rounds
+    if (cfg.mode == 1 && (rc = prep_bags(c, cur, cur_mmax, prunes(c, cfg, cv)))) return rc;
     // Rounds 2.. repeat the same launches (same pairs, warm bases): round 1
     // is captured into a CUDA graph once and replayed.
     cudaGraphExec_t gexec = nullptr;
@@ -1887,7 +1902,7 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
       cudaStreamIsCapturing(c->stream, &cst);
       const bool capturing = cst == cudaStreamCaptureStatusActive;
       int rc2 = run_assign(c, cur, cv, seg, K, cfg.mode, cur_mmax, om, lab, ld2, lterms, fo, cand,
-                           ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr, moments);
+                           ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr, cfg.mode == 1);
       cudaError_t ue = cudaSuccess;
       if (rc2 == D2_OK && it < iters && alg1) {
         // Alg. 1 Step 1: support weights of every cluster of the level by the
@@ -1927,7 +1942,7 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
           // run the round directly instead
           if ((rc = run_assign(c, cur, cv, seg, K, cfg.mode, cur_mmax, om, lab, ld2, lterms, fo,
                                cand, ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr,
-                               moments)))
+                               cfg.mode == 1)))
             return rc;
           if (it < iters)
             CK(d2k::update_locations(cur, om, lab, seg, K, fo, KT, loff, d, c->cent_ldt, l32, l64,

@@ -126,6 +126,10 @@ struct SolveCfg {
   // run and the merged lists are in place
   bool lanes = false;
   bool screened = false;
+  // object masses made ahead (bag_prep; null: the screen makes its own)
+  const long long* mass = nullptr;
+  const unsigned char* bad = nullptr;
+  int mstride = 0;
   bool lane_exact = true;  // the exact pass too (needs centroids whose FP32 copy is exact)
   long long max_pairs = 1LL << 24;  // pairs of one lane_screen chunk
   int start = 0;              // cold start basis: 0 ranked northwest staircase, 1 Vogel
@@ -316,15 +320,28 @@ D2_LANE_DECL(f)
 // about the mean), an upper bound of D^2.  So centroid j cannot be object
 // i's argmin when ||mu_i - mu_j||^2 > UB_i = var_i + min_j' (||mu_i -
 // mu_j'||^2 + var_j').  All in FP64, compared with 2^-40 relative margins.
-// Means [count][d] and spreads [count] of a batch (FP64; NaN for a bag the
-// solver rejects, which keeps all its pairs).
-cudaError_t bag_moments(const ObjView& ob, double* mu, double* var, cudaStream_t st);
-// The same for the centroids of a set (masses from Qpre, locations loc64).
-cudaError_t cent_moments(const CentView& cv, double* mu, double* var, cudaStream_t st);
-// Keep bits of every object: kw = ceil(K / 32) words per object.
+// Masses [count][mstride] as the solver uses them, flags of the bags it rejects
+// and (mu, var not null) means [count][d] and spreads [count] of a batch in
+// FP64 (NaN for a rejected bag, which keeps all its pairs).  range: the
+// launch's objects (null: all).
+cudaError_t bag_prep(const ObjView& ob, const SolveCfg* range, int mmax, long long* mass,
+                     unsigned char* bad, int mstride, double* mu, double* var, cudaStream_t st);
+// The same for the centroids of a set (masses from Qpre, locations loc64):
+// mu [K][d], var [K], and the means in FP32, muT32 [d][K], with norms cn [K]
+// and the spreads rounded down and up, vb [K].
+struct CentMoments {
+  double* mu = nullptr;
+  double* var = nullptr;
+  float* muT32 = nullptr;
+  float* cn = nullptr;
+  float2* vb = nullptr;
+};
+cudaError_t cent_moments(const CentView& cv, const CentMoments& cm, cudaStream_t st);
+// Keep bits of every object: kw = ceil(K / 32) words per object; keep_was
+// (optional) receives the bits they replace.
 cudaError_t prune_keep(const ObjView& ob, long long seg_size, int K, long long KT, int d,
-                       const double* mu_o, const double* var_o, const double* mu_c,
-                       const double* var_c, unsigned* keep, int kw, cudaStream_t st);
+                       const double* mu_o, const double* var_o, const CentMoments& cm,
+                       unsigned* keep, int kw, unsigned* keep_was, cudaStream_t st);
 
 // Raise kErrInvalid into d_err unless every location of the T supports is
 // an integer symbol id in [0, A) (d = 1).
@@ -419,10 +436,13 @@ struct UpdateScratch {
   int* seg_label;      // [N] global centroid per object
 };
 size_t update_scratch_bytes(long long N, long long KT);
-// Blocks per centroid of the accumulation: about 512 members each, at most 64.
+// Blocks per centroid of the accumulation: one while the clusters average at
+// most 512 members, else about 64 members each, at most 64 blocks (clusters
+// are uneven, and the largest one's blocks end the launch).
 inline long long update_parts(long long N, long long KT) {
-  const long long u = (N + KT * 512 - 1) / (KT * 512);
-  return u < 1 ? 1 : (u > 64 ? 64 : u);
+  if (N <= KT * 512) return 1;
+  const long long u = (N + KT * 64 - 1) / (KT * 64);
+  return u > 64 ? 64 : u;
 }
 // Room for the per-part sums (0: one block per centroid suffices).
 size_t update_part_bytes(long long N, long long KT, int d);

@@ -152,33 +152,136 @@ __device__ __forceinline__ void bag_mean_var(const Grp<32>& g, const long long* 
   if (g.lane == 0) *var = v;
 }
 
-// One warp per object: the masses the solver will use (load_prefix), then
-// the mean and spread.
-__global__ void k_bag_moments(ObjView ob, double* mu, double* var) {
-  __shared__ long long pre[4][64];
-  Grp<32> g;
-  const int wb = threadIdx.x >> 5;
-  for (long long i = (long long)blockIdx.x * 4 + wb; i < ob.count; i += (long long)gridDim.x * 4) {
-    const long long o0 = ob.off[i];
-    const int m = (int)(ob.off[i + 1] - o0);
-    const int d = ob.d;
-    bool ok = m >= 1 && m <= 64;
-    if (ok) ok = ob.wdt == 0 ? load_prefix<32>(g, static_cast<const double*>(ob.w) + o0, m, pre[wb])
-                             : load_prefix<32>(g, static_cast<const float*>(ob.w) + o0, m, pre[wb]);
-    if (!ok) {
-      if (g.lane == 0) var[i] = NAN;
-      continue;
+// Masses, means and spreads of the bags, 8 lanes per object (4 objects a warp:
+// the FP64 pipe charges a warp instruction the same for 6 active lanes as for
+// 32, and a warp per object kept it at 6 to 16; 200,000 image bags 1.14 ms).
+// The arithmetic is load_prefix's and bag_mean_var's on 32 lanes, sum by sum:
+// slot l of a sum holds supports l and l + 32, and the slots are added in
+// halves (16, 8 within a lane, 4, 2, 1 across lanes), so the values are the
+// same to the last bit.  Masses [count][mstride] and flags (1: a bag the
+// solver rejects), moments optional.
+__device__ __forceinline__ double slots8(const double (&v)[4]) {
+  double x = (v[0] + v[2]) + (v[1] + v[3]);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+__global__ void __launch_bounds__(128) k_bag_prep(ObjView ob, const int* oidx, const long long* lo,
+                                                  const long long* hi, long long obase,
+                                                  long long total, int mmax, long long* mass,
+                                                  unsigned char* bad, int mstride, double* mu,
+                                                  double* var) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31, l8 = lane & 7;
+  const long long first = lo ? *lo : 0;
+  const long long cnt = lo ? *hi - first : total;
+  const int d = ob.d;
+  const long long step = (long long)gridDim.x * 16;
+  for (long long t0 = (long long)blockIdx.x * 16 + (threadIdx.x >> 5) * 4; t0 < cnt; t0 += step) {
+    const long long t = t0 + (lane >> 3);
+    const bool have = t < cnt;
+    const long long i = have ? (oidx ? (long long)oidx[first + t] : obase + first + t) : 0;
+    long long o0 = 0;
+    int m = 0;
+    if (have) {
+      o0 = ob.off[i];
+      const long long mm = ob.off[i + 1] - o0;
+      m = mm >= 1 && mm <= mmax ? (int)mm : 0;
     }
-    const void* loc = ob.loc;
-    const int ldt = ob.ldt;
-    bag_mean_var(g, pre[wb], m, d,
-                 [&](int a, int k) { return ldx<double>(loc, ldt, (o0 + a) * d + k); },
-                 mu + i * d, var + i);
+    double w[8];
+    bool wrong = m == 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int a = l8 + 8 * q;
+      w[q] = 0.0;
+      if (a < m) {
+        w[q] = ob.wdt == 0 ? static_cast<const double*>(ob.w)[o0 + a]
+                           : (double)static_cast<const float*>(ob.w)[o0 + a];
+        wrong |= !(w[q] >= 0.0) || isinf(w[q]);
+      }
+    }
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = w[q] + w[q + 4];
+    const double s = slots8(v);
+    wrong |= !(s > 0.0) || isinf(s);
+    const unsigned wb = __ballot_sync(kAll, wrong) >> (lane & 24);
+    const bool ok = have && (wb & 0xffu) == 0u;
+    const double inv = 1.0 / s;
+    long long qv[8], part = 0, bigv = -1;
+    int bigi = INT_MAX;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int a = l8 + 8 * q;
+      qv[q] = 0;
+      if (ok && a < m) {
+        qv[q] = __double2ll_rn(w[q] * inv * 4611686018427387904.0);
+        if (qv[q] < 0) qv[q] = 0;
+        part += qv[q];
+        if (qv[q] > bigv) { bigv = qv[q]; bigi = a; }
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      part += __shfl_xor_sync(kAll, part, o);
+      const long long ov = __shfl_xor_sync(kAll, bigv, o);
+      const int oi = __shfl_xor_sync(kAll, bigi, o);
+      if (ov > bigv || (ov == bigv && oi < bigi)) { bigv = ov; bigi = oi; }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {  // the rounding residual goes to the largest
+      if (l8 + 8 * q == bigi) qv[q] += kMass - part;
+      if (mass && ok && l8 + 8 * q < m) mass[i * mstride + l8 + 8 * q] = qv[q];
+    }
+    if (bad && have && l8 == 0) bad[i] = ok ? 0 : 1;
+    if (!mu) continue;
+    // mean: a lane per coordinate, supports in order; spread: a lane per
+    // support, coordinates in order
+    double wm[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) wm[q] = (double)qv[q] * kInvMass;
+    const int top = __reduce_max_sync(kAll, ok ? (unsigned)m : 0u);
+    for (int kb = 0; kb < d; kb += 8) {
+      const int k = kb + l8;
+      double acc = 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (8 * q < top) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const double wa = __shfl_sync(kAll, wm[q], (lane & 24) + u);
+            const int a = 8 * q + u;
+            if (ok && a < m && k < d) acc = fma(wa, ldx<double>(ob.loc, ob.ldt, (o0 + a) * d + k), acc);
+          }
+        }
+      }
+      if (ok && k < d) mu[i * d + k] = acc;
+    }
+    __syncwarp();
+    double vs[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int a = l8 + 8 * q;
+      if (ok && a < m) {
+        double s2 = 0.0;
+        for (int k = 0; k < d; ++k) {
+          const double df = ldx<double>(ob.loc, ob.ldt, (o0 + a) * d + k) - mu[i * d + k];
+          s2 = fma(df, df, s2);
+        }
+        vs[q & 3] = fma(wm[q], s2, vs[q & 3]);
+      }
+    }
+    const double vv = slots8(vs);
+    if (have && l8 == 0) var[i] = ok ? vv : (double)NAN;
     __syncwarp();
   }
 }
 
-__global__ void k_cent_moments(CentView cv, double* mu, double* var) {
+// Centroid moments; muT32 [d][K]: the means rounded to FP32, coordinate by
+// coordinate (k_prune_keep reads 32 centroids' worth at once), cn [K]: the
+// FP32 norm of each mean, rounded up, vb [K]: the spread rounded down and up.
+__global__ void k_cent_moments(CentView cv, double* mu, double* var, float* muT32, float* cn, float2* vb) {
   Grp<32> g;
   const int wb = threadIdx.x >> 5;
   for (long long j = (long long)blockIdx.x * 4 + wb; j < cv.K; j += (long long)gridDim.x * 4) {
@@ -189,22 +292,95 @@ __global__ void k_cent_moments(CentView cv, double* mu, double* var) {
     bag_mean_var(g, cv.Qpre + c0, n, d, [&](int r, int k) { return y[r * d + k]; }, mu + j * d,
                  var + j);
     __syncwarp();
+    float s = 0.f;
+    for (int k = g.lane; k < d; k += 32) {
+      const float x = __double2float_rn(mu[j * d + k]);
+      muT32[(long long)k * cv.K + j] = x;
+      s = __fmaf_ru(x, x, s);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s = __fadd_ru(s, __shfl_xor_sync(0xffffffffu, s, o));
+    if (g.lane == 0) {
+      cn[j] = __fsqrt_ru(s);
+      vb[j] = make_float2(__double2float_rd(var[j]), __double2float_ru(var[j]));
+    }
+    __syncwarp();
   }
 }
 
-// One warp per object: UB over its segment's K centroids, then the keep bits.
-__global__ void k_prune_keep(ObjView ob, long long seg_size, int K, long long KT, int d,
-                             const double* mu_o, const double* var_o, const double* mu_c,
-                             const double* var_c, unsigned* keep, int kw) {
-  Grp<32> g;
-  const int wb = threadIdx.x >> 5;
-  for (long long i = (long long)blockIdx.x * 4 + wb; i < ob.count; i += (long long)gridDim.x * 4) {
-    const long long cb = seg_of(ob, i, seg_size) * (long long)K;
-    const double vi = var_o[i];
-    const double* xi = mu_o + i * d;
-    const bool valid = !isnan(vi) && cb + K <= KT;
-    auto lb = [&](int j) {
-      const double* yj = mu_c + (cb + j) * d;
+// One warp per 4 objects of a segment: UB over the segment's K centroids, then
+// the keep bits.  The FP64 rule of the bounds (in d2_internal.h) decides, but
+// only where FP32 cannot: with the means rounded to FP32 (each by at most
+// 2^-24 of its coordinate), s32 = sum (x32 - y32)^2 by FMA is within
+//   e = (d + 4) 2^-24 s32 + 2 sqrt(s32) h + h^2,  h = 2^-23 (|x| + |y|),
+// of the FP64 s; UB is the FP64 minimum over the centroids whose FP32 value
+// plus spread reaches the smallest upper end, and a keep bit is the FP64
+// comparison only where the two intervals meet (about one centroid an object).
+// GB300 runs FP64 at 1/64 of FP32: all in FP64 this took 3.7 ms for 120,000 x
+// 256 in 16 dimensions (twice the K distances of d FP64 terms per object).
+template <int B>
+__global__ void __launch_bounds__(128) k_prune_keep(ObjView ob, long long seg_size, int K,
+                                                    long long KT, int d, const double* mu_o,
+                                                    const double* var_o, const double* mu_c,
+                                                    const double* var_c, const float* muT32,
+                                                    const float* cn, const float2* vb,
+                                                    unsigned* keep, int kw, unsigned* keep_was) {
+  constexpr unsigned kAll = 0xffffffffu;
+  // the objects' means in FP32 (a conversion costs an FP64 issue)
+  __shared__ float xs_[4][B][256];
+  const int lane = threadIdx.x & 31;
+  float(*xs)[256] = xs_[threadIdx.x >> 5];
+  const long long step = (long long)gridDim.x * 4 * B;
+  for (long long i0 = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * B; i0 < ob.count;
+       i0 += step) {
+    long long cb[B];
+    double vi[B], best[B];
+    float hx[B], up[B];
+    bool valid[B];
+    bool same = true;
+    __syncwarp();
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const long long i = min(i0 + b, ob.count - 1);
+      cb[b] = seg_of(ob, i, seg_size) * (long long)K;
+      vi[b] = var_o[i];
+      valid[b] = !isnan(vi[b]) && cb[b] + K <= KT;
+      same &= cb[b] == cb[0];
+      float s = 0.f;
+      for (int k = lane; k < d; k += 32) {
+        const float x = valid[b] ? __double2float_rn(mu_o[i * d + k]) : 0.f;
+        xs[b][k] = x;
+        s = __fmaf_ru(x, x, s);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s = __fadd_ru(s, __shfl_xor_sync(kAll, s, o));
+      hx[b] = __fsqrt_ru(s);
+      up[b] = INFINITY;
+      best[b] = INFINITY;
+    }
+    __syncwarp();
+    auto dist32 = [&](int j, float (&s)[B]) {
+#pragma unroll
+      for (int b = 0; b < B; ++b) s[b] = 0.f;
+      for (int k = 0; k < d; ++k) {
+        float y = same ? __ldg(muT32 + k * KT + min(cb[0] + j, KT - 1)) : 0.f;
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+          if (!same) y = __ldg(muT32 + k * KT + min(cb[b] + j, KT - 1));
+          const float df = xs[b][k] - y;
+          s[b] = fmaf(df, df, s[b]);
+        }
+      }
+    };
+    auto err32 = [&](int b, int j, float s) {
+      const float h = __fmul_ru(__fadd_ru(hx[b], __ldg(cn + min(cb[b] + j, KT - 1))), 0x1p-23f);
+      const float e = __fmaf_ru(__fmul_ru(2.f, __fsqrt_ru(s)), h, __fmul_ru(h, h));
+      return __fadd_ru(__fmul_ru(__fmaf_ru((float)(d + 4) * 0x1p-24f, s, e), 1.f + 0x1p-10f),
+                       FLT_MIN);  // underflow of the squares
+    };
+    auto lb = [&](int b, int j) {  // the FP64 value that decides
+      const double* xi = mu_o + min(i0 + b, ob.count - 1) * d;
+      const double* yj = mu_c + (cb[b] + j) * d;
       double s2 = 0.0;
       for (int k = 0; k < d; ++k) {
         const double df = xi[k] - yj[k];
@@ -212,18 +388,59 @@ __global__ void k_prune_keep(ObjView ob, long long seg_size, int K, long long KT
       }
       return s2;
     };
-    double best = INFINITY;
-    if (valid)
-      for (int j = g.lane; j < K; j += 32) best = fmin(best, lb(j) + var_c[cb + j]);
+    // smallest upper end of s + spread
+    for (int j = lane; j < K; j += 32) {
+      float s[B];
+      dist32(j, s);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
-    const double ub = (vi + best) * (1.0 + 0x1p-40);
+      for (int b = 0; b < B; ++b)
+        if (valid[b])
+          up[b] = fminf(up[b], __fadd_ru(__fadd_ru(s[b], err32(b, j, s[b])), __ldg(vb + cb[b] + j).y));
+    }
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) up[b] = fminf(up[b], __shfl_xor_sync(kAll, up[b], o));
+    for (int j = lane; j < K; j += 32) {
+      float s[B];
+      dist32(j, s);
+#pragma unroll
+      for (int b = 0; b < B; ++b)
+        if (valid[b]) {
+          const float low = __fadd_rd(__fsub_rd(s[b], err32(b, j, s[b])), __ldg(vb + cb[b] + j).x);
+          if (!(low > up[b])) best[b] = fmin(best[b], lb(b, j) + var_c[cb[b] + j]);
+        }
+    }
+    double ub[B];
+    float ubl[B], ubh[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) best[b] = fmin(best[b], __shfl_xor_sync(kAll, best[b], o));
+      ub[b] = (vi[b] + best[b]) * (1.0 + 0x1p-40);
+      ubl[b] = __fmul_rd(__double2float_rd(ub[b]), 1.f - 0x1p-20f);
+      ubh[b] = __fmul_ru(__double2float_ru(ub[b]), 1.f + 0x1p-20f);
+    }
     for (int w = 0; w < kw; ++w) {
-      const int j = w * 32 + g.lane;
-      // keep unless the lower bound is above the upper bound (NaN keeps)
-      const bool k = j < K && (!valid || !(lb(j) * (1.0 - 0x1p-40) > ub));
-      const unsigned bits = __ballot_sync(0xffffffffu, k);
-      if (g.lane == 0) keep[i * kw + w] = bits;
+      const int j = w * 32 + lane;
+      float s[B];
+      dist32(min(j, K - 1), s);
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        // keep unless the lower bound is above the upper bound (NaN keeps)
+        bool k = j < K;
+        if (k && valid[b]) {
+          const float e = err32(b, j, s[b]);
+          if (__fsub_rd(s[b], e) > ubh[b]) k = false;
+          else if (!(__fadd_ru(s[b], e) < ubl[b])) k = !(lb(b, j) * (1.0 - 0x1p-40) > ub[b]);
+        }
+        const unsigned bits = __ballot_sync(kAll, k);
+        if (lane == 0 && i0 + b < ob.count) {
+          unsigned* at = keep + (i0 + b) * kw + w;
+          if (keep_was) keep_was[(i0 + b) * kw + w] = *at;
+          *at = bits;
+        }
+      }
     }
   }
 }
@@ -390,30 +607,50 @@ cudaError_t check_bag_symbols(const void* loc, int ldt, const long long* off, lo
   return cudaGetLastError();
 }
 
-cudaError_t bag_moments(const ObjView& ob, double* mu, double* var, cudaStream_t st) {
-  if (ob.count <= 0) return cudaSuccess;
-  const long long blocks = (ob.count + 3) / 4;
-  k_bag_moments<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, st>>>(ob, mu, var);
+cudaError_t bag_prep(const ObjView& ob, const SolveCfg* range, int mmax, long long* mass,
+                     unsigned char* bad, int mstride, double* mu, double* var, cudaStream_t st) {
+  long long total = ob.count;
+  const int* oidx = nullptr;
+  const long long *lo = nullptr, *hi = nullptr;
+  long long obase = 0;
+  if (range) {
+    oidx = range->oidx;
+    lo = range->dev_lo;
+    hi = range->dev_hi;
+    obase = range->obase;
+    if (!lo && range->nobj >= 0) total = range->nobj;
+  }
+  if (total <= 0) return cudaSuccess;
+  const long long blocks = (total + 15) / 16;
+  k_bag_prep<<<(unsigned)(blocks < 4096 ? blocks : 4096), 128, 0, st>>>(
+      ob, oidx, lo, hi, obase, total, mmax, mass, bad, mstride, mu, var);
   note_launches(1);
   return cudaGetLastError();
 }
 
-cudaError_t cent_moments(const CentView& cv, double* mu, double* var, cudaStream_t st) {
+cudaError_t cent_moments(const CentView& cv, const CentMoments& cm, cudaStream_t st) {
   if (cv.K <= 0) return cudaSuccess;
   const long long blocks = (cv.K + 3) / 4;
-  k_cent_moments<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, st>>>(cv, mu, var);
+  k_cent_moments<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, st>>>(cv, cm.mu, cm.var,
+                                                                            cm.muT32, cm.cn, cm.vb);
   note_launches(1);
   return cudaGetLastError();
 }
 
 cudaError_t prune_keep(const ObjView& ob, long long seg_size, int K, long long KT, int d,
-                       const double* mu_o, const double* var_o, const double* mu_c,
-                       const double* var_c, unsigned* keep, int kw, cudaStream_t st) {
+                       const double* mu_o, const double* var_o, const CentMoments& cm,
+                       unsigned* keep, int kw, unsigned* keep_was, cudaStream_t st) {
   if (ob.count <= 0) return cudaSuccess;
   if (kw < (K + 31) / 32) return cudaErrorInvalidValue;
-  const long long blocks = (ob.count + 3) / 4;
-  k_prune_keep<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, st>>>(
-      ob, seg_size, K, KT, d, mu_o, var_o, mu_c, var_c, keep, kw);
+  // 4 objects a warp share the centroid loads once that still fills the GPU
+  auto go = [&](auto kern, int b) {
+    const long long blocks = (ob.count + 4 * b - 1) / (4 * b);
+    kern<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, st>>>(
+        ob, seg_size, K, KT, d, mu_o, var_o, cm.mu, cm.var, cm.muT32, cm.cn, cm.vb, keep, kw,
+        keep_was);
+  };
+  if (ob.count >= 16384) go(k_prune_keep<4>, 4);
+  else go(k_prune_keep<1>, 1);
   note_launches(1);
   return cudaGetLastError();
 }

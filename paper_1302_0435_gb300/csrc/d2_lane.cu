@@ -7,33 +7,6 @@
 namespace d2k {
 namespace {
 
-// Masses of the chunk's objects as the solver uses them (load_prefix), one
-// warp per object; obad marks the bags it rejects.
-__global__ void __launch_bounds__(128) k_lane_prep(ObjView ob, LaneArgs A, long long total_obj,
-                                                   int mmax, long long* omass, unsigned char* obad) {
-  __shared__ long long pre[4][64];
-  Grp<32> g;
-  const int wb = threadIdx.x >> 5;
-  long long first, cnt;
-  lane_chunk(A, total_obj, &first, &cnt);
-  for (long long t = (long long)blockIdx.x * 4 + wb; t < cnt; t += (long long)gridDim.x * 4) {
-    const long long i = A.oidx ? (long long)A.oidx[first + t] : A.obase + first + t;
-    const long long o0 = ob.off[i];
-    const long long mm = ob.off[i + 1] - o0;
-    bool ok = mm >= 1 && mm <= mmax;
-    if (ok) {
-      const int m = (int)mm;
-      ok = ob.wdt == 0 ? load_prefix<32>(g, static_cast<const double*>(ob.w) + o0, m, pre[wb])
-                       : load_prefix<32>(g, static_cast<const float*>(ob.w) + o0, m, pre[wb]);
-      if (ok)
-        for (int a = g.lane; a < m; a += 32)
-          omass[i * A.mstride + a] = pre[wb][a] - (a > 0 ? pre[wb][a - 1] : 0LL);
-      __syncwarp();
-    }
-    if (g.lane == 0) obad[i] = ok ? 0 : 1;
-  }
-}
-
 // The kept pairs of the chunk (bits of cfg.keep): a thread counts its
 // object's, a block takes its run of the list with one addition, so the list
 // is nearly in object order and an object's pairs are together, centroids
@@ -198,9 +171,14 @@ cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_siz
   X.err = d_err;
   cudaError_t e = cudaMemsetAsync(A.ctr, 0, 32, st);
   if (e != cudaSuccess) return e;
-  k_lane_prep<<<grid_for(total_obj, 4, 4 * cfg.sms * 4), 128, 0, st>>>(ob, A, total_obj, cfg.mmax,
-                                                                       omass, obad);
-  note_launches(1);
+  if (cfg.mass) {
+    A.omass = cfg.mass;
+    A.obad = cfg.bad;
+    A.mstride = cfg.mstride;
+  } else {
+    e = bag_prep(ob, &cfg, cfg.mmax, omass, obad, A.mstride, nullptr, nullptr, st);
+    if (e != cudaSuccess) return e;
+  }
   const bool tc = tw && tw->C && cfg.mmax <= 64;
   if (tc && cfg.dev_lo) return cudaErrorInvalidValue;  // its chunks are cut on the host
   long long per = ls.objects;

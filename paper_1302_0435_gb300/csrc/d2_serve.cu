@@ -82,6 +82,8 @@ struct Slot {
   double* d_mu = nullptr; size_t n_mu = 0;
   double* d_var = nullptr; size_t n_var = 0;
   unsigned* d_keep = nullptr; size_t n_keep = 0;
+  long long* d_mass = nullptr; size_t n_mass = 0;  // the request's masses
+  unsigned char* d_bad = nullptr; size_t n_bad = 0;
   int* d_err = nullptr;
   // pinned host
   unsigned char* h_in = nullptr; size_t n_in = 0;
@@ -128,8 +130,7 @@ struct d2_server {
   long long K = 0;
   bool lanes = false;  // the lane screen (no cold-start rule fixed by the caller)
   // means and spreads of the resident centroids (pruning; null: off)
-  double* d_cmu = nullptr;
-  double* d_cvar = nullptr;
+  d2k::CentMoments cm;
   size_t mem_budget = 0, mem_inflight = 0;
   std::vector<Slot> slots;
   std::deque<std::shared_ptr<Request>> queue;
@@ -146,6 +147,11 @@ struct d2_server {
   }
   long long scratch_ints(const std::shared_ptr<Request>& r) const {
     return d2k::assign_scratch_ints(r->count, K, sms, r->mmax, nmax, chunk_objects() * K);
+  }
+  void free_moments() {
+    cudaFree(cm.mu); cudaFree(cm.var); cudaFree(cm.muT32); cudaFree(cm.cn);
+    cudaFree(cm.vb);
+    cm = d2k::CentMoments();
   }
   bool launch(Slot& s, const std::shared_ptr<Request>& r);
   void run();
@@ -168,8 +174,10 @@ bool d2_server::launch(Slot& s, const std::shared_ptr<Request>& r) {
       !grow_dev(&s.d_lab, &s.n_lab, (size_t)N * 4 + 16) ||
       !grow_dev(&s.d_d2, &s.n_d2, (size_t)N * 8 + 16) ||
       !grow_dev(&s.d_cand, &s.n_cand, (size_t)scratch_ints(r) * 4 + 16) ||
-      (d_cmu && (!grow_dev(&s.d_mu, &s.n_mu, (size_t)N * r->dim * 8 + 16) ||
+      (cm.mu && (!grow_dev(&s.d_mu, &s.n_mu, (size_t)N * r->dim * 8 + 16) ||
                  !grow_dev(&s.d_var, &s.n_var, (size_t)N * 8 + 16) ||
+                 !grow_dev(&s.d_mass, &s.n_mass, (size_t)N * r->mmax * 8 + 16) ||
+                 !grow_dev(&s.d_bad, &s.n_bad, (size_t)N + 16) ||
                  !grow_dev(&s.d_keep, &s.n_keep, (size_t)N * ((K + 31) / 32) * 4 + 16))) ||
       !grow_host(&s.h_in, &s.n_in, b_in) ||
       !grow_host(&s.h_out, &s.n_out, b_out))
@@ -203,17 +211,21 @@ bool d2_server::launch(Slot& s, const std::shared_ptr<Request>& r) {
   cfg.lanes = lanes;
   cfg.max_pairs = chunk_objects() * K;
   d2k::FlowOut fo{nullptr, nullptr, 0};
-  if (d_cmu && cfg.mode == 1) {
+  if (cm.mu && cfg.mode == 1) {
     // skip the pairs that cannot be an object's argmin (d2k::prune_keep)
     const int kw = (int)((K + 31) / 32);
-    if (d2k::bag_moments(ob, s.d_mu, s.d_var, st) != cudaSuccess ||
-        d2k::prune_keep(ob, N, (int)K, K, ob.d, s.d_mu, s.d_var, d_cmu, d_cvar, s.d_keep, kw, st) !=
+    if (d2k::bag_prep(ob, nullptr, r->mmax, s.d_mass, s.d_bad, r->mmax, s.d_mu, s.d_var, st) !=
+            cudaSuccess ||
+        d2k::prune_keep(ob, N, (int)K, K, ob.d, s.d_mu, s.d_var, cm, s.d_keep, kw, nullptr, st) !=
             cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     cfg.keep = s.d_keep;
     cfg.keep_words = kw;
+    cfg.mass = s.d_mass;
+    cfg.bad = s.d_bad;
+    cfg.mstride = r->mmax;
   }
   // bounded chunks, bin by bin (largest trees first); one stream, so the
   // chunks of a request run in order and share its scratch
@@ -387,15 +399,15 @@ extern "C" int d2_server_create(d2_server** out, d2_ctx* ctx, int32_t nslots, in
   }
   if (d2k::ctx_prune(ctx) && sv->cv.A == 0) {
     // the resident centroids' means and spreads, once
-    if (cudaMalloc(&sv->d_cmu, (size_t)sv->K * sv->d * 8) != cudaSuccess ||
-        cudaMalloc(&sv->d_cvar, (size_t)sv->K * 8) != cudaSuccess ||
-        d2k::cent_moments(sv->cv, sv->d_cmu, sv->d_cvar, sv->slots[0].stream) != cudaSuccess ||
+    if (cudaMalloc(&sv->cm.mu, (size_t)sv->K * sv->d * 8) != cudaSuccess ||
+        cudaMalloc(&sv->cm.var, (size_t)sv->K * 8) != cudaSuccess ||
+        cudaMalloc(&sv->cm.muT32, (size_t)sv->K * sv->d * 4) != cudaSuccess ||
+        cudaMalloc(&sv->cm.cn, (size_t)sv->K * 4) != cudaSuccess ||
+        cudaMalloc(&sv->cm.vb, (size_t)sv->K * 8) != cudaSuccess ||
+        d2k::cent_moments(sv->cv, sv->cm, sv->slots[0].stream) != cudaSuccess ||
         cudaStreamSynchronize(sv->slots[0].stream) != cudaSuccess) {
       cudaGetLastError();
-      cudaFree(sv->d_cmu);
-      cudaFree(sv->d_cvar);
-      sv->d_cmu = nullptr;
-      sv->d_cvar = nullptr;
+      sv->free_moments();
     }
   }
   sv->worker = std::thread([sv] { sv->run(); });
@@ -524,13 +536,12 @@ extern "C" int d2_server_destroy(d2_server* sv) {
     cudaFree(s.d_loc); cudaFree(s.d_w); cudaFree(s.d_off); cudaFree(s.d_order); cudaFree(s.d_lab);
     cudaFree(s.d_d2);
     cudaFree(s.d_cand); cudaFree(s.d_err);
-    cudaFree(s.d_mu); cudaFree(s.d_var); cudaFree(s.d_keep);
+    cudaFree(s.d_mu); cudaFree(s.d_var); cudaFree(s.d_keep); cudaFree(s.d_mass); cudaFree(s.d_bad);
     if (s.h_in) cudaFreeHost(s.h_in);
     if (s.h_out) cudaFreeHost(s.h_out);
     if (s.h_err) cudaFreeHost(s.h_err);
   }
-  cudaFree(sv->d_cmu);
-  cudaFree(sv->d_cvar);
+  sv->free_moments();
   delete sv;
   return D2_OK;
 }

@@ -116,8 +116,8 @@ constexpr int kMaxStride = 127;
 // One block per centroid.  Members (objects assigned to it, increasing
 // index) are staged as many whole members at a time as fit kStageEntries
 // flow entries: each entry's centroid support r, object row and coefficient
-// omega_i * w go to shared memory, and one warp lists the entries of every
-// column r in entry order (a stable counting sort by r).  Then every (r, k)
+// omega_i * w go to shared memory, and the warps list the entries of every
+// column r in entry order.  Then every (r, k)
 // slot of the numerator sums, in entry order, the entries of its column
 // (coef * v^(a)_k) in FP64; the k == 0 slot also sums the denominator.  The
 // order of every sum is fixed, so results are deterministic.  Dynamic smem:
@@ -168,37 +168,60 @@ __global__ void k_accumulate(ObjView ob, const double* omega, FlowOut fo, const 
     }
     __syncthreads();
     const int ne = cm * stride;
-    if (threadIdx.x < 32) {
-      // counts per column, then starts, then a stable scatter in entry order
-      for (int r = lane; r <= n; r += 32) bend[r] = 0;
-      __syncwarp();
-      for (int base = 0; base < ne; base += 32) {
-        const int q = base + lane;
-        const int rr = q < ne ? e_r[q] : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, rr);
-        if (rr >= 0 && lane == __ffs(peers) - 1) bend[rr + 1] += __popc(peers);
-        __syncwarp();
+    // column lists in entry order: counts (any order), starts, then each warp
+    // collects its columns by ballots over the entries
+    for (int r = threadIdx.x; r <= n; r += blockDim.x) bend[r] = 0;
+    __syncthreads();
+    for (int q = threadIdx.x; q < ne; q += blockDim.x)
+      if (e_r[q] >= 0) atomicAdd(&bend[e_r[q] + 1], 1);
+    __syncthreads();
+    if (threadIdx.x < 32) {  // inclusive scan of up to 64 counts
+      const int v0 = lane < n ? bend[lane + 1] : 0, v1 = lane + 32 < n ? bend[lane + 33] : 0;
+      int x0 = v0, x1 = v1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u0 = __shfl_up_sync(0xffffffffu, x0, o), u1 = __shfl_up_sync(0xffffffffu, x1, o);
+        if (lane >= o) { x0 += u0; x1 += u1; }
       }
-      if (lane == 0)
-        for (int r = 0; r < n; ++r) bend[r + 1] += bend[r];
-      __syncwarp();
-      for (int base = 0; base < ne; base += 32) {
-        const int q = base + lane;
-        const int rr = q < ne ? e_r[q] : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, rr);
-        if (rr >= 0) blist[bend[rr] + __popc(peers & ((1u << lane) - 1u))] = q;
-        __syncwarp();
-        if (rr >= 0 && lane == __ffs(peers) - 1) bend[rr] += __popc(peers);
-        __syncwarp();
-      }
-      // column r now spans blist[(r ? bend[r-1] : 0) .. bend[r])
+      x1 += __shfl_sync(0xffffffffu, x0, 31);
+      if (lane < n) bend[lane + 1] = x0;
+      if (lane + 32 < n) bend[lane + 33] = x1;
     }
+    __syncthreads();
+    for (int r = threadIdx.x >> 5; r < n; r += blockDim.x >> 5) {
+      int at = bend[r];
+      const int end = bend[r + 1];
+      for (int base = 0; base < ne && at < end; base += 32) {
+        const int q = base + lane;
+        const bool in = q < ne && e_r[q] == r;
+        const unsigned b = __ballot_sync(0xffffffffu, in);
+        if (in) blist[at + __popc(b & ((1u << lane) - 1u))] = q;
+        at += __popc(b);
+      }
+    }
+    // column r spans blist[bend[r] .. bend[r + 1])
     __syncthreads();
     for (int t = threadIdx.x; t < slots; t += blockDim.x) {
       const int r = t / d, k = t - r * d;
       double sn = num[t], sd = (k == 0) ? den[r] : 0.0;
-      const int lo = r > 0 ? bend[r - 1] : 0, hi = bend[r];
-      for (int x = lo; x < hi; ++x) {
+      const int lo = bend[r], hi = bend[r + 1];
+      int x = lo;
+      // the loads of 8 entries go out together, their terms are added in order
+      for (; x + 8 <= hi; x += 8) {
+        double cf[8], v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int q = blist[x + u];
+          cf[u] = e_coef[q];
+          v[u] = ldloc(ob.loc, ob.ldt, e_row[q] * d + k);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          sn = fma(cf[u], v[u], sn);
+          if (k == 0) sd += cf[u];
+        }
+      }
+      for (; x < hi; ++x) {
         const int q = blist[x];
         const double cf = e_coef[q];
         sn = fma(cf, ldloc(ob.loc, ob.ldt, e_row[q] * d + k), sn);
