@@ -46,7 +46,7 @@ enum Slot {
   // d2_mallows_all
   kAllLab, kAllD2, kAllPair,
   // pruning of pairs that cannot be the argmin
-  kPrMuO, kPrVarO, kPrMuC, kPrVarC, kPrKeep, kPrMuT, kPrCn, kPrVb, kPrMass, kPrBad,
+  kPrMuO, kPrVarO, kPrMuC, kPrVarC, kPrKeep, kPrMuT, kPrCn, kPrVb, kPrMass, kPrBad, kPrKeepWas, kPrRows, kPrAxes,
   kSlots
 };
 
@@ -537,12 +537,27 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
     cm.vb = static_cast<float2*>(grow(c, kPrVb, (size_t)cv.K * 8, &rc));
     unsigned* keep = static_cast<unsigned*>(grow(c, kPrKeep, (size_t)v.count * kw * 4, &rc));
     if (rc != D2_OK) return rc;
+    // a level's rounds keep the bits of the round before as well: the pairs
+    // whose bases that round saved
+    unsigned* was = nullptr;
+    if (ws && base.lanes)
+      was = static_cast<unsigned*>(grow(c, kPrKeepWas, (size_t)v.count * kw * 4, &rc));
+    if (rc != D2_OK) return rc;
     CK(d2k::cent_moments(cv, cm, c->stream));
     CK(d2k::prune_keep(v, seg, K, cv.K, v.d, static_cast<const double*>(c->slot[kPrMuO].p),
-                       static_cast<const double*>(c->slot[kPrVarO].p), cm, keep, kw, nullptr,
+                       static_cast<const double*>(c->slot[kPrVarO].p), cm, keep, kw, was,
                        c->stream));
     base.keep = keep;
     base.keep_words = kw;
+    base.keep_was = was;
+  }
+  if (ws && base.lanes && !ws->warm && nmax <= 16) {
+    // the cold round of a level starts small trees from the ranked staircase
+    int rc = D2_OK;
+    base.rows = static_cast<unsigned char*>(grow(c, kPrRows, (size_t)v.count * mmax, &rc));
+    base.axes = static_cast<float*>(grow(c, kPrAxes, (size_t)v.count * 2 * v.d * 4, &rc));
+    if (rc != D2_OK) return rc;
+    CK(d2k::lane_axes(v, base, c->stream));
   }
   if (!bins.binned) {
     CK(d2k::assign(v, cv, seg, K, base, om, lab, d2o, terms, fo, cand, c->d_err, c->stream, ws, tw));
@@ -550,7 +565,7 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
   }
   // the lane screen has one launch shape per bound; the warp-per-pair screen
   // is tuned
-  const bool lanes = base.lanes && mode == 1 && !ws;
+  const bool lanes = base.lanes && mode == 1;
   const bool tuning = c->cfg.group_lanes == 0 && mode == 1 && v.count >= 8192 && !lanes;
   int cut[8];
   const int ncut = size_cuts(lanes, mmax, nmax, cut);
@@ -558,6 +573,11 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
     const int lo = b > 0 ? cut[b - 1] : 0;  // support counts lo + 1 .. cut[b]
     SolveCfg cfg = base;
     cfg.mmax = cut[b];
+    if (lanes && !tw) {
+      cfg.first = b == ncut - 1;
+      cfg.last = b == 0;
+      cfg.mall = mmax;
+    }
     const auto key = std::make_tuple((cfg.mmax + nmax + 31) / 32 - 1, (long long)K, cfg.mmax, nmax,
                                      v.d, mode + (cfg.certify ? 2 : 0));
     auto it = c->tuned.find(key);
@@ -913,10 +933,10 @@ int segment_impl(d2_ctx* c, const ObjView& v, int mmax, const double* om, long l
 }
 
 // Bin only when the batch is large and its launches then differ.
-bool want_bins(const d2_ctx* c, const SolveCfg& cfg, long long count, int mmax, bool warm) {
+bool want_bins(const d2_ctx* c, const SolveCfg& cfg, long long count, int mmax) {
   int cut[8];
   return count >= 4096 &&
-         size_cuts(cfg.lanes && cfg.mode == 1 && !warm, mmax, std::max(c->nmax, 1), cut) > 1;
+         size_cuts(cfg.lanes && cfg.mode == 1, mmax, std::max(c->nmax, 1), cut) > 1;
 }
 
 }  // namespace
@@ -1288,7 +1308,7 @@ int assign_impl(d2_ctx* c, const d2_bags* objs, const double* omega, int32_t* la
   if ((rc = check_bag_symbols(c, v))) return rc;
   const int mode = mode_for(c, objs->loc_dtype);
   Bins bins;
-  if (want_bins(c, solve_cfg(c, mode, mmax), N, mmax, false) && (rc = make_bins(c, v, &bins)))
+  if (want_bins(c, solve_cfg(c, mode, mmax), N, mmax) && (rc = make_bins(c, v, &bins)))
     return rc;
   d2k::TcWork tw;
   const bool tc = tc_wanted(c, objs, v, mode);
@@ -1844,18 +1864,30 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     const size_t flow_bytes = (size_t)npairs * ns * 8;
     // (not with Alg. 1 updates: the weights, so every pair's supplies, change each round)
     const size_t budget = (cfg.mode == 1 && iters > 1 && !alg1) ? warm_budget_bytes(c) : 0;
-    // (a certify-all level keeps full bases or none: its screening kernel
-    // carries no flow recomputation)
-    const bool flows = meta_bytes + flow_bytes <= budget;
-    if (flows || (meta_bytes <= budget && !cfg.certify)) {
-      unsigned char* meta = static_cast<unsigned char*>(grow(c, kWarmMeta, meta_bytes, &rc));
-      long long* wf = flows ? static_cast<long long*>(grow(c, kWarmFlow, flow_bytes, &rc)) : nullptr;
-      if (rc != D2_OK) return rc;
-      ws = d2k::WarmStore{meta, meta + (size_t)npairs * ns, meta + (size_t)npairs * ns * 2, wf, ns,
-                          0};
+    if (cfg.lanes) {
+      // the lane screen keeps a basis as its parents, a byte a node, and
+      // rebuilds flows and subtree sets as it loads them
+      const size_t bytes = (size_t)npairs * ns;
+      if (bytes <= budget) {
+        unsigned char* par = static_cast<unsigned char*>(grow(c, kWarmMeta, bytes, &rc));
+        if (rc != D2_OK) return rc;
+        ws = d2k::WarmStore{par, nullptr, nullptr, nullptr, ns, 0};
+      }
+    } else {
+      // (a certify-all level keeps full bases or none: its screening kernel
+      // carries no flow recomputation)
+      const bool flows = meta_bytes + flow_bytes <= budget;
+      if (flows || (meta_bytes <= budget && !cfg.certify)) {
+        unsigned char* meta = static_cast<unsigned char*>(grow(c, kWarmMeta, meta_bytes, &rc));
+        long long* wf =
+            flows ? static_cast<long long*>(grow(c, kWarmFlow, flow_bytes, &rc)) : nullptr;
+        if (rc != D2_OK) return rc;
+        ws = d2k::WarmStore{meta, meta + (size_t)npairs * ns, meta + (size_t)npairs * ns * 2, wf, ns,
+                            0};
+      }
     }
     Bins bins;
-    if (want_bins(c, cfg, n_l, cur_mmax, ws.par8 != nullptr) && (rc = make_bins(c, cur, &bins)))
+    if (want_bins(c, cfg, n_l, cur_mmax) && (rc = make_bins(c, cur, &bins)))
       return rc;
     // this level's bags (masses, pruning moments), once for all its rounds
     if (cfg.mode == 1 && (rc = prep_bags(c, cur, cur_mmax, prunes(c, cfg, cv)))) return rc;

@@ -49,6 +49,7 @@ struct FlowOut {
   long long pstride = 0;
 };
 
+// (pos8 null: parents only, as the lane screen keeps them.)
 // Saved optimal bases of every (object, centroid) pair of an assign call,
 // pair t = i*K + j, node y at [t*ns + y]: parent / position / size bytes and
 // int64 flow (flow == nullptr: trees only, the flows recomputed from the
@@ -126,6 +127,11 @@ struct SolveCfg {
   // run and the merged lists are in place
   bool lanes = false;
   bool screened = false;
+  // launches over parts of one batch (its size cuts): the objects left to
+  // k_exact are counted from the first on and solved after the last, whose
+  // rows go up to mall (0: mmax)
+  bool first = true, last = true;
+  int mall = 0;
   // object masses made ahead (bag_prep; null: the screen makes its own)
   const long long* mass = nullptr;
   const unsigned char* bad = nullptr;
@@ -151,6 +157,11 @@ struct SolveCfg {
   // screens that pick argmin candidates (not certify, not pair_out).
   const unsigned* keep = nullptr;
   int keep_words = 0;
+  // a level's rounds (lane screen): the bits of the round before, and the
+  // scratch of its cold start's orders (lane_axes)
+  const unsigned* keep_was = nullptr;
+  unsigned char* rows = nullptr;
+  float* axes = nullptr;
   TileView tile;              // precomputed FP32 tiles of the screen (optional)
   // mallows_pairs with mode 1: room (pair_tree_bytes) for the FP32 bases
   // handed from the FP32 launch to the FP64 launch; null: one fused launch
@@ -235,8 +246,15 @@ struct LaneArgs {
   const unsigned char* obad;  // [count] bags the solver rejects
   int mstride;
   PairRec* rec;               // [pairs of the chunk]
-  unsigned char* tree;        // saved bases of the chunk's pairs (parents)
+  unsigned char* tree;        // saved bases (parents) of the chunk's pairs, or
+  bool by_pair;               // of every pair of the batch (a level's rounds)
   int tstride;                // bytes a basis
+  // a level's rounds: bases were saved by the last round (of the pairs kept in
+  // it); the cold start's row ranks [count][mstride], means and directions
+  bool warm;
+  const unsigned* keep_was;
+  const unsigned char* rows;
+  const float* axes;
   int nb;                     // column blocks of 4 (set by the launch)
   int warp_bytes;             // shared memory of a warp (set by the launch)
 };
@@ -269,7 +287,9 @@ inline LaneScratch lane_scratch(long long count, long long K, int mmax, int nmax
   const long long n = count > 0 ? count : 1, k = K > 0 ? K : 1;
   s.objects = std::max<long long>(1, std::min(n, max_pairs / k));
   const size_t pairs = (size_t)s.objects * (size_t)k;
-  size_t b = 256;  // work queue and list length
+  size_t b = 256;  // work queue, list length, fallback count
+  s.fb = b;        // (in the same place for every bound mmax of a batch)
+  b += up((size_t)n * 4);
   s.mass = b;
   b += up((size_t)n * (size_t)mmax * 8);
   s.bad = b;
@@ -283,8 +303,6 @@ inline LaneScratch lane_scratch(long long count, long long K, int mmax, int nmax
   s.tstride = mmax + nmax;
   s.tree = b;
   b += up(pairs * (size_t)s.tstride);
-  s.fb = b;
-  b += up((size_t)n * 4);
   s.bytes = b;
   return s;
 }
@@ -296,7 +314,9 @@ size_t lane_scratch_offset(long long count);
 // to k_exact are X's fb list, *fb_hi of them (lane_fallback).
 cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_size, int K,
                         const SolveCfg& cfg, int* cand, int* d_err, cudaStream_t st,
-                        const TcWork* tw, ExactOut X);
+                        const TcWork* tw, const WarmStore* ws, ExactOut X);
+// Row ranks, means and principal directions of the bags (SolveCfg::rows, axes).
+cudaError_t lane_axes(const ObjView& ob, const SolveCfg& cfg, cudaStream_t st);
 // Launch settings of k_exact over the fallback list of lane_screen.
 void lane_fallback(const ObjView& ob, int K, int* cand, SolveCfg* cfg);
 #define D2_LANE_DECL(U)                                                                          \

@@ -551,7 +551,7 @@ cudaError_t assign(const ObjView& ob, const CentView& cv, long long seg_size, in
                    const WarmStore* ws, const TcWork* tw) {
   if (ob.count <= 0) return cudaSuccess;
   SolveCfg cfg = cfg0;
-  if (cfg.lanes && cfg.mode == 1 && cand && !ws) {
+  if (cfg.lanes && cfg.mode == 1 && cand && (!ws || !ws->pos8)) {
     ExactOut X;
     if (cfg.lane_exact && !cfg.screen_only) {
       X.omega = omega;
@@ -560,10 +560,14 @@ cudaError_t assign(const ObjView& ob, const CentView& cv, long long seg_size, in
       X.eps_terms = eps_terms;
       X.fo = fo;
     }
-    const cudaError_t e = lane_screen(ob, cv, seg_size, K, cfg, cand, d_err, st, tw, X);
+    const cudaError_t e = lane_screen(ob, cv, seg_size, K, cfg, cand, d_err, st, tw, ws, X);
     if (e != cudaSuccess || cfg.screen_only) return e;
     cfg.screened = true;
-    if (X.labels) lane_fallback(ob, K, cand, &cfg);  // the few objects k_exact still solves
+    if (X.labels) {  // the few objects k_exact still solves
+      if (!cfg.last) return cudaSuccess;
+      if (cfg.mall > cfg.mmax) cfg.mmax = cfg.mall;
+      lane_fallback(ob, K, cand, &cfg);
+    }
   }
   int G, NP;
   if (!pick_shape(cfg.mmax, cfg.nmax, &G, &NP)) return cudaErrorInvalidValue;

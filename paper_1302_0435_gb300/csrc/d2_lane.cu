@@ -7,6 +7,48 @@
 namespace d2k {
 namespace {
 
+// Ranks of the rows along each object's principal direction, one warp per
+// object: the orders of the ranked staircase (order_rows in d2_solve.cuh).
+__global__ void __launch_bounds__(128) k_lane_axes(ObjView ob, int mmax, const long long* mass,
+                                                   const unsigned char* bad, int mstride,
+                                                   unsigned char* rows, float* axes) {
+  __shared__ long long P[4][64], Pr[4][64];
+  __shared__ int rank[4][64], id[4][64];
+  __shared__ float mu[4][256], dir[4][256], proj[4][64];
+  Grp<32> g;
+  const int w = threadIdx.x >> 5;
+  const int d = ob.d;
+  for (long long i = (long long)blockIdx.x * 4 + w; i < ob.count; i += (long long)gridDim.x * 4) {
+    if (bad[i]) continue;
+    const long long o0 = ob.off[i];
+    const int m = (int)(ob.off[i + 1] - o0);
+    long long carry = 0;
+    for (int b = 0; b < m; b += 32) {  // inclusive prefix of the masses
+      const int a = b + g.lane;
+      long long v = a < m ? mass[i * mstride + a] : 0LL;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, v, o);
+        if (g.lane >= o) v += u;
+      }
+      v += carry;
+      if (a < m) P[w][a] = v;
+      carry = __shfl_sync(0xffffffffu, v, 31);
+    }
+    __syncwarp();
+    PairMem<float> s{};
+    s.P = P[w]; s.Pr = Pr[w]; s.rrank = rank[w]; s.rid = id[w];
+    s.mu = mu[w]; s.dir = dir[w]; s.proj = proj[w];
+    order_rows<32>(g, s, ob, o0, m, d);
+    for (int a = g.lane; a < m; a += 32) rows[i * mstride + a] = (unsigned char)id[w][a];
+    for (int k = g.lane; k < d; k += 32) {
+      axes[i * 2 * d + k] = mu[w][k];
+      axes[i * 2 * d + d + k] = dir[w][k];
+    }
+    __syncwarp();
+  }
+}
+
 // The kept pairs of the chunk (bits of cfg.keep): a thread counts its
 // object's, a block takes its run of the list with one addition, so the list
 // is nearly in object order and an object's pairs are together, centroids
@@ -140,7 +182,7 @@ static cudaError_t lane_dispatch(const ObjView& ob, const CentView& cv, long lon
 // at cand + 4, and with X.labels their exact pass.
 cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_size, int K,
                         const SolveCfg& cfg, int* cand, int* d_err, cudaStream_t st,
-                        const TcWork* tw, ExactOut X) {
+                        const TcWork* tw, const WarmStore* ws, ExactOut X) {
   const long long total_obj = cfg.dev_lo ? ob.count : (cfg.nobj >= 0 ? cfg.nobj : ob.count);
   if (total_obj <= 0) return cudaSuccess;
   const LaneScratch ls = lane_scratch(ob.count, K, cfg.mmax, cfg.nmax, cfg.max_pairs);
@@ -158,6 +200,15 @@ cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_siz
   A.rec = reinterpret_cast<PairRec*>(mem + ls.rec);
   A.tree = X.labels ? mem + ls.tree : nullptr;
   A.tstride = ls.tstride;
+  if (ws) {
+    A.by_pair = true;
+    A.tree = ws->par8;
+    A.tstride = ws->ns;
+    A.warm = ws->warm != 0;
+    A.keep_was = cfg.keep ? cfg.keep_was : nullptr;
+    A.rows = cfg.rows;
+    A.axes = cfg.axes;
+  }
   A.list = cfg.keep ? list : nullptr;
   A.oidx = cfg.oidx;
   A.obase = cfg.obase;
@@ -169,7 +220,7 @@ cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_siz
   X.ostart = ostart;
   X.fb = reinterpret_cast<int*>(mem + ls.fb);
   X.err = d_err;
-  cudaError_t e = cudaMemsetAsync(A.ctr, 0, 32, st);
+  cudaError_t e = cudaMemsetAsync(A.ctr, 0, cfg.first ? 32 : 16, st);
   if (e != cudaSuccess) return e;
   if (cfg.mass) {
     A.omass = cfg.mass;
@@ -217,6 +268,14 @@ cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_siz
       if (e != cudaSuccess) return e;
     }
   }
+  return cudaGetLastError();
+}
+
+cudaError_t lane_axes(const ObjView& ob, const SolveCfg& cfg, cudaStream_t st) {
+  if (ob.count <= 0) return cudaSuccess;
+  k_lane_axes<<<grid_for(ob.count, 4, 16 * cfg.sms), 128, 0, st>>>(
+      ob, cfg.mmax, cfg.mass, cfg.bad, cfg.mstride, cfg.rows, cfg.axes);
+  note_launches(1);
   return cudaGetLastError();
 }
 

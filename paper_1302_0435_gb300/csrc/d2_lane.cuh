@@ -90,6 +90,11 @@ struct Mask {
     for (int i = 0; i < MW; ++i)
       if ((e >> 5) == i) w[i] |= 1u << (e & 31);
   }
+  __device__ __forceinline__ void drop(int e) {
+#pragma unroll
+    for (int i = 0; i < MW; ++i)
+      if ((e >> 5) == i) w[i] &= ~(1u << (e & 31));
+  }
   __device__ __forceinline__ Mask minus(const Mask& o) const {
     Mask r;
 #pragma unroll
@@ -188,6 +193,12 @@ struct Lane {
       d.w[0] = v.x; d.w[1] = v.y; d.w[2] = v.z; d.w[3] = v.w;
     }
     return d;
+  }
+  __device__ __forceinline__ void putD(int y, const Mask<MW>& d) const {
+    if constexpr (MW == 1) *reinterpret_cast<unsigned*>(rec(y) + 8) = d.w[0];
+    else if constexpr (MW == 2) *reinterpret_cast<uint2*>(rec(y) + 8) = make_uint2(d.w[0], d.w[1]);
+    else *reinterpret_cast<uint4*>(sp + Sh::kD4 + y * PS) =
+        make_uint4(d.w[0], d.w[1], d.w[2], d.w[3]);
   }
   // the whole record
   __device__ __forceinline__ void load(int y, long long& f, Mask<MW>& d, unsigned& p) const {
@@ -355,7 +366,8 @@ struct Lane {
     }
     // the last line takes the rest
     const bool row_root = nr == 1;
-    root = row_root ? __ffsll((long long)ra) - 1 : MP + __ffsll((long long)ca) - 1;
+    if (live)
+      root = row_root ? __ffsll((long long)ra) - 1 : MP + __ffsll((long long)ca) - 1;
     Mask<MW> d;
     d.clear();
 #pragma unroll 1
@@ -373,6 +385,131 @@ struct Lane {
 #pragma unroll
     for (int i = 0; i < MW; ++i) d.w[i] = oru(d.w[i]);
     if (live && g == 0) store(root, 0, getD(root).plus(d), 0xffu);
+    __syncwarp();
+  }
+
+  // Flows (and with MASKS the subtree sets) of the tree in par: the edge above
+  // a node carries the net mass of its subtree, rows positive and columns
+  // negative, summed by walking every node's mass up to the root.  On entry
+  // flow holds the masses and D the singletons; exact integers, so the flows
+  // are those the tree was saved with.  Returns whether the tree is
+  // inconsistent or a flow negative.
+  template <bool MASKS>
+  __device__ __forceinline__ bool from_parents() {
+    bool bad = false;
+    long long b[NPL];
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) b[k] = k < KR ? flowk(k) : -flowk(k);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < NPL; ++k)
+      if (live) flowk(k) = 0;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      if (live && nodek(k)) {
+        const int y = node(k);
+        int x = y;
+        for (int it = 0; it < NS && x != root; ++it) {
+          atomicAdd(reinterpret_cast<unsigned long long*>(&flow(x)), (unsigned long long)b[k]);
+          if (MASKS && x != y) or_mask(x, y);
+          const unsigned p = par(x);
+          if (p >= (unsigned)NS || is_row(x) == is_row((int)p)) { bad = true; break; }
+          x = (int)p;
+        }
+        if (x != root) bad = true;  // no way to the root
+        else if (MASKS && y != root) or_mask(root, y);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      if (live) {
+        if (k >= KR) flowk(k) = -flowk(k);
+        bad |= nodek(k) && flowk(k) < 0;
+      }
+    }
+    return oru(bad ? 1u : 0u) != 0u;
+  }
+  __device__ __forceinline__ void or_mask(int x, int y) const {
+    char* at = MW == 4 ? sp + Sh::kD4 + x * PS : rec(x) + 8;
+    atomicOr(reinterpret_cast<unsigned*>(at) + (y >> 5), 1u << (y & 31));
+  }
+
+  // ---- start: northwest staircase ----
+  // Rows and columns in the orders of the code section (row of rank q at q,
+  // column of rank q at MP + q): down when the row is used up first (ties
+  // down), the new line hangs from the other kind's current one.  A node
+  // carries everything after it once a node hangs from it, else itself.
+  // flow holds the masses, D the singletons.
+  __device__ __forceinline__ void start_staircase() {
+    int iq = 0, jq = 0;
+    int a = u8at<Sh::kCode>(0), r = MP + u8at<Sh::kCode>(MP);
+    Mask<MW> rest;  // nodes not touched before `last`
+#pragma unroll
+    for (int w = 0; w < MW; ++w) rest.w[w] = 0u;
+    if (live) {
+      for (int y = 0; y < m; ++y) rest.set(y);
+      for (int y = 0; y < n; ++y) rest.set(MP + y);
+    }
+    long long p = 0, q = 0;
+    if (live) {
+      p = flow(a);
+      q = flow(r);
+      root = a;
+    }
+    __syncwarp();
+    // the root, then column r hanging from it
+    const Mask<MW> all = rest;
+    int last = r;
+    if (live) {
+      rest.drop(a);
+      const long long f = p < q ? p : q;
+      if (g == 0) {
+        store(a, 0, all, 0xffu);
+        Mask<MW> one;
+        one.clear();
+        one.set(r);
+        store(r, f, one, (unsigned)a);
+      }
+      p -= f;
+      q -= f;
+    }
+    for (int s = 2;; ++s) {
+      const bool act = live && s < N;
+      if (!__any_sync(kAll, act)) break;
+      int y = 0, z = 0;
+      long long f = 0;
+      if (act) {
+        const bool down = iq < m - 1 && (p <= q || jq == n - 1);
+        z = down ? r : a;  // the new node hangs from z
+        y = down ? (int)u8at<Sh::kCode>(++iq) : MP + (int)u8at<Sh::kCode>(MP + ++jq);
+        const long long w = flow(y);
+        if (down) {
+          f = w < q ? w : q;
+          p = w - f;
+          q -= f;
+          a = y;
+        } else {
+          f = p < w ? p : w;
+          q = w - f;
+          p -= f;
+          r = y;
+        }
+      }
+      __syncwarp();
+      if (act) {
+        if (g == 0) {
+          if (z == last) putD(last, rest);  // `last` and what follows it
+          Mask<MW> one;
+          one.clear();
+          one.set(y);
+          store(y, f, one, (unsigned)z);
+        }
+        rest.drop(last);
+        last = y;
+      }
+    }
     __syncwarp();
   }
 
@@ -1116,7 +1253,57 @@ __device__ __forceinline__ void lane_chunk(const LaneArgs& A, long long total, l
   *cnt = c < 0 ? 0 : (c < A.cap ? c : A.cap);
 }
 
-template <class Sh, bool CERT>
+// The staircase's orders into the code section: the rows' and columns' ranks
+// along the object's principal direction (order_rows wrote the rows, the mean
+// and the direction; the columns as order_cols), or their own order.
+template <class Sh>
+__device__ __forceinline__ void lane_order(Lane<Sh>& P, const LaneArgs& A, bool ranked, long long i,
+                                           const float* y32, int d) {
+  constexpr int NPL = Sh::NPL, KR = Sh::KR, MP = Sh::MP;
+  if (ranked) {
+    const float* mu = A.axes + i * 2 * d;
+    const float* dir = mu + d;
+#pragma unroll
+    for (int k = KR; k < NPL; ++k) {
+      if (P.live && P.nodek(k)) {
+        const float* y = y32 + (P.node(k) - MP) * d;
+        float dot = 0.f;
+        for (int t = 0; t < d; ++t) dot = fmaf(__ldg(y + t) - __ldg(mu + t), __ldg(dir + t), dot);
+        P.potk(k) = dot;
+      }
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < NPL; ++k) {
+    if (P.live && P.nodek(k)) {
+      const int y = P.node(k);
+      if (!ranked) {
+        P.template u8own<Sh::kCode>(k) = (unsigned char)(k < KR ? y : y - MP);
+      } else if (k < KR) {
+        P.template u8own<Sh::kCode>(k) = A.rows[i * A.mstride + y];
+      } else {
+        const int r = y - MP;
+        const float v = P.potk(k);
+        int rank = 0;
+        for (int b = 0; b < P.n; ++b) {
+          const float u = P.pot(MP + b);
+          rank += (u < v || (u == v && b < r)) ? 1 : 0;
+        }
+        P.template u8at<Sh::kCode>(MP + rank) = (unsigned char)r;
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// WARM: a level's rounds.  Every pair's basis (its parents) is kept in A.tree
+// by pair (i K + j), and a round starts from the one its last round saved, if
+// the pair was solved then (A.warm, A.keep_was); trees of at most 32 nodes
+// start cold from the ranked staircase, and in a later round from the plain
+// one, as the warp-per-pair screen does, so that a level's trajectory, which
+// depends on the basis where a centroid's supports coincide, stays the same.
+template <class Sh, bool CERT, bool WARM>
 __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     k_lane_screen(ObjView ob, CentView cv, long long seg_size, int K, SolveCfg cfg, LaneArgs A,
                   long long total_obj) {
@@ -1197,15 +1384,54 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     }
     float4 vm;
     const float cmax = lane_tile<Sh>(P, ob, o0, cv, c0, tile_g, cfg.tile.ldc, vm);
-    P.start_rows(vm);
+    bool wbad = false;  // a saved basis that is not a feasible tree
+    if constexpr (WARM) {
+      const bool lv = P.live;
+      const bool fresh = !A.warm || (A.keep_was &&
+                                     !((A.keep_was[i * cfg.keep_words + (j >> 5)] >> (j & 31)) & 1u));
+      const unsigned char* tr = A.tree + (unsigned long long)(i * (long long)K + j) * A.tstride;
+      P.live = lv && !fresh;
+      int root = INT_MAX;
+#pragma unroll
+      for (int k = 0; k < NPL; ++k) {
+        if (P.live && P.nodek(k)) {
+          const int y = P.node(k);
+          unsigned p = tr[k < Sh::KR ? y : y - Sh::MP + P.m];
+          if (p == 0xffu) root = min(root, y);
+          else if (p >= (unsigned)P.m) p = p - P.m + Sh::MP;
+          P.put_par(y, p);
+        }
+      }
+#pragma unroll
+      for (int o = Sh::G / 2; o > 0; o >>= 1)
+        root = min(root, __shfl_xor_sync(kAll, root, o * PW));
+      if (P.live) P.root = root == INT_MAX ? 0 : root;
+      __syncwarp();
+      if (__any_sync(kAll, P.live)) wbad = P.template from_parents<true>();
+      P.live = lv && fresh;
+      if (__any_sync(kAll, P.live)) {
+        if constexpr (Sh::MW == 1) {
+          lane_order<Sh>(P, A, !A.warm, i, cv.loc32 + c0 * cv.d, cv.d);
+          P.start_staircase();
+        } else {
+          P.start_rows(vm);
+        }
+      }
+      P.live = lv;
+      __syncwarp();
+    } else {
+      P.start_rows(vm);
+    }
     int piv = 0;
     int st = P.run(cfg.budget * P.N, tol32(cmax), &piv);
+    if (WARM && wbad) st = kStInvalid;
     if (P.live && P.g == 0) {
       ++n_scr;
       p_scr += piv;
     }
     if (A.tree && P.live) {  // the basis, for the exact pass (parents, compact node numbers)
-      unsigned char* tr = A.tree + q * (unsigned)A.tstride;
+      unsigned char* tr = A.tree + (WARM ? (unsigned long long)(i * (long long)K + j) : q) *
+                                       (unsigned long long)A.tstride;
 #pragma unroll
       for (int k = 0; k < NPL; ++k) {
         if (P.nodek(k)) {
@@ -1289,52 +1515,24 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
 // k_exact (no FP64 reduced cost below -2^-43 c_max) with the FP32 tile as its
 // filter: a cell whose FP32 reduced cost clears the rounding bound E of
 // lane_certify has a non-negative FP64 one, the few others are priced in FP64.
-// Returns false when the tree is inconsistent or not optimal (the object then
-// goes to k_exact).  `value`: only the flows are wanted (certified pairs).
+// Returns 0 if the basis is optimal, 1 with the most negative cell (key, dE)
+// if not, 2 for an inconsistent tree or a value that is not finite.  `value`
+// false: only the flows are wanted (certified pairs).
 template <class Sh>
-__device__ __forceinline__ bool lane_verify(Lane<Sh>& P, bool go, bool value, char* pot64,
-                                            const ObjView& ob, long long o0, const CentView& cv,
-                                            long long c0, double* D64) {
-  constexpr int NPL = Sh::NPL, MP = Sh::MP, NS = Sh::NS, PS = Sh::PS;
+__device__ __forceinline__ int lane_verify(Lane<Sh>& P, bool go, bool value, char* pot64,
+                                           const ObjView& ob, long long o0, const CentView& cv,
+                                           long long c0, double* D64, int* ekey, float* edE) {
+  constexpr int NPL = Sh::NPL, MP = Sh::MP, PS = Sh::PS;
   constexpr unsigned kAll = 0xffffffffu;
   P.live = go;
   auto u64 = [&](int y) -> double& {
     return *reinterpret_cast<double*>(pot64 + (y >> 1) * PS + (y & 1) * 8);
   };
-  // flows: the edge above a node carries the net mass of its subtree, summed
-  // by walking every node's mass up to the root (exact integers)
-  bool bad = false;
-  long long b[NPL];
-#pragma unroll
-  for (int k = 0; k < NPL; ++k) {
-    b[k] = P.flowk(k);
-    if (k >= Sh::KR) b[k] = -b[k];
-  }
-  __syncwarp();
-#pragma unroll
-  for (int k = 0; k < NPL; ++k) P.flowk(k) = 0;
-  __syncwarp();
-#pragma unroll
-  for (int k = 0; k < NPL; ++k) {
-    if (go && P.nodek(k)) {
-      int x = P.node(k);
-      for (int it = 0; it < NS && x != P.root; ++it) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&P.flow(x)), (unsigned long long)b[k]);
-        const unsigned p = P.par(x);
-        if (p >= (unsigned)NS || (x < MP) == (p < (unsigned)MP)) { bad = true; break; }
-        x = (int)p;
-      }
-      if (x != P.root) bad = true;  // no way to the root
-    }
-  }
-  __syncwarp();
-#pragma unroll
-  for (int k = Sh::KR; k < NPL; ++k) P.flowk(k) = -P.flowk(k);
-#pragma unroll
-  for (int k = 0; k < NPL; ++k) bad |= go && P.nodek(k) && P.flowk(k) < 0;
-  bad = Lane<Sh>::oru(bad ? 1u : 0u) != 0u;
+  const bool bad = P.template from_parents<false>();
   const bool full = go && value && !bad;
-  if (!__any_sync(kAll, full)) return go && !bad;
+  if (!__any_sync(kAll, full)) return go && bad ? 2 : 0;
+  double worst = 0.0;  // most negative reduced cost below -tol
+  int wkey = INT_MAX;
   P.live = full;
   float4 vm;
   const float cmax = lane_tile<Sh>(P, ob, o0, cv, c0, nullptr, 0, vm);
@@ -1393,8 +1591,13 @@ __device__ __forceinline__ bool lane_verify(Lane<Sh>& P, bool go, bool value, ch
       for (int t = 0; t < 4; ++t) flag |= !(cc[t] - u - vv[t] >= E) ? 1u << t : 0u;
       for (; flag; flag &= flag - 1) {
         const int r = 4 * P.gl + __ffs((int)flag) - 1;
-        if (a < P.m && r < P.n)
-          fail |= !(cost64_cell(ob, o0, cv, c0, a, r) - u64(a) - u64(MP + r) >= -tol);
+        if (a < P.m && r < P.n) {
+          const double dd = cost64_cell(ob, o0, cv, c0, a, r) - u64(a) - u64(MP + r);
+          if (!(dd >= -tol)) {
+            fail |= isnan(dd);
+            if (dd < worst) { worst = dd; wkey = (a << 8) | r; }
+          }
+        }
       }
     }
   }
@@ -1413,12 +1616,23 @@ __device__ __forceinline__ bool lane_verify(Lane<Sh>& P, bool go, bool value, ch
   if (full) *D64 = D;
   fail |= full && !isfinite(D);
   fail = Lane<Sh>::oru(fail ? 1u : 0u) != 0u;
-  return go && !bad && !(full && fail);
+#pragma unroll
+  for (int o = Sh::G / 2; o > 0; o >>= 1) {
+    const double od = __shfl_xor_sync(kAll, worst, o * Sh::PW);
+    const int ok = __shfl_xor_sync(kAll, wkey, o * Sh::PW);
+    if (od < worst || (od == worst && ok < wkey)) { worst = od; wkey = ok; }
+  }
+  *ekey = wkey;
+  *edE = __double2float_rn(worst);
+  if (go && (bad || (full && fail))) return 2;
+  return full && wkey != INT_MAX ? 1 : 0;
 }
 
 // The candidates of the chunk's objects (k_lane_merge's records) to their
-// labels and exact distances, as k_exact; an object with a candidate that
-// does not verify is listed for k_exact (fb, counted in ctr[2]).
+// labels and exact distances, as k_exact: a basis that is not optimal in FP64
+// takes its pivot here (the same entering cell) and is tested again; an object
+// with a candidate that still does not verify is listed for k_exact (fb,
+// counted in ctr[2]).
 template <class Sh>
 __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     k_lane_exact(ObjView ob, CentView cv, long long seg_size, int K, SolveCfg cfg, LaneArgs A,
@@ -1432,7 +1646,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
   const int lane = threadIdx.x & 31;
   long long first, cnt;
   lane_chunk(A, total_obj, &first, &cnt);
-  int n_ex = 0;
+  int n_ex = 0, p_ex = 0;
   const long long step = (long long)gridDim.x * (blockDim.x >> 5) * PW;
   for (long long t0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PW; t0 < cnt;
        t0 += step) {
@@ -1469,7 +1683,9 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
         j = mr[1 + c];
         c0 = cv.off[cb + j];
         P.n = (int)(cv.off[cb + j + 1] - c0);
-        if (A.list) {  // the pair's place in the list: kept centroids before j
+        if (A.by_pair) {
+          q = (unsigned long long)(i * (long long)K + j);
+        } else if (A.list) {  // the pair's place in the list: kept centroids before j
           const unsigned* kb = cfg.keep + i * cfg.keep_words;
           q = X.ostart[t] + __popc(kb[j >> 5] & ((1u << (j & 31)) - 1u));
           for (int w = 0; w < (j >> 5); ++w) q += __popc(kb[w]);
@@ -1479,40 +1695,74 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       }
       P.N = P.m + P.n;
       P.live = go;
-      // masses and the saved tree
-      const unsigned char* tr = A.tree + q * (unsigned)A.tstride;
+      // the saved tree, then (again after each pivot) the masses
+      const unsigned char* tr = A.tree + q * (unsigned long long)A.tstride;
       int root = INT_MAX;
       __syncwarp();
 #pragma unroll
       for (int k = 0; k < NPL; ++k) {
         const int y = P.node(k);
-        long long w = 0;
         unsigned p = 0xffu;
         if (go && P.nodek(k)) {
-          if (k < Sh::KR) {
-            w = A.omass[i * A.mstride + y];
-          } else {
-            const int r = y - MP;
-            w = cv.Qpre[c0 + r] - (r > 0 ? cv.Qpre[c0 + r - 1] : 0LL);
-          }
           p = tr[k < Sh::KR ? y : y - MP + P.m];
           if (p == 0xffu) root = min(root, y);
           else if (p >= (unsigned)P.m) p = p - P.m + MP;
         }
-        Mask<Sh::MW> none;
-        none.clear();
-        P.store(y, w, none, p);
+        P.put_par(y, p);
         P.potk(k) = 0.f;
       }
 #pragma unroll
       for (int o = Sh::G / 2; o > 0; o >>= 1)
         root = min(root, __shfl_xor_sync(kAll, root, o * PW));
       P.root = root == INT_MAX ? 0 : root;
-      __syncwarp();
+      auto masses = [&](bool on) {
+        __syncwarp();
+#pragma unroll 1
+        for (int k = 0; k < NPL; ++k) {
+          const int y = P.node(k);
+          if (!on) continue;
+          long long w = 0;
+          Mask<Sh::MW> one;
+          one.clear();
+          if (y < MP ? y < P.m : y - MP < P.n) {
+            one.set(y);
+            if (y < MP) {
+              w = A.omass[i * A.mstride + y];
+            } else {
+              const int r = y - MP;
+              w = cv.Qpre[c0 + r] - (r > 0 ? cv.Qpre[c0 + r - 1] : 0LL);
+            }
+          }
+          P.store(y, w, one, P.par(y));
+        }
+        __syncwarp();
+      };
       double D = d64c;
-      const bool ok = lane_verify<Sh>(P, go, !known, pot64, ob, o0, cv, c0, &D);
-      if (go && !ok) fallback = true;
-      if (go && ok && !known && P.g == 0) {
+      bool todo = go;
+      int verdict = go ? 2 : 0;
+      for (int att = 0; att < 24; ++att) {
+        masses(todo);
+        int key;
+        float dE;
+        const int v = lane_verify<Sh>(P, todo, !known, pot64, ob, o0, cv, c0, &D, &key, &dE);
+        if (todo) verdict = v;
+        todo = todo && v == 1;
+        if (!__any_sync(kAll, todo)) break;
+        masses(todo);
+        P.live = todo;
+        P.template from_parents<true>();
+        int moved;
+        if constexpr (Sh::G >= 16) moved = P.pivot_scan(todo, todo ? key : 0, dE);
+        else moved = P.pivot(todo, todo ? key : 0, dE);
+        if (todo && moved < 0) {
+          verdict = 2;
+          todo = false;
+        }
+        if (todo && P.g == 0) ++p_ex;
+      }
+      P.live = go;
+      if (go && verdict != 0) fallback = true;
+      if (go && verdict == 0 && !known && P.g == 0) {
         ++n_ex;
         if (cfg.pair64) cfg.pair64[i * (long long)K + j] = D;
       }
@@ -1554,8 +1804,11 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       }
     }
   }
-  for (int o = 16; o > 0; o >>= 1) n_ex += __shfl_xor_sync(kAll, n_ex, o);
-  if (lane == 0) add_stats(0, 0, n_ex, 0);
+  for (int o = 16; o > 0; o >>= 1) {
+    n_ex += __shfl_xor_sync(kAll, n_ex, o);
+    p_ex += __shfl_xor_sync(kAll, p_ex, o);
+  }
+  if (lane == 0) add_stats(0, 0, n_ex, p_ex);
 }
 
 // Blocks of two warps where they fit, one otherwise.
@@ -1586,11 +1839,13 @@ cudaError_t lane_launch(const ObjView& ob, const CentView& cv, long long seg_siz
     return lane_blocks(k_lane_exact<Sh>, A.warp_bytes, cfg.sms, warps, st, ob, cv, seg_size, K, cfg,
                        A, total_obj, X);
   }
-  if (cfg.certify)
-    return lane_blocks(k_lane_screen<Sh, true>, A.warp_bytes, cfg.sms, warps, st, ob, cv, seg_size,
-                       K, cfg, A, total_obj);
-  return lane_blocks(k_lane_screen<Sh, false>, A.warp_bytes, cfg.sms, warps, st, ob, cv, seg_size, K,
-                     cfg, A, total_obj);
+  auto screen = [&](auto kern) {
+    return lane_blocks(kern, A.warp_bytes, cfg.sms, warps, st, ob, cv, seg_size, K, cfg, A,
+                       total_obj);
+  };
+  if (A.by_pair)
+    return cfg.certify ? screen(k_lane_screen<Sh, true, true>) : screen(k_lane_screen<Sh, false, true>);
+  return cfg.certify ? screen(k_lane_screen<Sh, true, false>) : screen(k_lane_screen<Sh, false, false>);
 }
 
 }  // namespace

@@ -11,6 +11,9 @@
 #include <cfloat>
 #include <climits>
 #include <cmath>
+#include <map>
+#include <mutex>
+#include <tuple>
 
 #include "d2_internal.h"
 #include "d2_solver.cuh"
@@ -1359,6 +1362,10 @@ __global__ void __launch_bounds__(128) k_exact(ObjView ob, CentView cv, long lon
             const long long wt = (i * (long long)K + j) * ws.ns;
             if (ws.flow) {
               S.load_tree(ws.par8 + wt, ws.pos8 + wt, ws.sz8 + wt, ws.flow + wt);
+            } else if (!ws.pos8) {
+              load_cent_prefix<G>(g, cv, c0, n, s64.Q);
+              if (S.load_parents(ws.par8 + wt)) S.recompute_flows();
+              else S.init_northwest();
             } else {
               load_cent_prefix<G>(g, cv, c0, n, s64.Q);
               S.template load_tree<false>(ws.par8 + wt, ws.pos8 + wt, ws.sz8 + wt, nullptr);
@@ -1396,6 +1403,9 @@ __global__ void __launch_bounds__(128) k_exact(ObjView ob, CentView cv, long lon
                                            cv.loc64 + c0 * cv.d, cv.d);
           if (ws.flow) {
             S.load_tree(ws.par8 + wt, ws.pos8 + wt, ws.sz8 + wt, ws.flow + wt);
+          } else if (!ws.pos8) {  // parents only (the lane screen's)
+            if (S.load_parents(ws.par8 + wt)) S.recompute_flows();
+            else S.init_northwest();
           } else {
             S.template load_tree<false>(ws.par8 + wt, ws.pos8 + wt, ws.sz8 + wt, nullptr);
             S.recompute_flows();
@@ -1440,13 +1450,37 @@ static int groups_per_block(int G, size_t slice, int tpb = 128) {
   return gpb >= per_warp ? gpb : 0;
 }
 
+// Blocks of a kernel that fit an SM, asked once per shape.  The kernel's
+// dynamic shared memory limit goes to the hardware's (never down to one
+// launch's need: launches of other sizes, other threads' and captured ones,
+// share it).
+static cudaError_t blocks_per_sm(const void* kern, size_t smem, int threads, int* per_sm) {
+  static std::mutex mu;
+  static std::map<std::tuple<const void*, size_t, int, int>, int> known;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const auto key = std::make_tuple(kern, smem, threads, dev);
+  std::lock_guard<std::mutex> lk(mu);
+  const auto it = known.find(key);
+  if (it != known.end()) {
+    *per_sm = it->second;
+    return cudaSuccess;
+  }
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e != cudaSuccess) return e;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, threads, smem);
+  if (e != cudaSuccess) return e;
+  if (known.size() >= 4096) known.clear();
+  known.emplace(key, *per_sm);
+  return cudaSuccess;
+}
+
 template <typename KernelT>
 static cudaError_t launch_cfg(KernelT kern, size_t smem, int threads, int sms, long long work,
                               int gpb, unsigned* grid) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+  const cudaError_t e = blocks_per_sm(reinterpret_cast<const void*>(kern), smem, threads, &per_sm);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   long long need = (work + gpb - 1) / gpb;

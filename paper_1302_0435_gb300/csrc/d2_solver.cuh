@@ -1308,6 +1308,73 @@ struct Simplex {
     g.sync();
   }
 
+  // Restore a basis kept as parents only (255: the root): subtree sizes and
+  // preorder positions (siblings in index order) are rebuilt by walking up
+  // from every node; the caller recomputes the flows.  False if the parents
+  // are not a tree.
+  __device__ bool load_parents(const unsigned char* par8) {
+    int* pr = s.pj0;
+    int* szs = s.ppos;
+    int* off = s.psz;
+    bool ok = true;
+    int r0 = INT_MAX;
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const int y = node_of(k);
+      if (y < N) {
+        const int p = par8[y];
+        if (p == 0xff) r0 = y;
+        else if (p >= N || (y < m) == (p < m)) ok = false;
+        pr[y] = p;
+        szs[y] = 0;
+      }
+    }
+    root = (int)__reduce_min_sync(g.mask, (unsigned)r0);
+    if (gany<G>(g, !ok || (r0 != INT_MAX && r0 != root)) || root >= N) return false;
+    g.sync();
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const int y = node_of(k);
+      if (y < N) {
+        int x = y, it = 0;
+        for (; it < N; ++it) {
+          atomicAdd(&szs[x], 1);
+          if (x == root) break;
+          x = pr[x];
+        }
+        if (it == N) ok = false;
+      }
+    }
+    if (gany<G>(g, !ok)) return false;
+    g.sync();
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const int y = node_of(k);
+      if (y < N) {
+        int o = 1;
+        for (int x = 0; x < y; ++x) o += (pr[x] == pr[y] && x != root) ? szs[x] : 0;
+        off[y] = o;
+      }
+    }
+    g.sync();
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const int y = node_of(k);
+      if (y < N) {
+        int pos = 0;
+        for (int x = y, it = 0; x != root && it < N; ++it, x = pr[x]) pos += off[x];
+        t.par[k] = y == root ? -1 : pr[y];
+        t.pos[k] = pos;
+        t.sz[k] = szs[y];
+        t.flow[k] = 0LL;
+        s.pos[y] = pos;
+        s.sz[y] = t.sz[k];
+      }
+    }
+    g.sync();
+    return true;
+  }
+
   // sum over tree edges of flow * cost, in the accumulator type A
   template <typename A>
   __device__ __forceinline__ A objective() const {
