@@ -467,14 +467,18 @@ int bins_to_host(d2_ctx* c, Bins* b) {
 
 // The support counts at which a binned batch is cut into launches, increasing,
 // the last one mmax.  The lane screen's shared memory and row loops follow
-// the launch's row bound, so its launches step by a third to a half of it;
-// the warp-per-pair kernels change with the nodes per lane only.
-int size_cuts(bool lanes, int mmax, int nmax, int* cut) {
+// the launch's row bound, so its launches step by a third to a half of it, as
+// long as each of them has several waves of pairs to solve (a launch of one
+// wave costs a pair's latency, 50 to 150 us); small trees of a batch below
+// 2^17 objects go together, and only the mask widths part the larger ones.
+// The warp-per-pair kernels change with the nodes per lane only.
+int size_cuts(bool lanes, long long count, int mmax, int nmax, int* cut) {
   static const int steps[] = {4, 8, 12, 16, 24, 32, 48};
   int k = 0;
   if (lanes) {
+    const bool many = count >= (1LL << 17);
     for (int s : steps)
-      if (s < mmax) cut[k++] = s;
+      if (s < mmax && (many || s == 16 || s == 32 || (s == 8 && nmax > 16))) cut[k++] = s;
   } else {
     for (int b = 1; b < 4; ++b)
       if (32 * b - nmax >= 1 && 32 * b - nmax < mmax) cut[k++] = 32 * b - nmax;
@@ -568,7 +572,7 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
   const bool lanes = base.lanes && mode == 1;
   const bool tuning = c->cfg.group_lanes == 0 && mode == 1 && v.count >= 8192 && !lanes;
   int cut[8];
-  const int ncut = size_cuts(lanes, mmax, nmax, cut);
+  const int ncut = size_cuts(lanes, v.count, mmax, nmax, cut);
   for (int b = ncut - 1; b >= 0; --b) {
     const int lo = b > 0 ? cut[b - 1] : 0;  // support counts lo + 1 .. cut[b]
     SolveCfg cfg = base;
@@ -936,7 +940,7 @@ int segment_impl(d2_ctx* c, const ObjView& v, int mmax, const double* om, long l
 bool want_bins(const d2_ctx* c, const SolveCfg& cfg, long long count, int mmax) {
   int cut[8];
   return count >= 4096 &&
-         size_cuts(cfg.lanes && cfg.mode == 1, mmax, std::max(c->nmax, 1), cut) > 1;
+         size_cuts(cfg.lanes && cfg.mode == 1, count, mmax, std::max(c->nmax, 1), cut) > 1;
 }
 
 }  // namespace

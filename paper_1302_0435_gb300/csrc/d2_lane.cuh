@@ -405,22 +405,36 @@ struct Lane {
     for (int k = 0; k < NPL; ++k)
       if (live) flowk(k) = 0;
     __syncwarp();
+    // the own nodes walk together, a step of all of them at a time
+    int x[NPL];
+    unsigned going = 0u;
 #pragma unroll
     for (int k = 0; k < NPL; ++k) {
-      if (live && nodek(k)) {
-        const int y = node(k);
-        int x = y;
-        for (int it = 0; it < NS && x != root; ++it) {
-          atomicAdd(reinterpret_cast<unsigned long long*>(&flow(x)), (unsigned long long)b[k]);
-          if (MASKS && x != y) or_mask(x, y);
-          const unsigned p = par(x);
-          if (p >= (unsigned)NS || is_row(x) == is_row((int)p)) { bad = true; break; }
-          x = (int)p;
+      x[k] = node(k);
+      if (live && nodek(k)) going |= 1u << k;
+    }
+    for (int it = 0; it < NS && going; ++it) {
+#pragma unroll
+      for (int k = 0; k < NPL; ++k) {
+        if ((going >> k) & 1u) {
+          if (x[k] == root) {
+            if (MASKS && it > 0) or_mask(root, node(k));
+            going &= ~(1u << k);
+          } else {
+            atomicAdd(reinterpret_cast<unsigned long long*>(&flow(x[k])), (unsigned long long)b[k]);
+            if (MASKS && it > 0) or_mask(x[k], node(k));
+            const unsigned p = par(x[k]);
+            if (p >= (unsigned)NS || is_row(x[k]) == is_row((int)p)) {
+              bad = true;
+              going &= ~(1u << k);
+            } else {
+              x[k] = (int)p;
+            }
+          }
         }
-        if (x != root) bad = true;  // no way to the root
-        else if (MASKS && y != root) or_mask(root, y);
       }
     }
+    bad |= going != 0u;  // no way to the root
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < NPL; ++k) {
@@ -1478,13 +1492,15 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       }
       const float D = Lane<Sh>::sum(acc);
       const float e = D * rel + cmax * 0x1p-14f + tc_e;
-      const bool good = st == kStOk && !isnan(D) && !isnan(e);
+      const bool good = st == kStOk && isfinite(D) && isfinite(e);
       if (P.live && P.g == 0 && cfg.pair_out) {
         float* po = cfg.pair_out + 2 * (i * (long long)K + j);
         po[0] = D;
         po[1] = st != kStOk ? INFINITY : e;
       }
-      rec.lo = good ? D - e : -FLT_MAX;
+      // a solve that failed has no bound; one whose costs are not finite is
+      // no candidate
+      rec.lo = good ? D - e : (st == kStOk ? INFINITY : -FLT_MAX);
       rec.hi = good ? D + e : FLT_MAX;
     }
     if (q < total && P.g == 0) {
