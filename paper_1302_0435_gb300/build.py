@@ -65,8 +65,9 @@ def build(force=False, verbose=False, extra=None):
             sys.stderr.write(r.stdout + r.stderr)
         return obj
 
-    srcs = sources()
-    with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    # the largest sources first, so that none is left for the end alone
+    srcs = sorted(sources(), key=lambda p: -(os.path.getsize(p) + 100000 * ("lane_" in p)))
+    with cf.ThreadPoolExecutor(max_workers=min(max(8, os.cpu_count() or 8), len(srcs))) as ex:
         objs = list(ex.map(compile_one, srcs))
     tmp = LIB + ".tmp.%d" % os.getpid()
     cmd = [nvcc] + ARCH + ["-shared", "-o", tmp] + objs + ["-ldl"]  # NVTX 3 loads its injection

@@ -42,7 +42,7 @@ enum Slot {
   kMbPair, kMbTmpLab, kMbTmpD2, kMbCnt, kMbStart, kMbPObj, kMbPCen, kMbD2, kMbSt,
   // joint weights (Alg. 1 Step 1)
   kJState, kJPot, kJPStart, kJEps, kJIters, kJSort, kJPObj, kJPCen, kJW, kJSt, kJTree,
-  kPairTree, kPairTree2,
+  kPairTree, kPairTree2, kPairDone,
   // d2_mallows_all
   kAllLab, kAllD2, kAllPair,
   // pruning of pairs that cannot be the argmin
@@ -286,6 +286,15 @@ int attach_tree(d2_ctx* c, SolveCfg* cfg, long long npairs, int slot = kPairTree
   return D2_OK;
 }
 
+// A pair list solved by lanes: its flag byte per pair.  (A caller that fixed a
+// cold-start rule keeps the warp-per-pair kernels.)
+int attach_done(d2_ctx* c, SolveCfg* cfg, long long npairs) {
+  if (!cfg->lanes || npairs <= 0) return D2_OK;
+  int rc = D2_OK;
+  cfg->done = static_cast<unsigned char*>(grow(c, kPairDone, (size_t)npairs, &rc));
+  return rc;
+}
+
 CentView resident_view(const d2_ctx* c) {
   CentView v;
   v.loc32 = c->c_loc32;
@@ -520,7 +529,7 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
   if (certify_all && mode == 1) base.certify = true;
   base.pair64 = pair64;
   const bool prune = prunes(c, base, cv);
-  if (base.mode == 1 && (prune || base.lanes)) {
+  if (prune || base.lanes) {
     // (a level prepares its bags once: prep_bags)
     int rc = D2_OK;
     if (!bags_ready && (rc = prep_bags(c, v, mmax, prune))) return rc;
@@ -569,7 +578,7 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
   }
   // the lane screen has one launch shape per bound; the warp-per-pair screen
   // is tuned
-  const bool lanes = base.lanes && mode == 1;
+  const bool lanes = base.lanes;
   const bool tuning = c->cfg.group_lanes == 0 && mode == 1 && v.count >= 8192 && !lanes;
   int cut[8];
   const int ncut = size_cuts(lanes, v.count, mmax, nmax, cut);
@@ -940,7 +949,7 @@ int segment_impl(d2_ctx* c, const ObjView& v, int mmax, const double* om, long l
 bool want_bins(const d2_ctx* c, const SolveCfg& cfg, long long count, int mmax) {
   int cut[8];
   return count >= 4096 &&
-         size_cuts(cfg.lanes && cfg.mode == 1, count, mmax, std::max(c->nmax, 1), cut) > 1;
+         size_cuts(cfg.lanes, count, mmax, std::max(c->nmax, 1), cut) > 1;
 }
 
 }  // namespace
@@ -1242,7 +1251,9 @@ int d2_mallows_batch(d2_ctx* c, const d2_bags* objs, const int64_t* pair_obj, co
   }
   if ((rc = check_bag_symbols(c, v))) return rc;
   SolveCfg cfg = solve_cfg(c, mode_for(c, objs->loc_dtype), mmax);
-  if ((rc = attach_tree(c, &cfg, npairs))) return rc;
+  if (cfg.lanes) rc = attach_done(c, &cfg, npairs);
+  else rc = attach_tree(c, &cfg, npairs);
+  if (rc != D2_OK) return rc;
   CK(d2k::mallows_pairs(v, resident_view(c), po, pc, npairs, cfg, dd, fo, ds, c->d_err, c->stream));
   if (h1) CK(cudaMemcpyAsync(dist2, dd, (size_t)npairs * 8, cudaMemcpyDeviceToHost, c->stream));
   if (h2) CK(cudaMemcpyAsync(status, ds, (size_t)npairs * 4, cudaMemcpyDeviceToHost, c->stream));
@@ -1546,6 +1557,7 @@ int resolve_assigned(d2_ctx* c, const ObjView& v, const int* dl, int mmax, const
   k_pairs_from_labels<<<blocks_for(N), 256, 0, c->stream>>>(dl, N, po, pc);
   d2k::note_launches(1);
   SolveCfg cfg = solve_cfg(c, 0, mmax);
+  if ((rc = attach_done(c, &cfg, N))) return rc;
   CK(d2k::mallows_pairs(v, cv, po, pc, N, cfg, dd, *fo, nullptr, c->d_err, c->stream));
   return D2_OK;
 }
@@ -1894,7 +1906,8 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     if (want_bins(c, cfg, n_l, cur_mmax) && (rc = make_bins(c, cur, &bins)))
       return rc;
     // this level's bags (masses, pruning moments), once for all its rounds
-    if (cfg.mode == 1 && (rc = prep_bags(c, cur, cur_mmax, prunes(c, cfg, cv)))) return rc;
+    if ((cfg.lanes || cfg.mode == 1) && (rc = prep_bags(c, cur, cur_mmax, prunes(c, cfg, cv))))
+      return rc;
     // Rounds 2.. repeat the same launches (same pairs, warm bases): round 1
     // is captured into a CUDA graph once and replayed.
     cudaGraphExec_t gexec = nullptr;
@@ -1938,7 +1951,8 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
       cudaStreamIsCapturing(c->stream, &cst);
       const bool capturing = cst == cudaStreamCaptureStatusActive;
       int rc2 = run_assign(c, cur, cv, seg, K, cfg.mode, cur_mmax, om, lab, ld2, lterms, fo, cand,
-                           ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr, cfg.mode == 1);
+                           ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr,
+                           cfg.lanes || cfg.mode == 1);
       cudaError_t ue = cudaSuccess;
       if (rc2 == D2_OK && it < iters && alg1) {
         // Alg. 1 Step 1: support weights of every cluster of the level by the
@@ -1978,7 +1992,7 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
           // run the round directly instead
           if ((rc = run_assign(c, cur, cv, seg, K, cfg.mode, cur_mmax, om, lab, ld2, lterms, fo,
                                cand, ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr,
-                               cfg.mode == 1)))
+                               cfg.lanes || cfg.mode == 1)))
             return rc;
           if (it < iters)
             CK(d2k::update_locations(cur, om, lab, seg, K, fo, KT, loff, d, c->cent_ldt, l32, l64,

@@ -167,6 +167,9 @@ struct SolveCfg {
   // handed from the FP32 launch to the FP64 launch; null: one fused launch
   unsigned char* tree = nullptr;
   size_t tree_bytes = 0;
+  // mallows_pairs by lanes: a byte per pair (null: the warp-per-pair kernels);
+  // there: pairs to skip
+  unsigned char* done = nullptr;
   // joint-weights rounds (mallows_pairs with the hand-over above): the
   // optimal basis of each object's pair from the previous round, indexed by
   // OBJECT (node y of object i at [i*jw.ns + y]; sz8 of node 0 == 0: none
@@ -272,6 +275,18 @@ struct ExactOut {
   int* err = nullptr;
 };
 
+// A list of pairs for lane_pairs.
+struct PairJob {
+  const long long* pobj;
+  const long long* pcen;
+  long long npairs;
+  double* dist2;
+  int* status;           // may be null
+  FlowOut fo;
+  unsigned char* done;   // [npairs] 1: solved here
+  int* err;
+};
+
 // Scratch of lane_screen behind the merged lists: byte offsets of the object
 // masses, flags and list starts, the pair list and the pair records, for
 // chunks of `objects` objects (about max_pairs pairs).
@@ -317,19 +332,29 @@ cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_siz
                         const TcWork* tw, const WarmStore* ws, ExactOut X);
 // Row ranks, means and principal directions of the bags (SolveCfg::rows, axes).
 cudaError_t lane_axes(const ObjView& ob, const SolveCfg& cfg, cudaStream_t st);
+// Listed pairs by lanes (mode 0: FP64 throughout); J.done says which it solved.
+cudaError_t lane_pairs(const ObjView& ob, const CentView& cv, const PairJob& J,
+                       const SolveCfg& cfg, cudaStream_t st);
 // Launch settings of k_exact over the fallback list of lane_screen.
 void lane_fallback(const ObjView& ob, int K, int* cand, SolveCfg* cfg);
-#define D2_LANE_DECL(U)                                                                          \
-  cudaError_t lane_screen_##U(const ObjView& ob, const CentView& cv, long long seg_size, int K,  \
-                              const SolveCfg& cfg, const LaneArgs& A, long long total_obj,       \
-                              long long work, const ExactOut& X, cudaStream_t st);               \
+#define D2_LANE_SHAPES(X) \
+  X(a6) X(a7) X(a8) X(b5) X(b6) X(b7) X(b8) X(c6) X(c8) X(d5) X(e5) X(e6) X(f3) X(f4)
+#define D2_LANE_WIDE(X) X(a8) X(b6) X(b8) X(c8) X(d5) X(e6) X(f4)
+#define D2_LANE_DECL(U)                                                                        \
+  cudaError_t lane_run_##U(const ObjView& ob, const CentView& cv, long long seg_size, int K,   \
+                           const SolveCfg& cfg, const LaneArgs& A, long long total_obj,        \
+                           long long work, const ExactOut& X, cudaStream_t st);                \
   cudaError_t stats_lane_##U(long long out[6]);
-D2_LANE_DECL(a)
-D2_LANE_DECL(b)
-D2_LANE_DECL(c)
-D2_LANE_DECL(d)
-D2_LANE_DECL(e)
-D2_LANE_DECL(f)
+#define D2_LANE_DECL2(U)                                                                       \
+  cudaError_t lane_all64_##U(const ObjView& ob, const CentView& cv, long long seg_size, int K, \
+                             const SolveCfg& cfg, const LaneArgs& A, long long total_obj,      \
+                             long long work, const ExactOut& X, cudaStream_t st);              \
+  cudaError_t lane_pairs_##U(const ObjView& ob, const CentView& cv, const PairJob& J,          \
+                             const SolveCfg& cfg, cudaStream_t st);                            \
+  cudaError_t stats_lane_##U##_pairs(long long out[6]);
+D2_LANE_SHAPES(D2_LANE_DECL)
+D2_LANE_WIDE(D2_LANE_DECL2)
+#undef D2_LANE_DECL2
 #undef D2_LANE_DECL
 
 // ---- pairs that cannot be the argmin (Alg. 2 Step 2 needs only it) ----

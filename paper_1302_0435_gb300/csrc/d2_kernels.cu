@@ -467,9 +467,12 @@ long long launches() { return (long long)__atomic_load_n(&g_launches, __ATOMIC_R
 
 // Sum of the solver counters of the units that hold the solver kernels.
 cudaError_t solver_stats(long long out[6]) {
-  cudaError_t (*const units[])(long long*) = {
-      stats_npl1,   stats_npl2,   stats_npl3,   stats_npl4,   stats_lane_a,
-      stats_lane_b, stats_lane_c, stats_lane_d, stats_lane_e, stats_lane_f};
+#define X(u) stats_lane_##u,
+#define XP(u) stats_lane_##u##_pairs,
+  cudaError_t (*const units[])(long long*) = {stats_npl1, stats_npl2, stats_npl3, stats_npl4,
+                                              D2_LANE_SHAPES(X) D2_LANE_WIDE(XP)};
+#undef X
+#undef XP
   for (int i = 0; i < 6; ++i) out[i] = 0;
   for (auto f : units) {
     long long v[6];
@@ -537,6 +540,11 @@ cudaError_t mallows_pairs(const ObjView& ob, const CentView& cv, const long long
   if (npairs <= 0) return cudaSuccess;
   int G, NP;
   if (!pick_shape(cfg.mmax, cfg.nmax, &G, &NP)) return cudaErrorInvalidValue;
+  if (cfg.done) {  // by lanes; below, the few pairs it left
+    const PairJob J{pobj, pcen, npairs, dist2, status, fo, cfg.done, d_err};
+    const cudaError_t e = lane_pairs(ob, cv, J, cfg, st);
+    if (e != cudaSuccess) return e;
+  }
 #define X(g_, n_)                                                                          \
   if (G == g_ && NP == n_)                                                                \
     return mallows_pairs_npl##n_(ob, cv, pobj, pcen, npairs, cfg, dist2, fo, status, d_err, st);
@@ -551,9 +559,9 @@ cudaError_t assign(const ObjView& ob, const CentView& cv, long long seg_size, in
                    const WarmStore* ws, const TcWork* tw) {
   if (ob.count <= 0) return cudaSuccess;
   SolveCfg cfg = cfg0;
-  if (cfg.lanes && cfg.mode == 1 && cand && (!ws || !ws->pos8)) {
+  if (cfg.lanes && cand && (cfg.mode == 1 ? !ws || !ws->pos8 : true)) {
     ExactOut X;
-    if (cfg.lane_exact && !cfg.screen_only) {
+    if ((cfg.lane_exact || cfg.mode == 0) && !cfg.screen_only) {
       X.omega = omega;
       X.labels = labels;
       X.dist2 = dist2;
@@ -563,6 +571,7 @@ cudaError_t assign(const ObjView& ob, const CentView& cv, long long seg_size, in
     const cudaError_t e = lane_screen(ob, cv, seg_size, K, cfg, cand, d_err, st, tw, ws, X);
     if (e != cudaSuccess || cfg.screen_only) return e;
     cfg.screened = true;
+    if (cfg.mode == 0) return cudaSuccess;
     if (X.labels) {  // the few objects k_exact still solves
       if (!cfg.last) return cudaSuccess;
       if (cfg.mall > cfg.mmax) cfg.mmax = cfg.mall;

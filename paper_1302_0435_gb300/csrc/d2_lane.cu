@@ -99,7 +99,8 @@ __global__ void __launch_bounds__(256) k_lane_list(LaneArgs A, long long total_o
 // the smallest upper end), as k_merge writes them.  One warp per object.
 __global__ void __launch_bounds__(128) k_lane_merge(ObjView ob, LaneArgs A, long long total_obj,
                                                     int K, int mmax, const unsigned* keep, int kw,
-                                                    const unsigned long long* ostart, int* cand) {
+                                                    const unsigned long long* ostart, int* cand,
+                                                    bool fp64) {
   long long first, cnt;
   lane_chunk(A, total_obj, &first, &cnt);
   const int lane = threadIdx.x & 31;
@@ -119,6 +120,30 @@ __global__ void __launch_bounds__(128) k_lane_merge(ObjView ob, LaneArgs A, long
       unsigned x = 0;
       for (int k = lane; k < kw; k += 32) x += __popc(keep[i * kw + k]);
       c = (int)__reduce_add_sync(0xffffffffu, x);
+    }
+    if (fp64) {  // exact values: the smallest, ties to the smallest centroid
+      double best = NAN;
+      int bj = INT_MAX;
+      for (int p = lane; p < c; p += 32) {
+        const double v = A.rec[s + p].d64;
+        if (v < best || bj == INT_MAX || (isnan(best) && !isnan(v))) { best = v; bj = p; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+        const bool take = isnan(best) ? (!isnan(ov) || oj < bj)
+                                      : (ov < best || (ov == best && oj < bj));
+        if (take) { best = ov; bj = oj; }
+      }
+      if (lane == 0) {
+        out[0] = 1;
+        out[1] = bj;
+        const long long bits = __double_as_longlong(best);
+        out[1 + kCandCap] = (int)(unsigned)(bits & 0xffffffffLL);
+        out[2 + kCandCap] = (int)(bits >> 32);
+      }
+      continue;
     }
     float hi = FLT_MAX;
     int at = INT_MAX;
@@ -171,11 +196,33 @@ static cudaError_t lane_dispatch(const ObjView& ob, const CentView& cv, long lon
                                  const SolveCfg& cfg, const LaneArgs& A, long long total_obj,
                                  long long work, const ExactOut& X, cudaStream_t st) {
   auto run = [&](auto unit) { return unit(ob, cv, seg_size, K, cfg, A, total_obj, work, X, st); };
-  if (cfg.mmax > 64 || cfg.nmax > 64) return cudaErrorInvalidValue;
-  if (cfg.nmax <= 16) return run(cfg.mmax <= 16 ? lane_screen_a : lane_screen_d);
-  if (cfg.nmax <= 32)
-    return run(cfg.mmax <= 16 ? lane_screen_b : cfg.mmax <= 32 ? lane_screen_c : lane_screen_e);
-  return run(lane_screen_f);
+  const int m = cfg.mmax, n = cfg.nmax;
+  if (m > 64 || n > 64) return cudaErrorInvalidValue;
+  if (cfg.mode == 0 && !X.labels) {  // FP64 throughout: the widest shapes only
+    if (n <= 16) return run(m <= 16 ? lane_all64_a8 : m <= 48 ? lane_all64_c8 : lane_all64_d5);
+    if (n <= 32) return run(m <= 16 ? lane_all64_b6 : m <= 32 ? lane_all64_b8 : lane_all64_e6);
+    return run(lane_all64_f4);
+  }
+  if (n <= 16) {
+    if (m <= 16) return run(m <= 8 ? lane_run_a6 : m <= 12 ? lane_run_a7 : lane_run_a8);
+    return run(m <= 32 ? lane_run_c6 : m <= 48 ? lane_run_c8 : lane_run_d5);
+  }
+  if (n <= 32) {
+    if (m <= 16) return run(m <= 8 ? lane_run_b5 : lane_run_b6);
+    if (m <= 32) return run(m <= 24 ? lane_run_b7 : lane_run_b8);
+    return run(m <= 48 ? lane_run_e5 : lane_run_e6);
+  }
+  return run(m <= 32 ? lane_run_f3 : lane_run_f4);
+}
+
+cudaError_t lane_pairs(const ObjView& ob, const CentView& cv, const PairJob& J,
+                       const SolveCfg& cfg, cudaStream_t st) {
+  auto run = [&](auto unit) { return unit(ob, cv, J, cfg, st); };
+  const int m = cfg.mmax, n = cfg.nmax;
+  if (m > 64 || n > 64) return cudaErrorInvalidValue;
+  if (n <= 16) return run(m <= 16 ? lane_pairs_a8 : m <= 48 ? lane_pairs_c8 : lane_pairs_d5);
+  if (n <= 32) return run(m <= 16 ? lane_pairs_b6 : m <= 32 ? lane_pairs_b8 : lane_pairs_e6);
+  return run(lane_pairs_f4);
 }
 
 // Screen of the launch's objects: merged candidate lists (k_merge's records)
@@ -257,11 +304,13 @@ cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_siz
                                                                     cfg.keep_words, list, ostart);
       note_launches(1);
     }
-    e = lane_dispatch(ob, cv, seg_size, K, sc, A, total_obj, most * (long long)K, ExactOut{}, st);
+    ExactOut none;
+    none.err = d_err;
+    e = lane_dispatch(ob, cv, seg_size, K, sc, A, total_obj, most * (long long)K, none, st);
     if (e != cudaSuccess) return e;
     if (cfg.screen_only) continue;
     k_lane_merge<<<grid_for(most, 4, 16 * cfg.sms), 128, 0, st>>>(
-        ob, A, total_obj, K, cfg.mmax, cfg.keep, cfg.keep_words, ostart, merged);
+        ob, A, total_obj, K, cfg.mmax, cfg.keep, cfg.keep_words, ostart, merged, cfg.mode == 0);
     note_launches(1);
     if (X.labels) {
       e = lane_dispatch(ob, cv, seg_size, K, cfg, A, total_obj, most, X, st);

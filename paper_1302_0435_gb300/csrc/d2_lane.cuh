@@ -43,9 +43,11 @@ namespace {
 // G lanes per pair, L of them across the blocks of 4 columns (the other
 // factor G / L splits the rows), MW 32-bit words per node mask, NPL node
 // slots per lane: 4 L columns and G NPL - 4 L rows.
-template <int G_, int L_, int MW_, int NPL_>
+template <int G_, int L_, int MW_, int NPL_, typename T_ = float>
 struct LaneShape {
+  using T = T_;  // costs and potentials: FP32 screens, or FP64 throughout
   static constexpr int G = G_, L = L_, MW = MW_, NPL = NPL_;
+  static constexpr int TS = (int)sizeof(T);
   static constexpr int PW = 32 / G;           // pairs per warp
   static constexpr int RS = G / L;            // row groups
   static constexpr int PS = PW * 16;          // bytes between a pair's units
@@ -59,7 +61,7 @@ struct LaneShape {
   // the fourth word where the mask is one word (one 128-bit access per step
   // of a walk); masks of 4 words have a unit of their own.
   static constexpr int kPot = 0;
-  static constexpr int kNode = kPot + NPL * 128;
+  static constexpr int kNode = kPot + NPL * 32 * TS;
   static constexpr int kD4 = kNode + NPL * 512;               // MW = 4
   static constexpr int kPar = kD4 + (MW == 4 ? NPL * 512 : 0);  // MW > 1
   static constexpr int kCode = kPar + (MW > 1 ? (NS + 15) / 16 * PS : 0);
@@ -69,7 +71,7 @@ struct LaneShape {
 // Bytes of a warp with room for mmax rows of nb column blocks.
 template <class Sh>
 inline size_t lane_warp_bytes(int mmax, int nb) {
-  return (size_t)Sh::kTile + (size_t)((mmax + 3) & ~3) * nb * Sh::PS;
+  return (size_t)Sh::kTile + (size_t)((mmax + 3) & ~3) * nb * Sh::PS * (Sh::TS / 4);
 }
 
 template <int MW>
@@ -112,8 +114,14 @@ struct Mask {
 // One pair's view of its warp's shared memory and its solver state; every
 // lane of the warp runs the same code (a pair without work has live = false
 // and only joins the shuffles).
+template <typename T>
+struct V4 {
+  T x, y, z, w;
+};
+
 template <class Sh>
 struct Lane {
+  using T = typename Sh::T;
   static constexpr int G = Sh::G, L = Sh::L, MW = Sh::MW, NPL = Sh::NPL, RS = Sh::RS;
   static constexpr int PW = Sh::PW, PS = Sh::PS, MP = Sh::MP, NS = Sh::NS, KR = Sh::KR;
   static constexpr unsigned kAll = 0xffffffffu;
@@ -136,20 +144,50 @@ struct Lane {
   }
 
   // ---- shared memory: any node, and the own node of slot k (y = g + G k) ----
-  __device__ __forceinline__ float4& tile4(int a, int cb) const {
-    return *reinterpret_cast<float4*>(sp + Sh::kTile + (a * nb + cb) * PS);
+  // a block of 4 columns of row a (one unit of floats, two of doubles)
+  __device__ __forceinline__ char* tp(int a, int cb) const {
+    return sp + Sh::kTile + (a * nb + cb) * (PS * (Sh::TS / 4));
   }
-  __device__ __forceinline__ float& cell(int a, int r) const {
-    return *reinterpret_cast<float*>(sp + Sh::kTile + (a * nb + (r >> 2)) * PS + (r & 3) * 4);
+  __device__ __forceinline__ float4& tile4(int a, int cb) const {
+    return *reinterpret_cast<float4*>(tp(a, cb));
+  }
+  __device__ __forceinline__ static V4<T> ld4(const char* p) {
+    if constexpr (Sh::TS == 4) {
+      const float4 v = *reinterpret_cast<const float4*>(p);
+      return V4<T>{v.x, v.y, v.z, v.w};
+    } else {
+      const double2 a = *reinterpret_cast<const double2*>(p);
+      const double2 b = *reinterpret_cast<const double2*>(p + PS);
+      return V4<T>{a.x, a.y, b.x, b.y};
+    }
+  }
+  __device__ __forceinline__ static void st4(char* p, const V4<T>& v) {
+    if constexpr (Sh::TS == 4) {
+      *reinterpret_cast<float4*>(p) = make_float4(v.x, v.y, v.z, v.w);
+    } else {
+      *reinterpret_cast<double2*>(p) = make_double2(v.x, v.y);
+      *reinterpret_cast<double2*>(p + PS) = make_double2(v.z, v.w);
+    }
+  }
+  __device__ __forceinline__ T& cell(int a, int r) const {
+    constexpr int per = 16 / Sh::TS;  // values a unit
+    return *reinterpret_cast<T*>(tp(a, r >> 2) + ((r & 3) / per) * PS + (r % per) * Sh::TS);
   }
   __device__ __forceinline__ float4& pot4(int q) const {
     return *reinterpret_cast<float4*>(sp + Sh::kPot + q * PS);
   }
-  __device__ __forceinline__ float& pot(int y) const {
-    return *reinterpret_cast<float*>(sp + Sh::kPot + (y >> 2) * PS + (y & 3) * 4);
+  // potentials of nodes 4 q .. 4 q + 3
+  __device__ __forceinline__ V4<T> potq(int q) const {
+    return ld4(sp + Sh::kPot + q * (PS * (Sh::TS / 4)));
   }
-  __device__ __forceinline__ float& potk(int k) const {
-    return *reinterpret_cast<float*>(sp + Sh::kPot + (g >> 2) * PS + (g & 3) * 4 + k * 128);
+  __device__ __forceinline__ T& pot(int y) const {
+    constexpr int per = 16 / Sh::TS;
+    return *reinterpret_cast<T*>(sp + Sh::kPot + (y / per) * PS + (y % per) * Sh::TS);
+  }
+  __device__ __forceinline__ T& potk(int k) const {
+    constexpr int per = 16 / Sh::TS;
+    return *reinterpret_cast<T*>(sp + Sh::kPot + (g / per) * PS + (g % per) * Sh::TS +
+                                 k * (32 * Sh::TS));
   }
   __device__ __forceinline__ char* rec(int y) const { return sp + Sh::kNode + y * PS; }
   __device__ __forceinline__ long long& flow(int y) const {
@@ -269,11 +307,11 @@ struct Lane {
     return v;
   }
   // smallest (value, key) over W neighbouring lanes of the pair
-  template <int W>
-  __device__ __forceinline__ static void min_key(float& v, int& key) {
+  template <int W, typename V>
+  __device__ __forceinline__ static void min_key(V& v, int& key) {
 #pragma unroll
     for (int o = W / 2; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(kAll, v, o * PW);
+      const V ov = __shfl_xor_sync(kAll, v, o * PW);
       const int ok = __shfl_xor_sync(kAll, key, o * PW);
       if (ov < v || (ov == v && ok < key)) { v = ov; key = ok; }
     }
@@ -320,23 +358,23 @@ struct Lane {
   // 36 (117, 55, 84), high_dim 52 (217, 55, 76), sequences 11.2 (37, 9.8,
   // 13.8).  A step reads one row of the tile, where Vogel's rule keeps the two
   // best of every line.  flow holds the masses, D the singletons.
-  __device__ __forceinline__ void start_rows(const float4& vm) {
+  __device__ __forceinline__ void start_rows(const V4<T>& vm) {
     unsigned long long ra = m >= 64 ? ~0ull : ((1ull << m) - 1ull);
     unsigned long long ca = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
     int nr = m, nc = n, cur = -1;
     for (;;) {
       const bool act = live && nr > 1 && nc > 1;
       if (!__any_sync(kAll, act)) break;
-      float best = INFINITY;
+      T best = T(INFINITY);
       int key = INT_MAX;
       int a = 0;
       if (act) {
         const unsigned long long later = ra & ~((2ull << (cur & 63)) - 1ull);
         a = __ffsll((long long)((cur >= 0 && later) ? later : ra)) - 1;
         if (gl < nb) {
-          const float4 c = tile4(a, gl);
+          const V4<T> c = ld4(tp(a, gl));
           const unsigned al = (unsigned)(ca >> (4 * gl)) & 15u;
-          const float d[4] = {c.x - vm.x, c.y - vm.y, c.z - vm.z, c.w - vm.w};
+          const T d[4] = {c.x - vm.x, c.y - vm.y, c.z - vm.z, c.w - vm.w};
 #pragma unroll
           for (int i = 0; i < 4; ++i)
             if (((al >> i) & 1u) && d[i] < best) { best = d[i]; key = 4 * gl + i; }
@@ -386,6 +424,63 @@ struct Lane {
     for (int i = 0; i < MW; ++i) d.w[i] = oru(d.w[i]);
     if (live && g == 0) store(root, 0, getD(root).plus(d), 0xffu);
     __syncwarp();
+  }
+
+  // The object's masses into its rows' flow slots, as load_prefix makes them
+  // (the same sums in the same order: slot l holds supports l and l + 32, the
+  // slots are added in halves).  Returns false for a bag the solver rejects.
+  template <typename W>
+  __device__ __forceinline__ bool row_masses(bool act, const W* w, bool put = true) {
+    constexpr int SL = 32 / G;  // own slots of the sum
+    double x[KR];
+    bool wrong = false;
+#pragma unroll
+    for (int k = 0; k < KR; ++k) {
+      x[k] = 0.0;
+      if (act && node(k) < m) {
+        x[k] = (double)w[node(k)];
+        wrong |= !(x[k] >= 0.0) || isinf(x[k]);
+      }
+    }
+    double v[SL];
+#pragma unroll
+    for (int s = 0; s < SL; ++s) {
+      v[s] = s < KR ? x[s] : 0.0;
+      if (s + SL < KR) v[s] += x[s + SL];
+    }
+#pragma unroll
+    for (int h = SL / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int s = 0; s < h; ++s) v[s] += v[s + h];
+    const double s = sum(v[0]);
+    wrong |= act && (!(s > 0.0) || isinf(s));
+    if (oru(wrong ? 1u : 0u)) act = false;
+    const double inv = 1.0 / s;
+    long long q[KR], part = 0, bigv = -1;
+    int bigi = INT_MAX;
+#pragma unroll
+    for (int k = 0; k < KR; ++k) {
+      q[k] = 0;
+      if (act && node(k) < m) {
+        q[k] = __double2ll_rn(x[k] * inv * 4611686018427387904.0);
+        if (q[k] < 0) q[k] = 0;
+        part += q[k];
+        if (q[k] > bigv) { bigv = q[k]; bigi = node(k); }
+      }
+    }
+    part = sum(part);
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+      const long long ov = __shfl_xor_sync(kAll, bigv, o * PW);
+      const int oi = __shfl_xor_sync(kAll, bigi, o * PW);
+      if (ov > bigv || (ov == bigv && oi < bigi)) { bigv = ov; bigi = oi; }
+    }
+#pragma unroll
+    for (int k = 0; k < KR; ++k) {
+      if (act && node(k) == bigi) q[k] += kMass - part;
+      if (put) flowk(k) = q[k];
+    }
+    return act;
   }
 
   // Flows (and with MASKS the subtree sets) of the tree in par: the edge above
@@ -574,47 +669,54 @@ struct Lane {
 
   // Potentials from the tree: pot(root) = 0, pot(y) = c(y, par y) - pot(par y).
   __device__ __forceinline__ bool refresh() {
-    float acc[NPL];
+    T acc[NPL];
 #pragma unroll
     for (int k = 0; k < NPL; ++k) {
-      acc[k] = 0.f;
+      acc[k] = T(0);
       if (live && nodek(k) && node(k) != root) {
         const int p = (int)par(node(k));
         if (p < NS && (k < KR) != is_row(p))
           acc[k] = k < KR ? cell(node(k), p - MP) : cell(p, node(k) - MP);
       }
     }
-    return jump(acc, [&](int y) -> float& { return pot(y); });
+    return jump(acc, [&](int y) -> T& { return pot(y); });
   }
 
   // Most negative reduced cost of the tile (ties to the smallest cell
   // key (a << 8) | r); key INT_MAX if none is negative.
-  __device__ __forceinline__ void price(bool act, float& best, int& key) {
-    best = 0.f;
+  __device__ __forceinline__ void price(bool act, T& best, int& key) {
+    best = T(0);
     key = INT_MAX;
     if (act && gl < nb) {
       int brow = -1;
-      const float4 v = pot4((MP >> 2) + gl);
-      const float2 nv0 = make_float2(-v.x, -v.y), nv1 = make_float2(-v.z, -v.w);
-      const char* tp = sp + Sh::kTile + (4 * rg * nb + gl) * PS;
-      const int step = nb * PS;
+      const V4<T> v = potq((MP >> 2) + gl);
+      const char* at = tp(4 * rg, gl);
+      const int step = nb * (PS * (Sh::TS / 4));
       for (int a = 4 * rg; a < m; a += 4 * RS) {
-        const float4 u = pot4(a >> 2);
-        const float uu[4] = {u.x, u.y, u.z, u.w};
+        const V4<T> u = potq(a >> 2);
+        const T uu[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float4 c = *reinterpret_cast<const float4*>(tp + i * step);
-          const float2 nu = make_float2(-uu[i], -uu[i]);
-          const float2 d0 = __fadd2_rn(__fadd2_rn(make_float2(c.x, c.y), nu), nv0);
-          const float2 d1 = __fadd2_rn(__fadd2_rn(make_float2(c.z, c.w), nu), nv1);
-          const float lo = fminf(fminf(d0.x, d0.y), fminf(d1.x, d1.y));
+          const V4<T> c = ld4(at + i * step);
+          T lo;
+          if constexpr (Sh::TS == 4) {  // two columns an instruction
+            const float2 nu = make_float2(-uu[i], -uu[i]);
+            const float2 d0 = __fadd2_rn(__fadd2_rn(make_float2(c.x, c.y), nu),
+                                         make_float2(-v.x, -v.y));
+            const float2 d1 = __fadd2_rn(__fadd2_rn(make_float2(c.z, c.w), nu),
+                                         make_float2(-v.z, -v.w));
+            lo = fminf(fminf(d0.x, d0.y), fminf(d1.x, d1.y));
+          } else {
+            lo = fmin(fmin(c.x - uu[i] - v.x, c.y - uu[i] - v.y),
+                      fmin(c.z - uu[i] - v.z, c.w - uu[i] - v.w));
+          }
           if (lo < best) { best = lo; brow = a + i; }
         }
-        tp += 4 * RS * step;
+        at += 4 * RS * step;
       }
       if (brow >= 0) {
-        const float4 c = tile4(brow, gl);
-        const float u = pot(brow);
+        const V4<T> c = ld4(tp(brow, gl));
+        const T u = pot(brow);
         int r = 3;
         if (c.z - u - v.z == best) r = 2;
         if (c.y - u - v.y == best) r = 1;
@@ -626,22 +728,22 @@ struct Lane {
   }
 
   // Bland's rule: the smallest cell with reduced cost below -tol.
-  __device__ void price_bland(bool act, float tol, float& best, int& key) {
-    best = 0.f;
+  __device__ void price_bland(bool act, T tol, T& best, int& key) {
+    best = T(0);
     key = INT_MAX;
     if (act && gl < nb) {
       for (int a = 0; a < m && key == INT_MAX; ++a) {
         if ((a >> 2) % RS != rg) continue;
         for (int i = 0; i < 4 && key == INT_MAX; ++i) {
           const int r = 4 * gl + i;
-          const float d = cell(a, r) - pot(a) - pot(MP + r);
+          const T d = cell(a, r) - pot(a) - pot(MP + r);
           if (d < -tol) { best = d; key = (a << 8) | r; }
         }
       }
     }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(kAll, best, o * PW);
+      const T ov = __shfl_xor_sync(kAll, best, o * PW);
       const int ok = __shfl_xor_sync(kAll, key, o * PW);
       if (ok < key) { best = ov; key = ok; }
     }
@@ -669,7 +771,7 @@ struct Lane {
   // its subtree holds exactly one), and a node of the cut path hands its old
   // parent the edge between them.  At 64 x 64 a side's walk is about 11 steps
   // of dependent loads: 6.0 k cycles a pivot against 3.6 k for this form.
-  __device__ __forceinline__ int pivot_scan(bool act, int key, float dE) {
+  __device__ __forceinline__ int pivot_scan(bool act, int key, T dE) {
     const int ea = act ? key >> 8 : 0;
     const int eB = act ? MP + (key & 0xff) : MP;
     Mask<MW> mA, mB;
@@ -736,7 +838,7 @@ struct Lane {
       }
     }
     __syncwarp();
-    const float se = is_row(enode) ? dE : -dE;  // shift of a row's potential
+    const T se = is_row(enode) ? dE : -dE;  // shift of a row's potential
 #pragma unroll
     for (int k = 0; k < NPL; ++k) {
       const bool inS = ink(Sg, k);
@@ -755,7 +857,7 @@ struct Lane {
   // One pivot on entering cell `key` with reduced cost dE < 0.  Returns 1 if
   // flow moved, 0 if none did, -1 if the tree is inconsistent.  Lane 0 of the pair walks
   // the row side of the cycle, lane 1 the column side.
-  __device__ __forceinline__ int pivot(bool act, int key, float dE) {
+  __device__ __forceinline__ int pivot(bool act, int key, T dE) {
     const int ea = key >> 8, eB = MP + (key & 0xff);
     const bool walker = act && g < 2;
     const bool colside = (g & 1) != 0;
@@ -805,7 +907,7 @@ struct Lane {
     if (good) S = getD(zL);
     __syncwarp();
     // 2. potentials of the cut-off side
-    const float se = is_row(enode) ? dE : -dE;
+    const T se = is_row(enode) ? dE : -dE;
     Mask<MW> Sg;  // S seen from the own slots
 #pragma unroll
     for (int i = 0; i < MW; ++i) Sg.w[i] = S.w[i] >> g;
@@ -843,7 +945,8 @@ struct Lane {
   // Pivot until no reduced cost is below -tol.  Optimality is accepted on the
   // incrementally shifted potentials (the screen's error bound covers their
   // drift).  Returns kStOk, kStNotConverged or kStInvalid.
-  __device__ __forceinline__ int run(int max_pivots, float tol, int* pivots) {
+  // With fresh_stop it is accepted on potentials just recomputed only.
+  __device__ __forceinline__ int run(int max_pivots, T tol, int* pivots, bool fresh_stop = false) {
     int st = kStOk;
     int done = 0, degen = 0, since = 64;
     bool bland = false, open = live;
@@ -857,22 +960,29 @@ struct Lane {
         if (due) since = 0;
         if (maxu(due && b ? 1u : 0u)) { st = kStInvalid; open = false; }
       }
-      float dE;
+      T dE;
       int key;
       price(open && !bland, dE, key);
       if (__any_sync(kAll, open && bland)) {
-        float d2;
+        T d2;
         int k2;
         price_bland(open && bland, tol, d2, k2);
         if (bland) { dE = d2; key = k2; }
       }
-      if (open && !(dE < -tol && key != INT_MAX)) open = false;
+      bool none = open && !(dE < -tol && key != INT_MAX);
+      if (fresh_stop && none && since > 0) {  // once more on fresh potentials
+        none = false;
+        since = 64;
+        key = INT_MAX;
+      }
+      if (none) open = false;
       if (open && done >= max_pivots) { st = kStNotConverged; open = false; }
       if (!__any_sync(kAll, open)) break;
+      const bool go = open && key != INT_MAX;
       int moved;
-      if constexpr (G >= 16) moved = pivot_scan(open, key, dE);
-      else moved = pivot(open, key, dE);
-      if (open) {
+      if constexpr (G >= 16) moved = pivot_scan(go, go ? key : 0, dE);
+      else moved = pivot(go, go ? key : 0, dE);
+      if (go) {
         if (moved < 0) {
           st = kStInvalid;
           open = false;
@@ -1053,7 +1163,7 @@ __device__ __forceinline__ float4 lane_col_means(const Lane<Sh>& P) {
 template <class Sh>
 __device__ __forceinline__ float lane_tile(const Lane<Sh>& P, const ObjView& ob, long long o0,
                                            const CentView& cv, long long c0, const float* tile_g,
-                                           long long ldc, float4& vm) {
+                                           long long ldc, V4<float>& vm) {
   float cmax;
   if (tile_g) {  // made ahead by the tensor cores: rows of 16 B where aligned
     if (((reinterpret_cast<uintptr_t>(tile_g) | (uintptr_t)(ldc * 4)) & 15) == 0 &&
@@ -1113,7 +1223,8 @@ __device__ __forceinline__ float lane_tile(const Lane<Sh>& P, const ObjView& ob,
     }
   }
   cmax = Lane<Sh>::maxf(cmax);
-  vm = lane_col_means(P);  // the lane's own cells
+  const float4 mean = lane_col_means(P);  // the lane's own cells
+  vm = V4<float>{mean.x, mean.y, mean.z, mean.w};
   __syncwarp();
   return cmax;
 }
@@ -1396,7 +1507,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       }
       nxm = Lane<Sh>::maxf(nxm);
     }
-    float4 vm;
+    V4<float> vm;
     const float cmax = lane_tile<Sh>(P, ob, o0, cv, c0, tile_g, cfg.tile.ldc, vm);
     bool wbad = false;  // a saved basis that is not a feasible tree
     if constexpr (WARM) {
@@ -1524,6 +1635,29 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
   if (lane == 0) add_stats(n_scr, p_scr, 0, 0, n_cert, n_chk);
 }
 
+// Basis flows of the tree in shared memory as records (one entry
+// per node but the root, in node order).
+template <class Sh>
+__device__ __forceinline__ void lane_flows(const Lane<Sh>& P, int* fc, double* fw,
+                                           long long stride) {
+  constexpr int MP = Sh::MP;
+  const int rc = P.root < MP ? P.root : P.root - MP + P.m;
+#pragma unroll
+  for (int k = 0; k < Sh::NPL; ++k) {
+    const int y = P.node(k);
+    if (P.nodek(k) && y != P.root) {
+      const int p = (int)P.par(y);
+      const int e = k < Sh::KR ? y : y - MP + P.m;
+      fc[e < rc ? e : e - 1] = k < Sh::KR ? (y << 16) | (p - MP) : (p << 16) | (y - MP);
+      fw[e < rc ? e : e - 1] = (double)P.flowk(k) * kInvMass;
+    }
+  }
+  for (long long e = P.N - 1 + P.g; e < stride; e += Sh::G) {
+    fc[e] = -1;
+    fw[e] = 0.0;
+  }
+}
+
 // ---- the exact pass --------------------------------------------------------
 
 // Exact value of one pair from the basis the screen saved: the basic cells'
@@ -1550,7 +1684,7 @@ __device__ __forceinline__ int lane_verify(Lane<Sh>& P, bool go, bool value, cha
   double worst = 0.0;  // most negative reduced cost below -tol
   int wkey = INT_MAX;
   P.live = full;
-  float4 vm;
+  V4<float> vm;
   const float cmax = lane_tile<Sh>(P, ob, o0, cv, c0, nullptr, 0, vm);
   // basic cells in FP64
   double edge[NPL];
@@ -1683,10 +1817,10 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     bool fallback = have && (nc == -1 || nc == 0);
     if (!have || nc < 1) { nc = 0; P.m = 1; }
     double d64c = NAN;
-    if (cfg.certify && nc == 1)
+    if ((cfg.certify || cfg.mode == 0) && nc == 1)
       d64c = __longlong_as_double(((long long)mr[2 + kCandCap] << 32) |
                                   (long long)(unsigned)mr[1 + kCandCap]);
-    const bool known = !isnan(d64c);
+    const bool known = cfg.mode == 0 || !isnan(d64c);  // (FP64 throughout: always)
     double best = NAN;
     int best_j = -1;
     for (int c = 0; __any_sync(kAll, c < nc); ++c) {
@@ -1787,23 +1921,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
         best = D;
         best_j = mr[1 + c];
         if (X.fo.cell) {  // basis flows: one entry per node but the root
-          int* fc = X.fo.cell + i * X.fo.stride;
-          double* fw = X.fo.w + i * X.fo.stride;
-          const int rc = P.root < MP ? P.root : P.root - MP + P.m;
-#pragma unroll
-          for (int k = 0; k < NPL; ++k) {
-            const int y = P.node(k);
-            if (P.nodek(k) && y != P.root) {
-              const int p = (int)P.par(y);
-              const int e = k < Sh::KR ? y : y - MP + P.m;
-              fc[e < rc ? e : e - 1] = k < Sh::KR ? (y << 16) | (p - MP) : (p << 16) | (y - MP);
-              fw[e < rc ? e : e - 1] = (double)P.flowk(k) * kInvMass;
-            }
-          }
-          for (long long e = P.N - 1 + P.g; e < X.fo.stride; e += Sh::G) {
-            fc[e] = -1;
-            fw[e] = 0.0;
-          }
+          lane_flows<Sh>(P, X.fo.cell + i * X.fo.stride, X.fo.w + i * X.fo.stride, X.fo.stride);
         }
       }
       __syncwarp();
@@ -1819,6 +1937,313 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
         if (invalid) atomicOr(X.err, kErrInvalid);
       }
     }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    n_ex += __shfl_xor_sync(kAll, n_ex, o);
+    p_ex += __shfl_xor_sync(kAll, p_ex, o);
+  }
+  if (lane == 0) add_stats(0, 0, n_ex, p_ex);
+}
+
+// ---- pair lists, and FP64 throughout ---------------------------------------
+
+// FP64 tile, its largest cost and its column means (the arithmetic of
+// cost64_cell).
+template <class Sh>
+__device__ __forceinline__ double lane_tile64(const Lane<Sh>& P, const ObjView& ob, long long o0,
+                                              const CentView& cv, long long c0, V4<double>& vm) {
+  double cmax = 0.0;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  if (P.live && P.gl < P.nb) {
+    const int mq = (P.m + 3) >> 2;
+    for (int q = P.rg; q < mq; q += Sh::RS) {
+#pragma unroll 1
+      for (int a = 4 * q; a < 4 * q + 4; ++a) {
+        double c[4];
+        const double p = a < P.m ? (double)P.flow(a) * kInvMass : 0.0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int r = 4 * P.gl + j;
+          c[j] = INFINITY;
+          if (a < P.m && r < P.n) {
+            c[j] = cost64_cell(ob, o0, cv, c0, a, r);
+            cmax = c[j] > cmax ? c[j] : cmax;
+            v[j] = fma(p, c[j], v[j]);
+          }
+        }
+        P.st4(P.tp(a, P.gl), V4<double>{c[0], c[1], c[2], c[3]});
+      }
+    }
+  }
+#pragma unroll
+  for (int o = Sh::G / 2; o >= Sh::L; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o * Sh::PW);
+#pragma unroll
+  for (int o = Sh::G / 2; o > 0; o >>= 1) {
+    const double w = __shfl_xor_sync(0xffffffffu, cmax, o * Sh::PW);
+    cmax = w > cmax ? w : cmax;
+  }
+  vm = V4<double>{v[0], v[1], v[2], v[3]};
+  __syncwarp();
+  return cmax;
+}
+
+// Masses, singleton sets and zero potentials of a pair (m, n, live set); the
+// object's weights are quantised here.  Returns false for a rejected bag.
+template <class Sh>
+__device__ __forceinline__ bool lane_load(Lane<Sh>& P, bool act, const ObjView& ob, long long o0,
+                                          const CentView& cv, long long c0) {
+#pragma unroll
+  for (int k = 0; k < Sh::NPL; ++k) {
+    const int y = P.node(k);
+    long long w = 0;
+    Mask<Sh::MW> d;
+    d.clear();
+    if (act && P.nodek(k)) {
+      d.set(y);
+      if (k >= Sh::KR) {
+        const int r = y - Sh::MP;
+        w = cv.Qpre[c0 + r] - (r > 0 ? cv.Qpre[c0 + r - 1] : 0LL);
+      }
+    }
+    P.store(y, w, d, 0xffu);
+    P.potk(k) = 0;
+  }
+  __syncwarp();
+  const bool ok = ob.wdt == 0 ? P.row_masses(act, static_cast<const double*>(ob.w) + o0)
+                              : P.row_masses(act, static_cast<const float*>(ob.w) + o0);
+  __syncwarp();
+  return ok;
+}
+
+// The masses and singleton sets again, the tree kept.
+template <class Sh>
+__device__ __forceinline__ void lane_reset(Lane<Sh>& P, bool on, const ObjView& ob, long long o0,
+                                           const CentView& cv, long long c0) {
+  __syncwarp();
+#pragma unroll 1
+  for (int k = 0; k < Sh::NPL; ++k) {
+    const int y = P.node(k);
+    if (!on) continue;
+    long long w = 0;
+    Mask<Sh::MW> one;
+    one.clear();
+    if (y < Sh::MP ? y < P.m : y - Sh::MP < P.n) {
+      one.set(y);
+      if (y >= Sh::MP) {
+        const int r = y - Sh::MP;
+        w = cv.Qpre[c0 + r] - (r > 0 ? cv.Qpre[c0 + r - 1] : 0LL);
+      }
+    }
+    P.store(y, w, one, P.par(y));
+  }
+  __syncwarp();
+  if (ob.wdt == 0) P.row_masses(on, static_cast<const double*>(ob.w) + o0, on);
+  else P.row_masses(on, static_cast<const float*>(ob.w) + o0, on);
+  __syncwarp();
+}
+
+// FP64 throughout: start, pivots and objective on the FP64 tile.
+template <class Sh>
+__device__ __forceinline__ int lane_solve64(Lane<Sh>& P, const ObjView& ob, long long o0,
+                                            const CentView& cv, long long c0, int budget,
+                                            double* D, int* piv) {
+  V4<double> vm;
+  const double cmax = lane_tile64<Sh>(P, ob, o0, cv, c0, vm);
+  P.start_rows(vm);
+  const int st = P.run(budget * P.N, tol64(cmax), piv, true);
+  long long fl[Sh::NPL];
+#pragma unroll
+  for (int k = 0; k < Sh::NPL; ++k) {
+    fl[k] = P.flowk(k);
+    const int y = P.node(k);
+    double t = 0.0;
+    if (P.live && P.nodek(k) && y != P.root) {
+      const int p = (int)P.par(y);
+      if (p < Sh::NS && (k < Sh::KR) != (p < Sh::MP))
+        t = ((double)fl[k] * kInvMass) *
+            (k < Sh::KR ? P.cell(y, p - Sh::MP) : P.cell(p, y - Sh::MP));
+    }
+    if (P.live && P.nodek(k)) *reinterpret_cast<double*>(&P.flowk(k)) = t;
+  }
+  *D = P.sum_nodes();
+#pragma unroll
+  for (int k = 0; k < Sh::NPL; ++k) P.flowk(k) = fl[k];
+  __syncwarp();
+  return st;
+}
+
+// Listed pairs, one pass: FP32 shapes solve in FP32, then verify and repair in
+// FP64 as the exact pass does; FP64 shapes solve in FP64 throughout.  done[t]:
+// the pair's results are written (0: left to the warp-per-pair kernel).
+template <class Sh>
+__global__ void __launch_bounds__(64, Sh::kMinBlocks)
+    k_lane_pairs(ObjView ob, CentView cv, PairJob J, SolveCfg cfg, int nb, int warp_bytes) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int PW = Sh::PW;
+  char* warp_base = reinterpret_cast<char*>(smem) + (threadIdx.x >> 5) * warp_bytes;
+  Lane<Sh> P(warp_base, nb);
+  char* pot64 = warp_base + warp_bytes - (Sh::NS / 2) * Sh::PS + (P.sp - warp_base);
+  const int lane = threadIdx.x & 31;
+  int n_ex = 0, p_ex = 0;
+  const long long step = (long long)gridDim.x * (blockDim.x >> 5) * PW;
+  for (long long t0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PW;
+       t0 < J.npairs; t0 += step) {
+    const long long t = t0 + (lane & (PW - 1));
+    bool act = false;
+    long long o0 = 0, c0 = 0;
+    P.m = P.n = 1;
+    if (t < J.npairs) {
+      const long long i = J.pobj[t], j = J.pcen[t];
+      if (i >= 0 && i < ob.count && j >= 0 && j < cv.K) {
+        o0 = ob.off[i];
+        c0 = cv.off[j];
+        const long long mm = ob.off[i + 1] - o0, nn = cv.off[j + 1] - c0;
+        act = mm >= 1 && mm <= cfg.mmax && nn >= 1 && nn <= cfg.nmax;
+        if (act) {
+          P.m = (int)mm;
+          P.n = (int)nn;
+        }
+      }
+    }
+    P.N = P.m + P.n;
+    P.live = act;
+    P.root = 0;
+    __syncwarp();
+    act = lane_load<Sh>(P, act, ob, o0, cv, c0);
+    P.live = act;
+    double D = NAN;
+    int st = kStInvalid, piv = 0;
+    if constexpr (Sh::TS == 8) {
+      st = lane_solve64<Sh>(P, ob, o0, cv, c0, cfg.budget, &D, &piv);
+    } else {
+      V4<float> vm;
+      const float cmax = lane_tile<Sh>(P, ob, o0, cv, c0, nullptr, 0, vm);
+      P.start_rows(vm);
+      const int s32 = P.run(cfg.budget * P.N, tol32(cmax), &piv);
+      // the basis in FP64, pivots while it is not optimal there
+      bool todo = act && s32 == kStOk;
+      bool good = false;
+      for (int att = 0; att < 24; ++att) {
+        lane_reset<Sh>(P, todo, ob, o0, cv, c0);
+        int key;
+        float dE;
+        const int v = lane_verify<Sh>(P, todo, true, pot64, ob, o0, cv, c0, &D, &key, &dE);
+        if (todo && v == 0) good = true;
+        todo = todo && v == 1;
+        if (!__any_sync(kAll, todo)) break;
+        lane_reset<Sh>(P, todo, ob, o0, cv, c0);
+        P.live = todo;
+        P.template from_parents<true>();
+        int moved;
+        if constexpr (Sh::G >= 16) moved = P.pivot_scan(todo, todo ? key : 0, dE);
+        else moved = P.pivot(todo, todo ? key : 0, dE);
+        if (todo && moved < 0) todo = false;
+        if (todo) ++piv;
+      }
+      P.live = act;
+      st = good ? kStOk : kStInvalid;
+    }
+    if (act && P.g == 0) {
+      ++n_ex;
+      p_ex += piv;
+    }
+    const bool write = act && (Sh::TS == 8 ? st != kStInvalid : st == kStOk);
+    if (t < J.npairs && P.g == 0) {
+      J.done[t] = write ? 1 : 0;
+      if (write) {
+        J.dist2[t] = D;
+        if (J.status) J.status[t] = st == kStOk ? 0 : -3;
+        if (st == kStNotConverged) atomicOr(J.err, kErrNotConverged);
+      }
+    }
+    if (write && J.fo.cell) lane_flows<Sh>(P, J.fo.cell + t * J.fo.stride, J.fo.w + t * J.fo.stride, J.fo.stride);
+    __syncwarp();
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    n_ex += __shfl_xor_sync(kAll, n_ex, o);
+    p_ex += __shfl_xor_sync(kAll, p_ex, o);
+  }
+  if (lane == 0) add_stats(0, 0, n_ex, p_ex);
+}
+
+// Every pair of the chunk in FP64 throughout: its value (rec) and basis (tree).
+template <class Sh>
+__global__ void __launch_bounds__(64, Sh::kMinBlocks)
+    k_lane_all64(ObjView ob, CentView cv, long long seg_size, int K, SolveCfg cfg, LaneArgs A,
+                 long long total_obj, int* err) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int PW = Sh::PW;
+  Lane<Sh> P(reinterpret_cast<char*>(smem) + (threadIdx.x >> 5) * A.warp_bytes, A.nb);
+  const int lane = threadIdx.x & 31;
+  long long first, cnt;
+  lane_chunk(A, total_obj, &first, &cnt);
+  const long long total = cnt * (long long)K;
+  int n_ex = 0, p_ex = 0;
+  const long long step = (long long)gridDim.x * (blockDim.x >> 5) * PW;
+  for (long long q0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PW;
+       q0 < total; q0 += step) {
+    const long long q = q0 + (lane & (PW - 1));
+    bool act = q < total;
+    long long i = 0, o0 = 0, c0 = 0;
+    int j = 0;
+    P.m = P.n = 1;
+    if (act) {
+      const long long tt = q / K;
+      j = (int)(q - tt * K);
+      i = A.oidx ? (long long)A.oidx[first + tt] : A.obase + first + tt;
+      o0 = ob.off[i];
+      const long long mm = ob.off[i + 1] - o0;
+      const long long cb = seg_of(ob, i, seg_size) * (long long)K;
+      act = mm >= 1 && mm <= cfg.mmax && cb + K <= cv.K && !A.obad[i];
+      if (act) {
+        c0 = cv.off[cb + j];
+        const long long nn = cv.off[cb + j + 1] - c0;
+        act = nn >= 1 && nn <= cfg.nmax;
+        if (act) {
+          P.m = (int)mm;
+          P.n = (int)nn;
+        }
+      }
+    }
+    P.N = P.m + P.n;
+    P.live = act;
+    P.root = 0;
+    __syncwarp();
+    act = lane_load<Sh>(P, act, ob, o0, cv, c0);
+    P.live = act;
+    double D = NAN;
+    int piv = 0;
+    const int st = lane_solve64<Sh>(P, ob, o0, cv, c0, cfg.budget, &D, &piv);
+    if (act && P.g == 0) {
+      ++n_ex;
+      p_ex += piv;
+      if (st == kStInvalid) atomicOr(err, kErrInvalid);
+      if (st == kStNotConverged) atomicOr(err, kErrNotConverged);
+    }
+    if (act && A.tree) {
+      unsigned char* tr = A.tree + (unsigned long long)q * A.tstride;
+#pragma unroll
+      for (int k = 0; k < Sh::NPL; ++k) {
+        if (P.nodek(k)) {
+          const int y = P.node(k);
+          const unsigned p = P.par(y);
+          tr[k < Sh::KR ? y : y - Sh::MP + P.m] = (unsigned char)(
+              y == P.root ? 0xffu : (p < (unsigned)Sh::MP ? p : p - Sh::MP + P.m));
+        }
+      }
+    }
+    if (q < total && P.g == 0) {
+      PairRec r;
+      r.lo = r.hi = 0.f;
+      r.d64 = act && st != kStInvalid ? D : NAN;
+      A.rec[q] = r;
+      if (cfg.pair64) cfg.pair64[i * (long long)K + j] = r.d64;
+    }
+    __syncwarp();
   }
   for (int o = 16; o > 0; o >>= 1) {
     n_ex += __shfl_xor_sync(kAll, n_ex, o);
@@ -1846,6 +2271,7 @@ template <class Sh>
 cudaError_t lane_launch(const ObjView& ob, const CentView& cv, long long seg_size, int K,
                         const SolveCfg& cfg, LaneArgs A, long long total_obj, long long work,
                         const ExactOut& X, cudaStream_t st) {
+  if (cfg.mode == 0 && !X.labels) return cudaErrorInvalidValue;  // lane_all64_launch
   A.nb = (cfg.nmax + 3) / 4;
   if (cfg.mmax > Sh::MP || A.nb > Sh::L) return cudaErrorInvalidConfiguration;
   A.warp_bytes = (int)lane_warp_bytes<Sh>(cfg.mmax, A.nb);
@@ -1862,6 +2288,35 @@ cudaError_t lane_launch(const ObjView& ob, const CentView& cv, long long seg_siz
   if (A.by_pair)
     return cfg.certify ? screen(k_lane_screen<Sh, true, true>) : screen(k_lane_screen<Sh, false, true>);
   return cfg.certify ? screen(k_lane_screen<Sh, true, false>) : screen(k_lane_screen<Sh, false, false>);
+}
+
+// Every pair of the chunk in FP64 throughout.
+template <class Sh>
+cudaError_t lane_all64_launch(const ObjView& ob, const CentView& cv, long long seg_size, int K,
+                              const SolveCfg& cfg, LaneArgs A, long long total_obj, long long work,
+                              const ExactOut& X, cudaStream_t st) {
+  using S8 = LaneShape<Sh::G, Sh::L, Sh::MW, Sh::NPL, double>;
+  A.nb = (cfg.nmax + 3) / 4;
+  if (cfg.mmax > S8::MP || A.nb > S8::L) return cudaErrorInvalidConfiguration;
+  A.warp_bytes = (int)lane_warp_bytes<S8>(cfg.mmax, A.nb);
+  return lane_blocks(k_lane_all64<S8>, A.warp_bytes, cfg.sms, (work + S8::PW - 1) / S8::PW, st, ob,
+                     cv, seg_size, K, cfg, A, total_obj, X.err);
+}
+
+// The shape's pair-list kernel, FP32 with the exact test or FP64 throughout.
+template <class Sh>
+cudaError_t lane_pairs_launch(const ObjView& ob, const CentView& cv, const PairJob& J,
+                              const SolveCfg& cfg, cudaStream_t st) {
+  const int nb = (cfg.nmax + 3) / 4;
+  if (cfg.mmax > Sh::MP || nb > Sh::L) return cudaErrorInvalidConfiguration;
+  const long long warps = (J.npairs + Sh::PW - 1) / Sh::PW;
+  if (cfg.mode == 0) {
+    using S8 = LaneShape<Sh::G, Sh::L, Sh::MW, Sh::NPL, double>;
+    const int wb = (int)lane_warp_bytes<S8>(cfg.mmax, nb);
+    return lane_blocks(k_lane_pairs<S8>, wb, cfg.sms, warps, st, ob, cv, J, cfg, nb, wb);
+  }
+  const int wb = (int)lane_warp_bytes<Sh>(cfg.mmax, nb) + Sh::NS / 2 * Sh::PS;
+  return lane_blocks(k_lane_pairs<Sh>, wb, cfg.sms, warps, st, ob, cv, J, cfg, nb, wb);
 }
 
 }  // namespace

@@ -433,6 +433,7 @@ __global__ void __launch_bounds__(128) k_mallows_pairs(ObjView ob, CentView cv,
   int n_pairs = 0, n_piv = 0;
   for (long long t = (long long)blockIdx.x * gpb + threadIdx.x / G; t < npairs;
        t += (long long)gridDim.x * gpb) {
+    if (cfg.done && cfg.done[t]) continue;  // solved by lanes
     const long long i = pobj[t], j = pcen[t];
     int st = kStInvalid;
     double res = nan("");
@@ -1500,7 +1501,7 @@ static cudaError_t mallows_pairs_g(const ObjView& ob, const CentView& cv, const 
   if (gpb == 0) return cudaErrorInvalidConfiguration;
   const size_t smem = slice * gpb;
   unsigned grid = 1;
-  if (cfg.mode == 1 && cfg.tree &&
+  if (cfg.mode == 1 && cfg.tree && !cfg.done &&
       cfg.tree_bytes >= pair_tree_bytes(npairs, cfg.mmax, cfg.nmax)) {
     const int ns = cfg.mmax + cfg.nmax;
     const size_t nodes = (size_t)npairs * ns;
