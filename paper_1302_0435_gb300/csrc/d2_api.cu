@@ -286,10 +286,13 @@ int attach_tree(d2_ctx* c, SolveCfg* cfg, long long npairs, int slot = kPairTree
   return D2_OK;
 }
 
-// A pair list solved by lanes: its flag byte per pair.  (A caller that fixed a
-// cold-start rule keeps the warp-per-pair kernels.)
+// A pair list solved by lanes: its flag byte per pair.  A caller that fixed a
+// cold-start rule keeps the warp-per-pair kernels, and so does a list whose
+// pairs all have a warp of their own at once: there a call is one pair's
+// latency, and a pair that shares its warp with seven others takes longer (48
+// image pairs 30 us against 42; 6,000 uneven ones 837 us against 488).
 int attach_done(d2_ctx* c, SolveCfg* cfg, long long npairs) {
-  if (!cfg->lanes || npairs <= 0) return D2_OK;
+  if (!cfg->lanes || npairs < 24LL * c->sms) return D2_OK;
   int rc = D2_OK;
   cfg->done = static_cast<unsigned char*>(grow(c, kPairDone, (size_t)npairs, &rc));
   return rc;
@@ -1251,9 +1254,8 @@ int d2_mallows_batch(d2_ctx* c, const d2_bags* objs, const int64_t* pair_obj, co
   }
   if ((rc = check_bag_symbols(c, v))) return rc;
   SolveCfg cfg = solve_cfg(c, mode_for(c, objs->loc_dtype), mmax);
-  if (cfg.lanes) rc = attach_done(c, &cfg, npairs);
-  else rc = attach_tree(c, &cfg, npairs);
-  if (rc != D2_OK) return rc;
+  if ((rc = attach_done(c, &cfg, npairs)) || (!cfg.done && (rc = attach_tree(c, &cfg, npairs))))
+    return rc;
   CK(d2k::mallows_pairs(v, resident_view(c), po, pc, npairs, cfg, dd, fo, ds, c->d_err, c->stream));
   if (h1) CK(cudaMemcpyAsync(dist2, dd, (size_t)npairs * 8, cudaMemcpyDeviceToHost, c->stream));
   if (h2) CK(cudaMemcpyAsync(status, ds, (size_t)npairs * 4, cudaMemcpyDeviceToHost, c->stream));

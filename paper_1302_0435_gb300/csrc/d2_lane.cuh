@@ -274,6 +274,7 @@ struct Lane {
     return k < KR ? g + G * k < m : g + G * k - MP < n;
   }
   __device__ __forceinline__ static bool is_row(int y) { return y < MP; }
+  __device__ __forceinline__ bool has_node(int y) const { return y < MP ? y < m : y - MP < n; }
   // tile cell of the edge (y, p)
   __device__ __forceinline__ float edge_cost(int y, int p) const {
     return is_row(y) ? cell(y, p - MP) : cell(p, y - MP);
@@ -508,6 +509,7 @@ struct Lane {
       x[k] = node(k);
       if (live && nodek(k)) going |= 1u << k;
     }
+#pragma unroll 1
     for (int it = 0; it < NS && going; ++it) {
 #pragma unroll
       for (int k = 0; k < NPL; ++k) {
@@ -558,7 +560,9 @@ struct Lane {
 #pragma unroll
     for (int w = 0; w < MW; ++w) rest.w[w] = 0u;
     if (live) {
+#pragma unroll 1
       for (int y = 0; y < m; ++y) rest.set(y);
+#pragma unroll 1
       for (int y = 0; y < n; ++y) rest.set(MP + y);
     }
     long long p = 0, q = 0;
@@ -584,6 +588,7 @@ struct Lane {
       p -= f;
       q -= f;
     }
+#pragma unroll 1
     for (int s = 2;; ++s) {
       const bool act = live && s < N;
       if (!__any_sync(kAll, act)) break;
@@ -639,6 +644,7 @@ struct Lane {
         else cd[k] = p | 128u;
       }
     }
+#pragma unroll 1
     for (int round = 0; round < 9; ++round) {  // depth < 128: at most 8
       __syncwarp();
 #pragma unroll
@@ -692,6 +698,7 @@ struct Lane {
       const V4<T> v = potq((MP >> 2) + gl);
       const char* at = tp(4 * rg, gl);
       const int step = nb * (PS * (Sh::TS / 4));
+#pragma unroll 1
       for (int a = 4 * rg; a < m; a += 4 * RS) {
         const V4<T> u = potq(a >> 2);
         const T uu[4] = {u.x, u.y, u.z, u.w};
@@ -732,8 +739,10 @@ struct Lane {
     best = T(0);
     key = INT_MAX;
     if (act && gl < nb) {
+#pragma unroll 1
       for (int a = 0; a < m && key == INT_MAX; ++a) {
         if ((a >> 2) % RS != rg) continue;
+#pragma unroll 1
         for (int i = 0; i < 4 && key == INT_MAX; ++i) {
           const int r = 4 * gl + i;
           const T d = cell(a, r) - pot(a) - pot(MP + r);
@@ -801,6 +810,7 @@ struct Lane {
     th = min64(th);
     int tkey = INT_MAX;
     if (own == th && th != LLONG_MAX) {
+#pragma unroll 1
       for (unsigned t = tk; t; t &= t - 1) {
         const int y = node(__ffs((int)t) - 1), p = (int)par(y);
         const int kk = ((is_row(y) ? (y << 8) | (p - MP) : (p << 8) | (y - MP)) << 7) | y;
@@ -873,6 +883,7 @@ struct Lane {
     if (walker) {
       int x = x0;
       lost = true;
+#pragma unroll 1
       for (int it = 0; it < NS; ++it) {
         long long f;
         Mask<MW> D;
@@ -922,6 +933,7 @@ struct Lane {
       long long carry = th;
       Mask<MW> dprev;
       dprev.clear();
+#pragma unroll 1
       for (int it = 0; it < NS; ++it) {
         long long f;
         Mask<MW> D;
@@ -1009,39 +1021,38 @@ __device__ __forceinline__ float lane_cost_small(const Lane<Sh>& P, const float*
                                                  const float* __restrict__ y) {
   float cmax = 0.f;
   if (!P.live || P.gl >= P.nb) return cmax;
-  float yv[4][D];
+  float2 y0[D], y1[D];  // columns 0, 1 and 2, 3, negated
+  const int r0 = 4 * P.gl, last = P.n - 1;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int r = min(4 * P.gl + j, P.n - 1);
-#pragma unroll
-    for (int k = 0; k < D; ++k) yv[j][k] = __ldg(y + r * D + k);
+  for (int k = 0; k < D; ++k) {
+    y0[k] = make_float2(-__ldg(y + min(r0, last) * D + k), -__ldg(y + min(r0 + 1, last) * D + k));
+    y1[k] = make_float2(-__ldg(y + min(r0 + 2, last) * D + k),
+                        -__ldg(y + min(r0 + 3, last) * D + k));
   }
   const int mq = (P.m + 3) >> 2;
-  for (int q = P.rg; q < mq; q += Sh::RS) {
+#pragma unroll 1
+  for (int a = 4 * P.rg; a < 4 * mq; a += (a & 3) == 3 ? 4 * Sh::RS - 3 : 1) {
+    float4 c = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+    if (a < P.m) {
+      float2 c0 = make_float2(0.f, 0.f), c1 = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int a = 4 * q + i;
-      float c[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-      if (a < P.m) {
-        float xv[D];
-#pragma unroll
-        for (int k = 0; k < D; ++k) xv[k] = __ldg(x + a * D + k);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float acc = 0.f;
-#pragma unroll
-          for (int k = 0; k < D; ++k) {
-            const float df = xv[k] - yv[j][k];
-            acc = fmaf(df, df, acc);
-          }
-          if (4 * P.gl + j < P.n) {
-            c[j] = acc;
-            cmax = acc > cmax ? acc : cmax;
-          }
-        }
+      for (int k = 0; k < D; ++k) {
+        const float xv = __ldg(x + a * D + k);
+        const float2 xx = make_float2(xv, xv);
+        const float2 d0 = __fadd2_rn(xx, y0[k]), d1 = __fadd2_rn(xx, y1[k]);
+        c0 = __ffma2_rn(d0, d0, c0);
+        c1 = __ffma2_rn(d1, d1, c1);
       }
-      P.tile4(a, P.gl) = make_float4(c[0], c[1], c[2], c[3]);
+      c.x = r0 <= last ? c0.x : INFINITY;
+      c.y = r0 + 1 <= last ? c0.y : INFINITY;
+      c.z = r0 + 2 <= last ? c1.x : INFINITY;
+      c.w = r0 + 3 <= last ? c1.y : INFINITY;
+      cmax = r0 <= last && c0.x > cmax ? c0.x : cmax;
+      cmax = r0 + 1 <= last && c0.y > cmax ? c0.y : cmax;
+      cmax = r0 + 2 <= last && c1.x > cmax ? c1.x : cmax;
+      cmax = r0 + 3 <= last && c1.y > cmax ? c1.y : cmax;
     }
+    P.tile4(a, P.gl) = c;
   }
   return cmax;
 }
@@ -1057,6 +1068,7 @@ __device__ __forceinline__ float lane_cost_any(const Lane<Sh>& P, const X* __res
   const float* yp[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) yp[j] = y + (long long)min(4 * P.gl + j, P.n - 1) * d;
+#pragma unroll 1
   for (int q = P.rg; q < mq; q += Sh::RS) {
     const X* xp[4];
 #pragma unroll
@@ -1066,6 +1078,7 @@ __device__ __forceinline__ float lane_cost_any(const Lane<Sh>& P, const X* __res
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 1
     for (int k = 0; k < d; k += V) {
       float xv[4][V], yv[4][V];
 #pragma unroll
@@ -1111,6 +1124,7 @@ __device__ __forceinline__ float lane_cost_from(const Lane<Sh>& P, F f) {
   float cmax = 0.f;
   if (!P.live || P.gl >= P.nb) return cmax;
   const int mq = (P.m + 3) >> 2;
+#pragma unroll 1
   for (int q = P.rg; q < mq; q += Sh::RS) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1135,18 +1149,14 @@ template <class Sh>
 __device__ __forceinline__ float4 lane_col_means(const Lane<Sh>& P) {
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (P.live && P.gl < P.nb) {
-    for (int a = 4 * P.rg; a < P.m; a += 4 * Sh::RS) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (a + i < P.m) {
-          const float p = (float)P.flow(a + i) * (float)kInvMass;
-          const float4 c = P.tile4(a + i, P.gl);
-          v.x = fmaf(p, c.x, v.x);
-          v.y = fmaf(p, c.y, v.y);
-          v.z = fmaf(p, c.z, v.z);
-          v.w = fmaf(p, c.w, v.w);
-        }
-      }
+#pragma unroll 1
+    for (int a = 4 * P.rg; a < P.m; a += (a & 3) == 3 ? 4 * Sh::RS - 3 : 1) {
+      const float p = (float)P.flow(a) * (float)kInvMass;
+      const float4 c = P.tile4(a, P.gl);
+      v.x = fmaf(p, c.x, v.x);
+      v.y = fmaf(p, c.y, v.y);
+      v.z = fmaf(p, c.z, v.z);
+      v.w = fmaf(p, c.w, v.w);
     }
   }
 #pragma unroll
@@ -1171,6 +1181,7 @@ __device__ __forceinline__ float lane_tile(const Lane<Sh>& P, const ObjView& ob,
       cmax = 0.f;
       if (P.live && P.gl < P.nb && 4 * P.gl < P.n) {
         const int mq = (P.m + 3) >> 2;
+#pragma unroll 1
         for (int q = P.rg; q < mq; q += Sh::RS) {
           float4 c[4];
 #pragma unroll
@@ -1187,7 +1198,9 @@ __device__ __forceinline__ float lane_tile(const Lane<Sh>& P, const ObjView& ob,
         }
       } else if (P.live && P.gl < P.nb) {
         const int mq = (P.m + 3) >> 2;
+#pragma unroll 1
         for (int q = P.rg; q < mq; q += Sh::RS)
+#pragma unroll 1
           for (int i = 0; i < 4; ++i)
             P.tile4(4 * q + i, P.gl) = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
       }
@@ -1283,19 +1296,19 @@ __device__ __forceinline__ bool lane_certify(Lane<Sh>& P, bool go, const ObjView
   for (int k = 0; k < NPL; ++k) delta[k] = go && P.nodek(k) ? P.aux(P.node(k)) : 0.f;
   bad |= P.jump(delta, [&](int y) -> float& { return P.aux(y); });  // corrections
   unsigned pm = 0u, dm = 0u;
-#pragma unroll
+#pragma unroll 1
   for (int k = 0; k < NPL; ++k) {
     const int y = P.node(k);
-    if (go && P.nodek(k)) {
-      const float b = P.potk(k);
-      *reinterpret_cast<float2*>(&P.flowk(k)) = make_float2(b, delta[k]);
-      const float u = b + delta[k];
-      P.potk(k) = u;
+    if (go && P.has_node(y)) {
+      const float b = P.pot(y), dl = P.aux(y);  // (aux holds the sums jump ended with)
+      *reinterpret_cast<float2*>(&P.flow(y)) = make_float2(b, dl);
+      const float u = b + dl;
+      P.pot(y) = u;
       pm = max(pm, __float_as_uint(fabsf(u)));
-      dm = max(dm, __float_as_uint(fabsf(delta[k])));
+      dm = max(dm, __float_as_uint(fabsf(dl)));
       if (y != P.root && !bad) {
         const int p = (int)P.par(y);
-        if (k < Sh::KR) P.cell(y, p - MP) = INFINITY;
+        if (y < MP) P.cell(y, p - MP) = INFINITY;
         else P.cell(p, y - MP) = INFINITY;
       }
     }
@@ -1321,6 +1334,7 @@ __device__ __forceinline__ bool lane_certify(Lane<Sh>& P, bool go, const ObjView
   const int mq = (P.m + 3) >> 2;
   if (col) {
     v = P.pot4((MP >> 2) + P.gl);
+#pragma unroll 1
     for (int q = P.rg; q < mq; q += Sh::RS) {
       const float4 u4 = P.pot4(q);
       const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
@@ -1338,7 +1352,9 @@ __device__ __forceinline__ bool lane_certify(Lane<Sh>& P, bool go, const ObjView
     // pass 2 (few pairs): the flagged cells re-priced in double-float
     int cnt = 0;
     if (flagged) {
+#pragma unroll 1
       for (int q = P.rg; q < mq; q += Sh::RS) {
+#pragma unroll 1
         for (int t = 0; t < 16; ++t) {
           const int a = 4 * q + (t >> 2), r = 4 * P.gl + (t & 3);
           if (a >= P.m || r >= P.n) continue;
@@ -1393,6 +1409,7 @@ __device__ __forceinline__ void lane_order(Lane<Sh>& P, const LaneArgs& A, bool 
       if (P.live && P.nodek(k)) {
         const float* y = y32 + (P.node(k) - MP) * d;
         float dot = 0.f;
+#pragma unroll 1
         for (int t = 0; t < d; ++t) dot = fmaf(__ldg(y + t) - __ldg(mu + t), __ldg(dir + t), dot);
         P.potk(k) = dot;
       }
@@ -1411,6 +1428,7 @@ __device__ __forceinline__ void lane_order(Lane<Sh>& P, const LaneArgs& A, bool 
         const int r = y - MP;
         const float v = P.potk(k);
         int rank = 0;
+#pragma unroll 1
         for (int b = 0; b < P.n; ++b) {
           const float u = P.pot(MP + b);
           rank += (u < v || (u == v && b < r)) ? 1 : 0;
@@ -1476,15 +1494,15 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     if (!P.live) P.m = P.n = 1;
     P.N = P.m + P.n;
     // masses, singleton masks, potentials of the unused slots
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < NPL; ++k) {
       const int y = P.node(k);
       long long w = 0;
       Mask<Sh::MW> d;
       d.clear();
-      if (P.live && P.nodek(k)) {
+      if (P.live && P.has_node(y)) {
         d.set(y);
-        if (k < Sh::KR) {
+        if (y < Sh::MP) {
           w = A.omass[i * A.mstride + y];
         } else {
           const int r = y - Sh::MP;
@@ -1501,6 +1519,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       if (P.live) {
         const long long trow0 = cfg.tile.trow[tt];
         tile_g = cfg.tile.C + trow0 * cfg.tile.ldc + (c0 - cfg.tile.col0);
+#pragma unroll 1
         for (int a = P.g; a < P.m; a += Sh::G) nxm = fmaxf(nxm, cfg.tile.nx[trow0 + a]);
       } else {
         tile_g = cfg.tile.C;
@@ -1557,12 +1576,12 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     if (A.tree && P.live) {  // the basis, for the exact pass (parents, compact node numbers)
       unsigned char* tr = A.tree + (WARM ? (unsigned long long)(i * (long long)K + j) : q) *
                                        (unsigned long long)A.tstride;
-#pragma unroll
+#pragma unroll 1
       for (int k = 0; k < NPL; ++k) {
-        if (P.nodek(k)) {
-          const int y = P.node(k);
+        const int y = P.node(k);
+        if (P.has_node(y)) {
           const unsigned p = P.par(y);
-          tr[k < Sh::KR ? y : y - Sh::MP + P.m] =
+          tr[y < Sh::MP ? y : y - Sh::MP + P.m] =
               (unsigned char)(y == P.root || st == kStInvalid
                                   ? 0xffu
                                   : (p < (unsigned)Sh::MP ? p : p - Sh::MP + P.m));
@@ -1593,12 +1612,12 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     } else {
       // FP32 objective and its error bound
       float acc = 0.f;
-#pragma unroll
+#pragma unroll 1
       for (int k = 0; k < NPL; ++k) {
         const int y = P.node(k);
-        if (P.live && P.nodek(k) && y != P.root) {
+        if (P.live && P.has_node(y) && y != P.root) {
           const int p = (int)P.par(y);
-          if (p < Sh::NS) acc += ((float)P.flowk(k) * (float)kInvMass) * P.edge_cost(y, p);
+          if (p < Sh::NS) acc += ((float)P.flow(y) * (float)kInvMass) * P.edge_cost(y, p);
         }
       }
       const float D = Lane<Sh>::sum(acc);
@@ -1626,6 +1645,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     }
     __syncwarp();
   }
+#pragma unroll 1
   for (int o = 16; o > 0; o >>= 1) {
     n_scr += __shfl_xor_sync(kAll, n_scr, o);
     p_scr += __shfl_xor_sync(kAll, p_scr, o);
@@ -1652,6 +1672,7 @@ __device__ __forceinline__ void lane_flows(const Lane<Sh>& P, int* fc, double* f
       fw[e < rc ? e : e - 1] = (double)P.flowk(k) * kInvMass;
     }
   }
+#pragma unroll 1
   for (long long e = P.N - 1 + P.g; e < stride; e += Sh::G) {
     fc[e] = -1;
     fw[e] = 0.0;
@@ -1732,6 +1753,7 @@ __device__ __forceinline__ int lane_verify(Lane<Sh>& P, bool go, bool value, cha
   if (full && P.gl < P.nb) {
     const float4 v = P.pot4((MP >> 2) + P.gl);
     const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll 1
     for (int a = 4 * P.rg; a < 4 * mq; a += (a & 3) == 3 ? 4 * Sh::RS - 3 : 1) {
       const float u = P.pot(a);
       const float4 c = P.tile4(a, P.gl);
@@ -1739,6 +1761,7 @@ __device__ __forceinline__ int lane_verify(Lane<Sh>& P, bool go, bool value, cha
       unsigned flag = 0u;
 #pragma unroll
       for (int t = 0; t < 4; ++t) flag |= !(cc[t] - u - vv[t] >= E) ? 1u << t : 0u;
+#pragma unroll 1
       for (; flag; flag &= flag - 1) {
         const int r = 4 * P.gl + __ffs((int)flag) - 1;
         if (a < P.m && r < P.n) {
@@ -1798,6 +1821,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
   lane_chunk(A, total_obj, &first, &cnt);
   int n_ex = 0, p_ex = 0;
   const long long step = (long long)gridDim.x * (blockDim.x >> 5) * PW;
+#pragma unroll 1
   for (long long t0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PW; t0 < cnt;
        t0 += step) {
     const long long t = t0 + (lane & (PW - 1));
@@ -1823,6 +1847,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     const bool known = cfg.mode == 0 || !isnan(d64c);  // (FP64 throughout: always)
     double best = NAN;
     int best_j = -1;
+#pragma unroll 1
     for (int c = 0; __any_sync(kAll, c < nc); ++c) {
       const bool go = c < nc && !fallback && (!known || X.fo.cell);
       int j = 0;
@@ -1838,6 +1863,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
         } else if (A.list) {  // the pair's place in the list: kept centroids before j
           const unsigned* kb = cfg.keep + i * cfg.keep_words;
           q = X.ostart[t] + __popc(kb[j >> 5] & ((1u << (j & 31)) - 1u));
+#pragma unroll 1
           for (int w = 0; w < (j >> 5); ++w) q += __popc(kb[w]);
         } else {
           q = (unsigned long long)t * (unsigned)K + (unsigned)j;
@@ -1890,6 +1916,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       double D = d64c;
       bool todo = go;
       int verdict = go ? 2 : 0;
+#pragma unroll 1
       for (int att = 0; att < 24; ++att) {
         masses(todo);
         int key;
@@ -1938,6 +1965,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       }
     }
   }
+#pragma unroll 1
   for (int o = 16; o > 0; o >>= 1) {
     n_ex += __shfl_xor_sync(kAll, n_ex, o);
     p_ex += __shfl_xor_sync(kAll, p_ex, o);
@@ -1956,6 +1984,7 @@ __device__ __forceinline__ double lane_tile64(const Lane<Sh>& P, const ObjView& 
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   if (P.live && P.gl < P.nb) {
     const int mq = (P.m + 3) >> 2;
+#pragma unroll 1
     for (int q = P.rg; q < mq; q += Sh::RS) {
 #pragma unroll 1
       for (int a = 4 * q; a < 4 * q + 4; ++a) {
@@ -2089,6 +2118,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
   const int lane = threadIdx.x & 31;
   int n_ex = 0, p_ex = 0;
   const long long step = (long long)gridDim.x * (blockDim.x >> 5) * PW;
+#pragma unroll 1
   for (long long t0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PW;
        t0 < J.npairs; t0 += step) {
     const long long t = t0 + (lane & (PW - 1));
@@ -2126,6 +2156,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       // the basis in FP64, pivots while it is not optimal there
       bool todo = act && s32 == kStOk;
       bool good = false;
+#pragma unroll 1
       for (int att = 0; att < 24; ++att) {
         lane_reset<Sh>(P, todo, ob, o0, cv, c0);
         int key;
@@ -2162,6 +2193,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     if (write && J.fo.cell) lane_flows<Sh>(P, J.fo.cell + t * J.fo.stride, J.fo.w + t * J.fo.stride, J.fo.stride);
     __syncwarp();
   }
+#pragma unroll 1
   for (int o = 16; o > 0; o >>= 1) {
     n_ex += __shfl_xor_sync(kAll, n_ex, o);
     p_ex += __shfl_xor_sync(kAll, p_ex, o);
@@ -2184,6 +2216,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
   const long long total = cnt * (long long)K;
   int n_ex = 0, p_ex = 0;
   const long long step = (long long)gridDim.x * (blockDim.x >> 5) * PW;
+#pragma unroll 1
   for (long long q0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PW;
        q0 < total; q0 += step) {
     const long long q = q0 + (lane & (PW - 1));
@@ -2245,6 +2278,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
     }
     __syncwarp();
   }
+#pragma unroll 1
   for (int o = 16; o > 0; o >>= 1) {
     n_ex += __shfl_xor_sync(kAll, n_ex, o);
     p_ex += __shfl_xor_sync(kAll, p_ex, o);

@@ -412,6 +412,7 @@ __device__ __forceinline__ double cost64_cell(const ObjView& ob, long long o0, c
   const double* y = cv.loc64 + (c0 + r) * d;
   const long long x0 = (o0 + a) * d;
   double acc = 0.0;
+#pragma unroll 1
   for (int k = 0; k < d; ++k) {
     const double df = ldx<double>(ob.loc, ob.ldt, x0 + k) - y[k];
     acc = fma(df, df, acc);
