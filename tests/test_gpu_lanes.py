@@ -93,3 +93,85 @@ def test_bins(d2, oracle_mod, n):
     cents = bags(rng, np.full(6, n), 4, "far")
     rows = np.sort(rng.choice(objs.count, size=120, replace=False))
     check(oracle_mod, objs, cents, run_all(d2, objs, cents), rows)
+
+
+def run_pairs(d2, objs, cents, po, pc, precision, flows=True):
+    import torch
+    ctx = d2.Context(0, precision=precision)
+    d2.d2_set_centroids(ctx, d2.bags_from_synth(cents, device="cuda:0"))
+    ob = d2.bags_from_synth(objs, device="cuda:0")
+    dist = torch.empty(len(po), dtype=torch.float64, device="cuda:0")
+    st = torch.full((len(po),), 9, dtype=torch.int32, device="cuda:0")
+    fl = (torch.empty((len(po), 127), dtype=torch.int32, device="cuda:0"),
+          torch.empty((len(po), 127), dtype=torch.float64, device="cuda:0"))
+    rc = d2.d2_mallows_batch(ctx, ob, torch.as_tensor(po, device="cuda:0"),
+                             torch.as_tensor(pc, device="cuda:0"), dist,
+                             flows=fl if flows else None, status=st)
+    assert rc == d2.D2_OK
+    d2.d2_sync(ctx)
+    ctx.close()
+    return dist.cpu().numpy(), st.cpu().numpy(), fl[0].cpu().numpy(), fl[1].cpu().numpy()
+
+
+@pytest.mark.parametrize("law", ["normal", "lattice"])
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("n,top", [(16, 16), (13, 48), (9, 64), (32, 16), (29, 32), (32, 64), (64, 64)])
+def test_pair_lists(d2, oracle_mod, n, top, precision, law):
+    """A list long enough for the lanes (24 pairs per SM of a 152-SM GPU), FP64
+    throughout and FP32 with the FP64 test: values to FP64 optimality
+    (2^-43 c_max plus rounding), plans that meet both marginals and cost D^2."""
+    rng = np.random.default_rng(7 * n + top + precision)
+    sizes = np.asarray([m for m in EDGES if m <= top] * 2)
+    objs = bags(rng, sizes, 5, law)
+    cents = bags(rng, np.full(4, n), 5, law)
+    if precision == 1:
+        objs = Bags(objs.loc.astype(np.float64), objs.w.astype(np.float64), objs.off, "f64", "f64")
+        cents = Bags(cents.loc.astype(np.float64), cents.w.astype(np.float64), cents.off, "f64",
+                     "f64")
+    N, K = objs.count, cents.count
+    t = 4096 + rng.integers(0, 9)
+    po, pc = rng.integers(0, N, size=t), rng.integers(0, K, size=t)
+    dist, st, cell, w = run_pairs(d2, objs, cents, po, pc, precision)
+    assert (st == 0).all()
+    _, _, ref = oracle_mod.assign(objs, cents, nthreads=8, return_all=True)
+    ref = ref[po, pc]
+    big = float(np.max(np.abs(objs.loc))) + float(np.max(np.abs(cents.loc)))
+    floor = 1e-12 * objs.dim * big * big
+    assert np.all(np.abs(dist - ref) <= 1e-11 * ref + floor)
+    for q in rng.choice(t, size=60, replace=False):
+        x, p = oracle_mod.bag(objs, int(po[q]))
+        y, r = oracle_mod.bag(cents, int(pc[q]))
+        ok = cell[q] >= 0
+        assert ok.sum() == len(p) + len(r) - 1
+        a, b, f = cell[q][ok] >> 16, cell[q][ok] & 0xFFFF, w[q][ok]
+        assert (f >= 0).all()
+        assert np.abs(np.bincount(a, weights=f, minlength=len(p)) - p / p.sum()).max() <= 1e-12
+        assert np.abs(np.bincount(b, weights=f, minlength=len(r)) - r / r.sum()).max() <= 1e-12
+        cost = float(np.dot(f, ((np.asarray(x)[a] - np.asarray(y)[b]) ** 2).sum(axis=1)))
+        assert abs(cost - dist[q]) <= 1e-11 * dist[q] + floor
+
+
+def test_pair_list_rejects_what_it_did(d2):
+    """Bad indices and bad weights in a long list keep their status and error."""
+    import torch
+    rng = np.random.default_rng(5)
+    objs = bags(rng, np.full(20, 8), 3, "normal")
+    objs.w[objs.off[3]] = -1.0
+    cents = bags(rng, np.full(4, 16), 3, "normal")
+    po, pc = rng.integers(0, 20, size=5000), rng.integers(0, 4, size=5000)
+    po[7], pc[9] = 20, -1
+    ctx = d2.Context(0)
+    d2.d2_set_centroids(ctx, d2.bags_from_synth(cents, device="cuda:0"))
+    ob = d2.bags_from_synth(objs, device="cuda:0")
+    dist = torch.empty(5000, dtype=torch.float64, device="cuda:0")
+    st = torch.empty(5000, dtype=torch.int32, device="cuda:0")
+    d2.d2_mallows_batch(ctx, ob, torch.as_tensor(po, device="cuda:0"),
+                        torch.as_tensor(pc, device="cuda:0"), dist, status=st)
+    with pytest.raises(d2.D2Error) as e:
+        d2.d2_sync(ctx)
+    assert e.value.code == d2.D2_EINVAL
+    bad = (po == 20) | (pc == -1) | (po == 3)
+    s, dd = st.cpu().numpy(), dist.cpu().numpy()
+    assert (s[bad] == -1).all() and np.isnan(dd[bad]).all()
+    assert (s[~bad] == 0).all() and np.isfinite(dd[~bad]).all()
+    ctx.close()
