@@ -163,11 +163,11 @@ def measured_peaks():
 
 
 def kernel_source_hash():
-    """Hash of the sources of the screening kernel's translation unit
-    (k_screen<32,1> is instantiated in d2_npl1.cu from these files)."""
+    """Hash of the sources of the screening kernel's translation units
+    (k_lane_screen's shapes are instantiated in d2_lane_*.cu from these files)."""
     h = hashlib.sha256()
     cs = os.path.join(ROOT, "paper_1302_0435_gb300", "csrc")
-    for f in ("d2_npl1.cu", "d2_solve.cuh", "d2_solver.cuh", "d2_internal.h"):
+    for f in ("d2_lane.cu", "d2_lane.cuh", "d2_solve.cuh", "d2_solver.cuh", "d2_internal.h"):
         with open(os.path.join(cs, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -177,7 +177,7 @@ def profiled_traffic(name):
     """DRAM bytes per launch of the screening kernel on workload `name`
     from the committed ncu summary, if it was taken on the current kernel
     sources (else None)."""
-    p = os.path.join(ROOT, "profiles", "k_screen_traffic.json")
+    p = os.path.join(ROOT, "profiles", "k_lane_screen_traffic.json")
     if not os.path.exists(p):
         return None
     with open(p) as f:
@@ -521,8 +521,8 @@ def measure_workload(name, d2, torch, dev, timer, sms, mhz, args, objs, cents, s
         cpu, sample = cpu_baseline(objs, cents, seconds=args.cpu_seconds, full=cpu_full)
         out["cpu_baseline"] = cpu
         out["error_vs_oracle"] = error_vs_oracle(gpu_all, sample)
-        kname = ("k_screen (certify) + k_merge + k_exact: cold d2_mallows_all" if not graph else
-                 "k_screen (certify) + k_merge + k_exact + update: the graph-replayed step")
+        kname = ("k_lane_screen (certify) + k_lane_merge + k_lane_exact: cold d2_mallows_all" if not graph else
+                 "k_lane_screen (certify) + k_lane_merge + k_lane_exact + update: the graph-replayed step")
         out["roofline"] = roofline_entry(kname, pairs, ta, cpu["ops_per_pair"], cpu["mean_pivots"],
                                          sms, mhz, profiled_traffic(name))
     return out
@@ -649,7 +649,7 @@ def run_ours(args):
     if not args.skip_cpu:
         cpu, sample = cpu_baseline(objs, cents, seconds=args.cpu_seconds)
         err = error_vs_oracle(gpu_all, sample)
-        roof = roofline_entry("k_screen (certify) + k_merge + k_exact: cold d2_mallows_all, "
+        roof = roofline_entry("k_lane_screen (certify) + k_lane_merge + k_lane_exact: cold d2_mallows_all, "
                               "200,000 x 64", k_pairs, k_sec, cpu["ops_per_pair"],
                               cpu["mean_pivots"], sms, mhz, profiled_traffic("image_like"))
         # the warm rounds as the step runs them: the GPU's own pivots
@@ -674,7 +674,7 @@ def run_ours(args):
             "uneven", d2, torch, dev, timer, sms, mhz, args, o3, c3, 2, 1,
             "uneven: N=1,000,000 bags, sizes P(m) ~ m^-2 on 2..64, d=16, FP32, Dirichlet(1); "
             "K=256 of 32 supports; all pairs + one location update, replayed from a CUDA graph "
-            "(autotuned tree-size bins, device-side bin ranges)", e2e_warm=False, graph=True)
+            "(support-count bins, device-side bin ranges)", e2e_warm=False, graph=True)
         del o3, c3
         o4, c4 = synth.high_dim()
         workloads["high_dim"] = measure_workload(
@@ -825,7 +825,7 @@ def run_profile_case(args):
     lanes = 32 if args.no_tune else 0  # a fixed launch shape: no autotuning launches
     if args.profile_workload == "image_level":
         # the benchmark step's level driver on profile_n bags (segments of
-        # 5,000, 10 rounds): k_screen launches after the first are warm
+        # 5,000, 10 rounds): k_lane_screen launches after the first are warm
         # rounds replayed from the CUDA graph
         objs, cents = synth.image_like(N=args.profile_n, K=WORKLOAD["K"])
         ctx = d2.Context(0, certify=cert)

@@ -30,9 +30,9 @@
  *    d2_mallows_batch, d2_assign, d2_mallows_all and d2_update_locations
  *    return without waiting when all their outputs are device pointers and
  *    their bags declare max_support (with 0, a scan of the offsets waits
- *    first); the first call of a new launch shape may also wait for the
- *    autotuner, and BF16 batches screened with tensor-core tiles wait for
- *    their bin counts.  Outputs are valid after d2_sync() or an event
+ *    first); with a cold-start rule fixed (start_rule), the first call of a
+ *    new launch shape may also wait for the autotuner, and BF16 batches
+ *    screened with tensor-core tiles wait for their bin counts.  Outputs are valid after d2_sync() or an event
  *    recorded on that stream.  A call with any host output waits before it
  *    returns; so do the other calls.
  *  - Errors of calls that return without waiting (bad offsets or weights,
@@ -92,10 +92,15 @@ extern "C" {
 #define D2_TC_ON 2    /* on for BF16 objects with dim a multiple of 16 in 16..256 */
 
 /* cold-start basis of the simplex (d2_config.start_rule) */
-#define D2_START_AUTO 0    /* the autotuner times both on large batches; otherwise
-                              Vogel for centroids of 64 supports, else RANKED */
-#define D2_START_RANKED 1  /* northwest staircase in principal-direction order */
-#define D2_START_VOGEL 2   /* Vogel's approximation (largest-penalty line first) */
+#define D2_START_AUTO 0    /* the lane solver (several pairs per warp) with its own
+                              start: rows in turn take the cheapest columns left, on
+                              costs less their column's mean.  What it does not take
+                              (short pair lists, d2_update_weights' members) starts
+                              by Vogel's rule for 64 supports, else RANKED */
+#define D2_START_RANKED 1  /* northwest staircase in principal-direction order, one
+                              warp per pair */
+#define D2_START_VOGEL 2   /* Vogel's approximation (largest-penalty line first), one
+                              warp per pair */
 
 /* centroid update of d2_cluster_level's rounds (d2_config.centroid_update) */
 #define D2_UPDATE_CONSTRAINED 0  /* Alg. 2 Step 3*: support weights fixed, locations by
@@ -154,12 +159,13 @@ typedef struct {
 typedef struct {
     int32_t precision;          /* D2_PREC_* ; 0 = AUTO */
     int32_t pivot_budget;       /* pivots per pair = pivot_budget*(m+n); 0 = 64 */
-    int32_t group_lanes;        /* lanes per pair: every pair is solved by one warp
-                                   (32 lanes, one tree node per lane and bin).
-                                   0 = the launch shape (threads per block, screening
-                                   items per SM, cold-start rule) is autotuned per
-                                   support bin on large batches; 32 = the default shape,
-                                   no tuning; other values are rejected (D2_EINVAL) */
+    int32_t group_lanes;        /* the warp-per-pair screen of a fixed start_rule:
+                                   0 = its launch shape (threads per block, screening
+                                   items per SM) is autotuned per support bin on large
+                                   batches; 32 = the default shape, no tuning; other
+                                   values are rejected (D2_EINVAL).  The lane solver of
+                                   D2_START_AUTO chooses its lanes per pair from the
+                                   sizes and is not tuned */
     int32_t cost_tc;            /* D2_TC_* ; 0 = AUTO */
     int32_t tile_budget_mib;    /* device memory for tensor-core cost tiles;
                                    0 = min(32 GiB, 40% of free memory) */
@@ -198,10 +204,11 @@ typedef struct {
                                    every round solves every member from a cold start */
     int32_t warm_budget_mib;    /* device memory d2_cluster_level may take for the bases it
                                    keeps between rounds; 0 = 40% of the free memory.  The
-                                   full store is 11 B per tree node and pair; when only its
-                                   trees fit (3 B per node) the flows are recomputed on
-                                   reload (same results, slower; not with
-                                   D2_CERTIFY_ALL); below that the rounds start cold */
+                                   store is 1 B per tree node and pair (the flows are
+                                   rebuilt on reload); with a fixed start_rule 11 B, or,
+                                   when only its trees fit, 3 B (same results, slower;
+                                   not with D2_CERTIFY_ALL); below that the rounds start
+                                   cold */
 } d2_config;
 
 /*

@@ -88,8 +88,9 @@ struct d2_ctx {
   int* d_err = nullptr;
   int* d_info = nullptr;
   int* h_pin = nullptr;  // pinned host ints
-  // autotuned launch per (nodes-per-lane bin, K, m bound, n bound, d, mode):
-  // threads per block, screening items per SM, cold-start rule
+  // autotuned launch of the warp-per-pair screen per (nodes-per-lane bin, K,
+  // m bound, n bound, d, mode): threads per block, screening items per SM,
+  // cold-start rule (the caller's: with none the lane screen runs, untuned)
   std::map<std::tuple<int, long long, int, int, int, int>, std::tuple<int, int, int>> tuned;
   int tuning_runs = 0;
 };
@@ -499,8 +500,6 @@ int size_cuts(bool lanes, long long count, int mmax, int nmax, int* cut) {
   return k;
 }
 
-// One assign over a batch, bin by bin (largest trees first), each bin with
-// its autotuned launch shape.  ws may be null.
 // Whether run_assign screens with pruning bits for these arguments.
 bool prunes(const d2_ctx* c, const SolveCfg& base, const CentView& cv) {
   return base.mode == 1 && !base.certify && !base.pair64 && cv.A == 0 && !c->cfg.no_prune;
@@ -623,8 +622,7 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
       t.pair64 = nullptr;
       // a sample of about 2^20 pairs, at least 256 objects: several waves of
       // warps, so the timing ranks throughput (a one-wave sample ranks the
-      // per-pair latency and favoured Vogel's start where the staircase is
-      // faster at scale)
+      // per-pair latency)
       t.nobj = std::min<long long>(cnt, std::max<long long>(256, (1LL << 20) / std::max(K, 1)));
       int rc = D2_OK;
       int* tl = static_cast<int*>(grow(c, kTuneLab, (size_t)v.count * 4, &rc));
@@ -643,17 +641,6 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
         cudaEventElapsedTime(ms, e0, e1);
         return D2_OK;
       };
-      // cold-start rule first (default shape), unless the caller fixed it
-      if (c->cfg.start_rule == D2_START_AUTO) {
-        float best_s = 1e30f;
-        for (int sr = 0; sr < 2; ++sr) {
-          t.start = sr;
-          float ms = 0.f;
-          if ((rc = time_one(t, &ms))) return rc;
-          if (ms < best_s) { best_s = ms; cfg.start = sr; }
-        }
-      }
-      t.start = cfg.start;
       float best = 1e30f;
       std::tuple<int, int, int> pick(128, 96, cfg.start);
       const int tpbs[2] = {64, 128};
@@ -1869,7 +1856,8 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     // Saved bases of all (object, centroid) pairs of this level: the rounds
     // re-solve the same pairs with the same marginals and moved centroid
     // locations, so each solve starts from its previous optimal basis.
-    // A basis is its tree (parent, preorder position and subtree size
+    // The lane screen keeps a byte per node (below).  For the warp-per-pair
+    // screen a basis is its tree (parent, preorder position and subtree size
     // bytes per node: 3 B) plus its int64 flows (8 B per node).  The flows
     // are the tree's basic solution for the pair's marginals, which the
     // rounds do not change, so when the whole store does not fit only the
