@@ -30,7 +30,7 @@
  *    d2_mallows_batch, d2_assign, d2_mallows_all and d2_update_locations
  *    return without waiting when all their outputs are device pointers and
  *    their bags declare max_support (with 0, a scan of the offsets waits
- *    first); with a cold-start rule fixed (start_rule), the first call of a
+ *    first); with a cold-start rule fixed (start_rule) the first call of a
  *    new launch shape may also wait for the autotuner, and BF16 batches
  *    screened with tensor-core tiles wait for their bin counts.  Outputs are valid after d2_sync() or an event
  *    recorded on that stream.  A call with any host output waits before it
@@ -95,8 +95,9 @@ extern "C" {
 #define D2_START_AUTO 0    /* the lane solver (several pairs per warp) with its own
                               start: rows in turn take the cheapest columns left, on
                               costs less their column's mean.  What it does not take
-                              (short pair lists, d2_update_weights' members) starts
-                              by Vogel's rule for 64 supports, else RANKED */
+                              (short pair lists, d2_update_weights' members, the
+                              rounds of a level without pruning that keeps bases)
+                              starts by Vogel's rule for 64 supports, else RANKED */
 #define D2_START_RANKED 1  /* northwest staircase in principal-direction order, one
                               warp per pair */
 #define D2_START_VOGEL 2   /* Vogel's approximation (largest-penalty line first), one
@@ -159,7 +160,8 @@ typedef struct {
 typedef struct {
     int32_t precision;          /* D2_PREC_* ; 0 = AUTO */
     int32_t pivot_budget;       /* pivots per pair = pivot_budget*(m+n); 0 = 64 */
-    int32_t group_lanes;        /* the warp-per-pair screen of a fixed start_rule:
+    int32_t group_lanes;        /* the warp-per-pair screen (a fixed start_rule, or a
+                                   level without pruning):
                                    0 = its launch shape (threads per block, screening
                                    items per SM) is autotuned per support bin on large
                                    batches; 32 = the default shape, no tuning; other
@@ -205,9 +207,10 @@ typedef struct {
     int32_t warm_budget_mib;    /* device memory d2_cluster_level may take for the bases it
                                    keeps between rounds; 0 = 40% of the free memory.  The
                                    store is 1 B per tree node and pair (the flows are
-                                   rebuilt on reload); with a fixed start_rule 11 B, or,
-                                   when only its trees fit, 3 B (same results, slower;
-                                   not with D2_CERTIFY_ALL); below that the rounds start
+                                   rebuilt on reload); without pruning 11 B where
+                                   that fits; with a fixed start_rule 11 B, or, when
+                                   only its trees fit, 3 B (same results, slower; not
+                                   with D2_CERTIFY_ALL); below that the rounds start
                                    cold */
 } d2_config;
 

@@ -90,7 +90,7 @@ struct d2_ctx {
   int* h_pin = nullptr;  // pinned host ints
   // autotuned launch of the warp-per-pair screen per (nodes-per-lane bin, K,
   // m bound, n bound, d, mode): threads per block, screening items per SM,
-  // cold-start rule (the caller's: with none the lane screen runs, untuned)
+  // cold-start rule
   std::map<std::tuple<int, long long, int, int, int, int>, std::tuple<int, int, int>> tuned;
   int tuning_runs = 0;
 };
@@ -622,7 +622,8 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
       t.pair64 = nullptr;
       // a sample of about 2^20 pairs, at least 256 objects: several waves of
       // warps, so the timing ranks throughput (a one-wave sample ranks the
-      // per-pair latency)
+      // per-pair latency and favoured Vogel's start where the staircase is
+      // faster at scale)
       t.nobj = std::min<long long>(cnt, std::max<long long>(256, (1LL << 20) / std::max(K, 1)));
       int rc = D2_OK;
       int* tl = static_cast<int*>(grow(c, kTuneLab, (size_t)v.count * 4, &rc));
@@ -641,6 +642,17 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
         cudaEventElapsedTime(ms, e0, e1);
         return D2_OK;
       };
+      // cold-start rule first (default shape), unless the caller fixed it
+      if (c->cfg.start_rule == D2_START_AUTO) {
+        float best_s = 1e30f;
+        for (int sr = 0; sr < 2; ++sr) {
+          t.start = sr;
+          float ms = 0.f;
+          if ((rc = time_one(t, &ms))) return rc;
+          if (ms < best_s) { best_s = ms; cfg.start = sr; }
+        }
+      }
+      t.start = cfg.start;
       float best = 1e30f;
       std::tuple<int, int, int> pick(128, 96, cfg.start);
       const int tpbs[2] = {64, 128};
@@ -1852,7 +1864,7 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     d2k::note_launches(1);
     CK(cudaGetLastError());
     CentView cv{l32, l64, lQ, loff, KT, d};
-    const SolveCfg cfg = solve_cfg(c, mode_for(c, cur.ldt), cur_mmax);
+    SolveCfg cfg = solve_cfg(c, mode_for(c, cur.ldt), cur_mmax);
     // Saved bases of all (object, centroid) pairs of this level: the rounds
     // re-solve the same pairs with the same marginals and moved centroid
     // locations, so each solve starts from its previous optimal basis.
@@ -1870,6 +1882,15 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     const size_t flow_bytes = (size_t)npairs * ns * 8;
     // (not with Alg. 1 updates: the weights, so every pair's supplies, change each round)
     const size_t budget = (cfg.mode == 1 && iters > 1 && !alg1) ? warm_budget_bytes(c) : 0;
+    // A level that is not pruned (certify-all, no_prune, a cost table)
+    // re-solves every pair every round, at 4.5 pivots from its saved basis:
+    // there reading flows or subtrees back beats rebuilding them by lanes (the
+    // certified image-like level of 200,000 bags 519 ms against 930), so with
+    // room for the bases its rounds keep a warp per pair.  With pruning only a
+    // few percent of the pairs are solved and the lanes win (78 against 47 ms).
+    const bool full = meta_bytes + flow_bytes <= budget;
+    if (!prunes(c, cfg, cv) && budget > 0 && (full || (meta_bytes <= budget && !cfg.certify)))
+      cfg.lanes = false;
     if (cfg.lanes) {
       // the lane screen keeps a basis as its parents, a byte a node, and
       // rebuilds flows and subtree sets as it loads them
