@@ -90,7 +90,7 @@ struct d2_ctx {
   int* h_pin = nullptr;  // pinned host ints
   // autotuned launch of the warp-per-pair screen per (nodes-per-lane bin, K,
   // m bound, n bound, d, mode): threads per block, screening items per SM,
-  // cold-start rule
+  // cold-start rule (the caller's)
   std::map<std::tuple<int, long long, int, int, int, int>, std::tuple<int, int, int>> tuned;
   int tuning_runs = 0;
 };
@@ -521,6 +521,39 @@ int prep_bags(d2_ctx* c, const ObjView& v, int mmax, bool moments) {
   return D2_OK;
 }
 
+// The keep bits of the objects of v (their moments are in place: prep_bags).
+int prune_bits(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, int K,
+               unsigned* was, unsigned** keep) {
+  int rc = D2_OK;
+  const int kw = (K + 31) / 32;
+  d2k::CentMoments cm;
+  cm.mu = static_cast<double*>(grow(c, kPrMuC, (size_t)cv.K * cv.d * 8, &rc));
+  cm.var = static_cast<double*>(grow(c, kPrVarC, (size_t)cv.K * 8, &rc));
+  cm.muT32 = static_cast<float*>(grow(c, kPrMuT, (size_t)cv.K * cv.d * 4, &rc));
+  cm.cn = static_cast<float*>(grow(c, kPrCn, (size_t)cv.K * 4, &rc));
+  cm.vb = static_cast<float2*>(grow(c, kPrVb, (size_t)cv.K * 8, &rc));
+  *keep = static_cast<unsigned*>(grow(c, kPrKeep, (size_t)v.count * kw * 4, &rc));
+  if (rc != D2_OK) return rc;
+  CK(d2k::cent_moments(cv, cm, c->stream));
+  CK(d2k::prune_keep(v, seg, K, cv.K, v.d, static_cast<const double*>(c->slot[kPrMuO].p),
+                     static_cast<const double*>(c->slot[kPrVarO].p), cm, *keep, kw, was,
+                     c->stream));
+  return D2_OK;
+}
+
+__global__ void __launch_bounds__(256) k_count_bits(const unsigned* w, int n, int* out) {
+  int s = 0;
+  for (int i = threadIdx.x; i < n; i += 256) s += __popc(w[i]);
+  s = __reduce_add_sync(0xffffffffu, s);
+  __shared__ int part[8];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) s += part[k];
+    *out = s;
+  }
+}
+
 int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, int K, int mode,
                int mmax, const double* om, int* lab, double* d2o, double* terms, FlowOut fo,
                int* cand, const d2k::WarmStore* ws, Bins& bins,
@@ -544,29 +577,18 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
     // the argmin: bounds from the bags' means and spreads, keep bits per object
     int rc = D2_OK;
     const int kw = (K + 31) / 32;
-    d2k::CentMoments cm;
-    cm.mu = static_cast<double*>(grow(c, kPrMuC, (size_t)cv.K * cv.d * 8, &rc));
-    cm.var = static_cast<double*>(grow(c, kPrVarC, (size_t)cv.K * 8, &rc));
-    cm.muT32 = static_cast<float*>(grow(c, kPrMuT, (size_t)cv.K * cv.d * 4, &rc));
-    cm.cn = static_cast<float*>(grow(c, kPrCn, (size_t)cv.K * 4, &rc));
-    cm.vb = static_cast<float2*>(grow(c, kPrVb, (size_t)cv.K * 8, &rc));
-    unsigned* keep = static_cast<unsigned*>(grow(c, kPrKeep, (size_t)v.count * kw * 4, &rc));
-    if (rc != D2_OK) return rc;
-    // a level's rounds keep the bits of the round before as well: the pairs
-    // whose bases that round saved
+    // a level's rounds by lanes keep the bits of the round before as well: the
+    // pairs whose bases that round saved
     unsigned* was = nullptr;
-    if (ws && base.lanes)
+    if (ws && !ws->pos8 && base.lanes)
       was = static_cast<unsigned*>(grow(c, kPrKeepWas, (size_t)v.count * kw * 4, &rc));
-    if (rc != D2_OK) return rc;
-    CK(d2k::cent_moments(cv, cm, c->stream));
-    CK(d2k::prune_keep(v, seg, K, cv.K, v.d, static_cast<const double*>(c->slot[kPrMuO].p),
-                       static_cast<const double*>(c->slot[kPrVarO].p), cm, keep, kw, was,
-                       c->stream));
+    unsigned* keep = nullptr;
+    if (rc != D2_OK || (rc = prune_bits(c, v, cv, seg, K, was, &keep))) return rc;
     base.keep = keep;
     base.keep_words = kw;
     base.keep_was = was;
   }
-  if (ws && base.lanes && !ws->warm && nmax <= 16) {
+  if (ws && !ws->pos8 && base.lanes && !ws->warm && nmax <= 16) {
     // the cold round of a level starts small trees from the ranked staircase
     int rc = D2_OK;
     base.rows = static_cast<unsigned char*>(grow(c, kPrRows, (size_t)v.count * mmax, &rc));
@@ -622,8 +644,7 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
       t.pair64 = nullptr;
       // a sample of about 2^20 pairs, at least 256 objects: several waves of
       // warps, so the timing ranks throughput (a one-wave sample ranks the
-      // per-pair latency and favoured Vogel's start where the staircase is
-      // faster at scale)
+      // per-pair latency)
       t.nobj = std::min<long long>(cnt, std::max<long long>(256, (1LL << 20) / std::max(K, 1)));
       int rc = D2_OK;
       int* tl = static_cast<int*>(grow(c, kTuneLab, (size_t)v.count * 4, &rc));
@@ -642,17 +663,6 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
         cudaEventElapsedTime(ms, e0, e1);
         return D2_OK;
       };
-      // cold-start rule first (default shape), unless the caller fixed it
-      if (c->cfg.start_rule == D2_START_AUTO) {
-        float best_s = 1e30f;
-        for (int sr = 0; sr < 2; ++sr) {
-          t.start = sr;
-          float ms = 0.f;
-          if ((rc = time_one(t, &ms))) return rc;
-          if (ms < best_s) { best_s = ms; cfg.start = sr; }
-        }
-      }
-      t.start = cfg.start;
       float best = 1e30f;
       std::tuple<int, int, int> pick(128, 96, cfg.start);
       const int tpbs[2] = {64, 128};
@@ -1882,15 +1892,35 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     const size_t flow_bytes = (size_t)npairs * ns * 8;
     // (not with Alg. 1 updates: the weights, so every pair's supplies, change each round)
     const size_t budget = (cfg.mode == 1 && iters > 1 && !alg1) ? warm_budget_bytes(c) : 0;
-    // A level that is not pruned (certify-all, no_prune, a cost table)
-    // re-solves every pair every round, at 4.5 pivots from its saved basis:
-    // there reading flows or subtrees back beats rebuilding them by lanes (the
-    // certified image-like level of 200,000 bags 519 ms against 930), so with
-    // room for the bases its rounds keep a warp per pair.  With pruning only a
-    // few percent of the pairs are solved and the lanes win (78 against 47 ms).
-    const bool full = meta_bytes + flow_bytes <= budget;
-    if (!prunes(c, cfg, cv) && budget > 0 && (full || (meta_bytes <= budget && !cfg.certify)))
-      cfg.lanes = false;
+    // this level's bags (masses, pruning moments), once for all its rounds
+    const bool pruned = prunes(c, cfg, cv);
+    if ((cfg.lanes || cfg.mode == 1) && (rc = prep_bags(c, cur, cur_mmax, pruned))) return rc;
+    // A round that solves most of its pairs from their saved bases (a level
+    // without pruning: certify-all, no_prune, a cost table; or bags that the
+    // bounds cannot tell apart) spends a few pivots on each, and reading flows
+    // or subtrees back beats rebuilding them by lanes: the certified
+    // image-like level of 200,000 bags 519 ms against 930, Gaussian bags with
+    // 42 % of the pairs kept 63 against 68, 10 % kept 126 against 82, 3 % kept
+    // 21 against 16.  So with room for the bases such rounds keep a warp per
+    // pair; with centroids of more than 32 supports the lanes win whatever is
+    // kept (587 against 330 ms).  The share that is kept is counted on the
+    // first objects, where the level has enough tree nodes (2^26: 7 ms and more)
+    // to pay for the count's wait.
+    const bool store = budget > 0 && (meta_bytes + flow_bytes <= budget ||
+                                      (meta_bytes <= budget && !cfg.certify));
+    if (cfg.lanes && store && !pruned) cfg.lanes = false;
+    if (cfg.lanes && store && c->nmax <= 32 && npairs * ns >= (1LL << 26)) {
+      ObjView first = cur;
+      first.count = std::min<long long>(cur.count, 2048);
+      unsigned* keep = nullptr;
+      if ((rc = prune_bits(c, first, cv, seg, K, nullptr, &keep))) return rc;
+      k_count_bits<<<1, 256, 0, c->stream>>>(keep, (int)(first.count * ((K + 31) / 32)), c->d_info);
+      d2k::note_launches(1);
+      CK(cudaGetLastError());
+      CK(cudaMemcpyAsync(c->h_pin, c->d_info, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+      CK(cudaStreamSynchronize(c->stream));
+      if (c->h_pin[0] > 0.3 * (double)first.count * K) cfg.lanes = false;
+    }
     if (cfg.lanes) {
       // the lane screen keeps a basis as its parents, a byte a node, and
       // rebuilds flows and subtree sets as it loads them
@@ -1915,9 +1945,6 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     }
     Bins bins;
     if (want_bins(c, cfg, n_l, cur_mmax) && (rc = make_bins(c, cur, &bins)))
-      return rc;
-    // this level's bags (masses, pruning moments), once for all its rounds
-    if ((cfg.lanes || cfg.mode == 1) && (rc = prep_bags(c, cur, cur_mmax, prunes(c, cfg, cv))))
       return rc;
     // Rounds 2.. repeat the same launches (same pairs, warm bases): round 1
     // is captured into a CUDA graph once and replayed.

@@ -175,3 +175,68 @@ def test_pair_list_rejects_what_it_did(d2):
     assert (s[bad] == -1).all() and np.isnan(dd[bad]).all()
     assert (s[~bad] == 0).all() and np.isfinite(dd[~bad]).all()
     ctx.close()
+
+
+def run_level(d2, objs, cents, iters, **kw):
+    import torch
+    ctx = d2.Context(0, **kw)
+    d2.d2_set_centroids(ctx, d2.bags_from_synth(cents, device="cuda:0"))
+    ob = d2.bags_from_synth(objs, device="cuda:0")
+    loc = torch.empty(cents.loc.shape, dtype=torch.float64, device="cuda:0")
+    w = torch.empty(cents.count, dtype=torch.float64, device="cuda:0")
+    lab = torch.empty(objs.count, dtype=torch.int32, device="cuda:0")
+    rc = d2.d2_cluster_level(ctx, ob, cents.count, objs.count, iters, loc, w, lab)
+    assert rc == d2.D2_OK
+    d2.d2_sync(ctx)
+    ctx.close()
+    return lab.cpu().numpy(), loc.cpu().numpy()
+
+
+@pytest.mark.parametrize("kw", [{}, {"no_prune": True}, {"certify": 1}])
+@pytest.mark.parametrize("N,lo,hi,n,K,law", [
+    (300, 2, 48, 32, 6, "normal"),      # trees of more than 32 nodes, most pairs kept
+    (300, 8, 16, 16, 6, "far"),         # few pairs kept: kept pairs without a saved basis
+    (200, 16, 64, 64, 5, "normal"),
+    (33000, 8, 16, 16, 64, "normal"),   # large enough that the kept share is counted
+    (33000, 8, 16, 16, 64, "far"),
+])
+def test_level_agrees_with_the_warp_screen(d2, N, lo, hi, n, K, law, kw):
+    """One segment of continuous bags: every LP has one optimal plan, so the
+    labels are equal and the locations are the same sums; two FP32 units
+    (2^-22) cover a stored location that rounds the other way.  A certified
+    plan is only within 2^-24 of the optimal cost, so two cold starts may end
+    in two of them: there the first round's labels are compared."""
+    rng = np.random.default_rng(N + n)
+    objs = bags(rng, rng.integers(lo, hi + 1, size=N), 6, law)
+    cents = bags(rng, np.full(K, n), 6, law)
+    for iters in (1,) if kw.get("certify") else (1, 4):
+        a = run_level(d2, objs, cents, iters, **kw)
+        b = run_level(d2, objs, cents, iters, start_rule=d2.D2_START_RANKED, **kw)
+        assert np.array_equal(a[0], b[0])
+        if kw.get("certify"):
+            continue
+        assert np.abs(a[1] - b[1]).max() <= 2.0 ** -22 * np.abs(b[1]).max()
+
+
+@pytest.mark.parametrize("law", ["normal", "lattice"])
+@pytest.mark.parametrize("n", [1, 16, 17, 32, 33, 64])
+def test_assign_fp64_throughout(d2, oracle_mod, n, law):
+    """FP64 assignments at the edges of their shapes, to FP64 optimality."""
+    import torch
+    rng = np.random.default_rng(31 * n + len(law))
+    objs = bags(rng, np.asarray(EDGES * 2), 5, law)
+    cents = bags(rng, np.asarray([n, max(1, n - 1), max(1, n // 2)]), 5, law)
+    ctx = d2.Context(0, precision=1)
+    d2.d2_set_centroids(ctx, d2.bags_from_synth(cents, device="cuda:0"))
+    lab = torch.empty(objs.count, dtype=torch.int32, device="cuda:0")
+    dist = torch.empty(objs.count, dtype=torch.float64, device="cuda:0")
+    assert d2.d2_assign(ctx, d2.bags_from_synth(objs, device="cuda:0"), lab, dist) == d2.D2_OK
+    d2.d2_sync(ctx)
+    ctx.close()
+    _, _, ref = oracle_mod.assign(objs, cents, nthreads=8, return_all=True)
+    big = float(np.max(np.abs(objs.loc))) + float(np.max(np.abs(cents.loc)))
+    floor = 1e-12 * objs.dim * big * big
+    best = ref.min(axis=1)
+    at = ref[np.arange(objs.count), lab.cpu().numpy()]
+    assert np.all(at <= best * (1 + 1e-11) + floor)
+    assert np.all(np.abs(dist.cpu().numpy() - at) <= 1e-11 * at + floor)
