@@ -1411,7 +1411,7 @@ __device__ __forceinline__ void lane_order(Lane<Sh>& P, const LaneArgs& A, bool 
         float dot = 0.f;
 #pragma unroll 1
         for (int t = 0; t < d; ++t) dot = fmaf(__ldg(y + t) - __ldg(mu + t), __ldg(dir + t), dot);
-        P.potk(k) = dot;
+        P.potk(k) = order_value(dot);
       }
     }
   }
