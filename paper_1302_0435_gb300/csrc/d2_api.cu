@@ -405,7 +405,9 @@ __global__ void k_merge_labels(const int* lab, long long n_l, long long seg, con
                                int K, int* ct) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_l;
        i += (long long)gridDim.x * blockDim.x)
-    ct[i] = lab[i] < 0 ? -1 : (int)((segof ? (long long)segof[i] : i / seg) * K + lab[i]);
+    ct[i] = lab[i] < 0 || lab[i] >= K
+                ? -1
+                : (int)((segof ? (long long)segof[i] : i / seg) * K + lab[i]);
 }
 __global__ void k_compose(int* C, long long N, const int* ct) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
@@ -468,6 +470,24 @@ int make_bins(d2_ctx* c, const ObjView& v, Bins* b) {
   b->binned = true;
   b->host = false;
   return D2_OK;
+}
+
+// The bags that are in no launch of a binned batch (no support, or more than
+// mmax): label -1, NaN for every distance, as a launch that holds such a bag
+// writes them.
+__global__ void k_reject_bags(const long long* off, long long N, int mmax, int K, int* labels,
+                              double* dist2, double* eps_terms, double* pair64, int* err) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long m = off[i + 1] - off[i];
+    if (m >= 1 && m <= mmax) continue;
+    labels[i] = -1;
+    dist2[i] = nan("");
+    if (eps_terms) eps_terms[i] = nan("");
+    if (pair64)
+      for (int j = 0; j < K; ++j) pair64[i * (long long)K + j] = nan("");
+    atomicOr(err, d2k::kErrInvalid);
+  }
 }
 
 int bins_to_host(d2_ctx* c, Bins* b) {
@@ -600,6 +620,10 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
     CK(d2k::assign(v, cv, seg, K, base, om, lab, d2o, terms, fo, cand, c->d_err, c->stream, ws, tw));
     return D2_OK;
   }
+  k_reject_bags<<<blocks_for(v.count), 256, 0, c->stream>>>(v.off, v.count, mmax, K, lab, d2o,
+                                                            terms, pair64, c->d_err);
+  d2k::note_launches(1);
+  CK(cudaGetLastError());
   // the lane screen has one launch shape per bound; the warp-per-pair screen
   // is tuned
   const bool lanes = base.lanes;
