@@ -582,6 +582,11 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
   const int nmax = std::max(c->nmax, 1);
   SolveCfg base = solve_cfg(c, mode, mmax);
   if (certify_all && mode == 1) base.certify = true;
+  // full saved bases are the warp-per-pair screen's: a level that keeps them
+  // takes that screen's cuts and tuned shapes (20,000 x 64 bags in trees of 34
+  // to 80 nodes, ten rounds of nearly every pair: 470 ms, by the lanes' cuts
+  // and untuned 488; certified 566 and 574)
+  if (ws && ws->pos8) base.lanes = false;
   base.pair64 = pair64;
   const bool prune = prunes(c, base, cv);
   if (prune || base.lanes) {
@@ -687,6 +692,17 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
         cudaEventElapsedTime(ms, e0, e1);
         return D2_OK;
       };
+      // cold-start rule first (default shape), unless the caller fixed it
+      if (c->cfg.start_rule == D2_START_AUTO) {
+        float best_s = 1e30f;
+        for (int sr = 0; sr < 2; ++sr) {
+          t.start = sr;
+          float ms = 0.f;
+          if ((rc = time_one(t, &ms))) return rc;
+          if (ms < best_s) { best_s = ms; cfg.start = sr; }
+        }
+      }
+      t.start = cfg.start;
       float best = 1e30f;
       std::tuple<int, int, int> pick(128, 96, cfg.start);
       const int tpbs[2] = {64, 128};

@@ -1,0 +1,76 @@
+"""Which screen a level's rounds run, and each of them against the others and
+the oracle."""
+import numpy as np
+import pytest
+
+from paper_1302_0435_gb300.synth import Bags
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def d2():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1302_0435_gb300 import build, d2 as mod
+    build.build()
+    mod.load()
+    return mod
+
+
+def bags(rng, sizes, d, spread=0.0):
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    T = int(off[-1])
+    loc = rng.normal(size=(T, d)) + np.repeat(rng.normal(0, spread, size=(len(sizes), d)), sizes,
+                                              axis=0)
+    return Bags(loc.astype(np.float32), rng.exponential(size=T).astype(np.float32), off, "f32",
+                "f32")
+
+
+def run_level(d2, objs, cents, iters, seg=None, **kw):
+    """Labels, locations and the change of the library's counters."""
+    import torch
+    ctx = d2.Context(0, **kw)
+    d2.d2_set_centroids(ctx, d2.bags_from_synth(cents, device="cuda:0"))
+    ob = d2.bags_from_synth(objs, device="cuda:0")
+    loc = torch.empty(cents.loc.shape, dtype=torch.float64, device="cuda:0")
+    w = torch.empty(cents.count, dtype=torch.float64, device="cuda:0")
+    lab = torch.empty(objs.count, dtype=torch.int32, device="cuda:0")
+    s0 = d2.d2_get_stats()
+    d2.d2_cluster_level(ctx, ob, cents.count, seg or objs.count, iters, loc, w, lab)
+    d2.d2_sync(ctx)
+    s1 = d2.d2_get_stats()
+    ctx.close()
+    return lab.cpu().numpy(), loc.cpu().numpy(), {k: s1[k] - s0[k] for k in s1}
+
+
+@pytest.mark.parametrize("kw", [{"no_prune": True}, {"certify": 1}])
+@pytest.mark.parametrize("tuned", [False, True])
+@pytest.mark.parametrize("n,top", [(32, 48), (16, 64)])
+def test_level_of_full_bases_runs_as_the_warp_screen(d2, n, top, tuned, kw):
+    """An unpruned level that keeps full bases solves a warp per pair: the same
+    launches (cuts by tree size, and where nothing fixes the launch shape its
+    timing) and the same bits as with the cold start fixed."""
+    rng = np.random.default_rng(n + top)
+    objs = bags(rng, rng.integers(2, top + 1, size=9000), 5, 1.0)
+    cents = bags(rng, np.full(6, n), 5, 1.0)
+    kw = dict(kw, group_lanes=0 if tuned else 32)
+    a = run_level(d2, objs, cents, 4, **kw)
+    b = run_level(d2, objs, cents, 4, start_rule=d2.D2_START_RANKED, **kw)
+    assert a[2]["kernel_launches"] == b[2]["kernel_launches"]
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+def test_level_of_full_bases_is_tuned(d2):
+    """Its bins of 8,192 objects and more are timed on the first round; two
+    starts of continuous bags end in the one optimal plan (the labels are
+    equal, the locations differ by FP32 units)."""
+    rng = np.random.default_rng(8)
+    objs = bags(rng, rng.integers(2, 49, size=20000), 5, 1.0)
+    cents = bags(rng, np.full(6, 32), 5, 1.0)
+    a = run_level(d2, objs, cents, 3, no_prune=True)
+    b = run_level(d2, objs, cents, 3, no_prune=True, group_lanes=32)
+    assert a[2]["kernel_launches"] > b[2]["kernel_launches"]
+    assert np.array_equal(a[0], b[0])
+    assert np.abs(a[1] - b[1]).max() <= 2.0 ** -22 * np.abs(b[1]).max()
