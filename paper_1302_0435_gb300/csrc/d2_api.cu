@@ -291,9 +291,13 @@ int attach_tree(d2_ctx* c, SolveCfg* cfg, long long npairs, int slot = kPairTree
 // cold-start rule keeps the warp-per-pair kernels, and so does a list whose
 // pairs all have a warp of their own at once: there a call is one pair's
 // latency, and a pair that shares its warp with seven others takes longer (48
-// image pairs 30 us against 42; 6,000 uneven ones 837 us against 488).
+// image pairs 30 us against 42; 6,000 uneven ones 837 us against 488).  Small
+// trees in FP64 are behind for longer, the FP64 pipe being what the lanes of a
+// warp share (8 x 8 supports: 3,700 pairs 150 us by warps, 206 by lanes, 10,000
+// 259 and 261, 64,000 1,214 and 1,040).
 int attach_done(d2_ctx* c, SolveCfg* cfg, long long npairs) {
-  if (!cfg->lanes || npairs < 24LL * c->sms) return D2_OK;
+  const bool small64 = cfg->mode == 0 && cfg->mmax <= 16 && cfg->nmax <= 16;
+  if (!cfg->lanes || npairs < (small64 ? 64LL : 24LL) * c->sms) return D2_OK;
   int rc = D2_OK;
   cfg->done = static_cast<unsigned char*>(grow(c, kPairDone, (size_t)npairs, &rc));
   return rc;

@@ -130,6 +130,13 @@ struct Lane {
   int g, gl, rg;    // lane in the pair, its column lane, its row group
   int m, n, N, root;
   bool live;
+  int cand;         // kList: the lane's best cell of the last full scan (INT_MAX: none)
+  // FP64 pricing by candidates: the scan of a tile costs the FP64 pipe (a 64th
+  // of the FP32 rate) 12 operations per 4 cells, so a pivot first takes the
+  // best of the lanes' cells of the last scan at the current potentials, and
+  // the tile is scanned when a pair of the warp has none left.
+  // (64,000 pairs in FP64: 64 x 64 182 -> 80 ms, 32 x 32 35 -> 27)
+  static constexpr bool kList = Sh::TS == 8 && Sh::G >= 8;
 
   __device__ __forceinline__ Lane(char* warp_base, int nb_) : nb(nb_) {
     const int lane = threadIdx.x & 31;
@@ -731,6 +738,21 @@ struct Lane {
         key = (brow << 8) | (4 * gl + r);
       }
     }
+    if constexpr (kList) {
+      if (act) cand = key;
+    }
+    min_key<G>(best, key);
+  }
+
+  // The most negative of the lanes' candidates below -tol, key INT_MAX if none.
+  __device__ __forceinline__ void price_list(bool act, T tol, T& best, int& key) {
+    best = T(0);
+    key = INT_MAX;
+    if (act && cand != INT_MAX) {
+      const int a = cand >> 8, r = cand & 0xff;
+      const T d = cell(a, r) - pot(a) - pot(MP + r);
+      if (d < -tol) { best = d; key = cand; }
+    }
     min_key<G>(best, key);
   }
 
@@ -962,6 +984,7 @@ struct Lane {
     int st = kStOk;
     int done = 0, degen = 0, since = 64;
     bool bland = false, open = live;
+    if constexpr (kList) cand = INT_MAX;
     for (;;) {
       const bool due = open && since >= 64;
       if (__any_sync(kAll, due)) {  // the first round, then every 64 pivots
@@ -974,7 +997,12 @@ struct Lane {
       }
       T dE;
       int key;
-      price(open && !bland, dE, key);
+      if constexpr (kList) {
+        price_list(open && !bland, tol, dE, key);
+        if (__any_sync(kAll, open && !bland && key == INT_MAX)) price(open && !bland, dE, key);
+      } else {
+        price(open && !bland, dE, key);
+      }
       if (__any_sync(kAll, open && bland)) {
         T d2;
         int k2;
@@ -2324,12 +2352,12 @@ cudaError_t lane_launch(const ObjView& ob, const CentView& cv, long long seg_siz
   return cfg.certify ? screen(k_lane_screen<Sh, true, false>) : screen(k_lane_screen<Sh, false, false>);
 }
 
-// Every pair of the chunk in FP64 throughout.
-template <class Sh>
+// Every pair of the chunk in FP64 throughout, on an FP64 shape.
+template <class S8>
 cudaError_t lane_all64_launch(const ObjView& ob, const CentView& cv, long long seg_size, int K,
                               const SolveCfg& cfg, LaneArgs A, long long total_obj, long long work,
                               const ExactOut& X, cudaStream_t st) {
-  using S8 = LaneShape<Sh::G, Sh::L, Sh::MW, Sh::NPL, double>;
+  static_assert(S8::TS == 8, "an FP64 shape");
   A.nb = (cfg.nmax + 3) / 4;
   if (cfg.mmax > S8::MP || A.nb > S8::L) return cudaErrorInvalidConfiguration;
   A.warp_bytes = (int)lane_warp_bytes<S8>(cfg.mmax, A.nb);
@@ -2337,18 +2365,19 @@ cudaError_t lane_all64_launch(const ObjView& ob, const CentView& cv, long long s
                      cv, seg_size, K, cfg, A, total_obj, X.err);
 }
 
-// The shape's pair-list kernel, FP32 with the exact test or FP64 throughout.
-template <class Sh>
+// Pair lists: FP32 with the exact test (shape Sh) or FP64 throughout (S8).
+template <class Sh, class S8>
 cudaError_t lane_pairs_launch(const ObjView& ob, const CentView& cv, const PairJob& J,
                               const SolveCfg& cfg, cudaStream_t st) {
+  static_assert(Sh::TS == 4 && S8::TS == 8 && S8::MP >= Sh::MP && S8::L == Sh::L, "pair shapes");
   const int nb = (cfg.nmax + 3) / 4;
   if (cfg.mmax > Sh::MP || nb > Sh::L) return cudaErrorInvalidConfiguration;
-  const long long warps = (J.npairs + Sh::PW - 1) / Sh::PW;
   if (cfg.mode == 0) {
-    using S8 = LaneShape<Sh::G, Sh::L, Sh::MW, Sh::NPL, double>;
     const int wb = (int)lane_warp_bytes<S8>(cfg.mmax, nb);
-    return lane_blocks(k_lane_pairs<S8>, wb, cfg.sms, warps, st, ob, cv, J, cfg, nb, wb);
+    return lane_blocks(k_lane_pairs<S8>, wb, cfg.sms, (J.npairs + S8::PW - 1) / S8::PW, st, ob, cv,
+                       J, cfg, nb, wb);
   }
+  const long long warps = (J.npairs + Sh::PW - 1) / Sh::PW;
   const int wb = (int)lane_warp_bytes<Sh>(cfg.mmax, nb) + Sh::NS / 2 * Sh::PS;
   return lane_blocks(k_lane_pairs<Sh>, wb, cfg.sms, warps, st, ob, cv, J, cfg, nb, wb);
 }
