@@ -1829,6 +1829,14 @@ __device__ __forceinline__ int lane_verify(Lane<Sh>& P, bool go, bool value, cha
   return full && wkey != INT_MAX ? 1 : 0;
 }
 
+// Tests of a basis before its pair is left to the warp-per-pair kernel.  A test
+// builds the tile and the FP64 potentials anew (130 us on one warp at 32 x 32 in
+// 16 dimensions), where that kernel pivots on.  Ordinary bags need no pivot at
+// all; one whose supports nearly coincide took up to 20, and its launch waited
+// (4,000 pairs of merged centroids 7.4 -> 2.1 ms, ten rounds of 256 such bags
+// 39.6 -> 15.0; 2 tests 13.5, 6 tests 19.6).
+constexpr int kRepairs = 3;
+
 // The candidates of the chunk's objects (k_lane_merge's records) to their
 // labels and exact distances, as k_exact: a basis that is not optimal in FP64
 // takes its pivot here (the same entering cell) and is tested again; an object
@@ -1945,7 +1953,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       bool todo = go;
       int verdict = go ? 2 : 0;
 #pragma unroll 1
-      for (int att = 0; att < 24; ++att) {
+      for (int att = 0; att < kRepairs; ++att) {
         masses(todo);
         int key;
         float dE;
@@ -2185,7 +2193,7 @@ __global__ void __launch_bounds__(64, Sh::kMinBlocks)
       bool todo = act && s32 == kStOk;
       bool good = false;
 #pragma unroll 1
-      for (int att = 0; att < 24; ++att) {
+      for (int att = 0; att < kRepairs; ++att) {
         lane_reset<Sh>(P, todo, ob, o0, cv, c0);
         int key;
         float dE;
