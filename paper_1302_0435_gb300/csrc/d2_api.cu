@@ -582,14 +582,15 @@ int run_assign(d2_ctx* c, const ObjView& v, const CentView& cv, long long seg, i
                int mmax, const double* om, int* lab, double* d2o, double* terms, FlowOut fo,
                int* cand, const d2k::WarmStore* ws, Bins& bins,
                const d2k::TcWork* tw = nullptr, bool certify_all = false,
-               double* pair64 = nullptr, bool bags_ready = false) {
+               double* pair64 = nullptr, bool bags_ready = false, bool warp_exact = false) {
   const int nmax = std::max(c->nmax, 1);
   SolveCfg base = solve_cfg(c, mode, mmax);
+  base.lane_exact = !warp_exact;
   if (certify_all && mode == 1) base.certify = true;
   // full saved bases are the warp-per-pair screen's: a level that keeps them
   // takes that screen's cuts and tuned shapes (20,000 x 64 bags in trees of 34
-  // to 80 nodes, ten rounds of nearly every pair: 470 ms, by the lanes' cuts
-  // and untuned 488; certified 566 and 574)
+  // to 80 nodes, ten rounds of nearly every pair: 443 ms, by the lanes' cuts
+  // and untuned 461; certified 565 and 574)
   if (ws && ws->pos8) base.lanes = false;
   base.pair64 = pair64;
   const bool prune = prunes(c, base, cv);
@@ -1953,6 +1954,22 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     const bool store = budget > 0 && (meta_bytes + flow_bytes <= budget ||
                                       (meta_bytes <= budget && !cfg.certify));
     if (cfg.lanes && store && !pruned) cfg.lanes = false;
+    // A round of few small trees is the latency of a screened pair and an exact
+    // one, which a warp each has shorter: trees of at most 32 nodes take the
+    // lanes from 40 objects per SM (ten rounds of N x 64 image bags by warps and
+    // by lanes, ms: 1,000 2.2 and 3.2, 4,000 5.2 and 5.9, 7,000 5.8 and 5.7,
+    // 12,000 9.2 and 8.3; x 256 4,000 5.5 and 5.5; x 16 8,000 13.9 and 14.5,
+    // 20,000 7.8 and 6.5).  Larger trees gain from the lanes' start at any size.
+    if (cfg.lanes && store && ns <= 32 && n_l < 40LL * c->sms) cfg.lanes = false;
+    // The exact pass of a level's lane rounds goes on from the saved bases by
+    // warps, with centroids of up to 32 supports, where that is shorter: few bags
+    // (300 x 64 bags of 2 to 40 supports, 16 a centroid: 3.8 ms, by lanes 4.1;
+    // 1,500 5.4 both; 32 a centroid, 1,000 bags, 9.6 and 8.7, but 512 merged
+    // centroids 6.0 and 9.0), and merged levels, whose bags are centroids that
+    // nearly coincide, so that many a basis needs pivots in FP64 (256 x 64 of
+    // them 9.8 and 14.9 ms, 2,560 10.5 and 14.1; other bags, 2,000 x 64, 12.5 by
+    // warps and 10.7 by lanes).
+    const bool warp_exact = c->nmax <= 32 && (n_l < 1024 || level > 0);
     if (cfg.lanes && store && c->nmax <= 32 && npairs * ns >= (1LL << 26)) {
       ObjView first = cur;
       first.count = std::min<long long>(cur.count, 2048);
@@ -2034,7 +2051,7 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
       const bool capturing = cst == cudaStreamCaptureStatusActive;
       int rc2 = run_assign(c, cur, cv, seg, K, cfg.mode, cur_mmax, om, lab, ld2, lterms, fo, cand,
                            ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr,
-                           cfg.lanes || cfg.mode == 1);
+                           cfg.lanes || cfg.mode == 1, warp_exact && ws.par8);
       cudaError_t ue = cudaSuccess;
       if (rc2 == D2_OK && it < iters && alg1) {
         // Alg. 1 Step 1: support weights of every cluster of the level by the
@@ -2074,7 +2091,7 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
           // run the round directly instead
           if ((rc = run_assign(c, cur, cv, seg, K, cfg.mode, cur_mmax, om, lab, ld2, lterms, fo,
                                cand, ws.par8 ? &ws : nullptr, bins, nullptr, false, nullptr,
-                               cfg.lanes || cfg.mode == 1)))
+                               cfg.lanes || cfg.mode == 1, warp_exact && ws.par8)))
             return rc;
           if (it < iters)
             CK(d2k::update_locations(cur, om, lab, seg, K, fo, KT, loff, d, c->cent_ldt, l32, l64,

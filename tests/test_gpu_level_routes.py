@@ -74,3 +74,35 @@ def test_level_of_full_bases_is_tuned(d2):
     assert a[2]["kernel_launches"] > b[2]["kernel_launches"]
     assert np.array_equal(a[0], b[0])
     assert np.abs(a[1] - b[1]).max() <= 2.0 ** -22 * np.abs(b[1]).max()
+
+
+@pytest.mark.parametrize("n,top", [(16, 16), (8, 24)])
+def test_small_level_of_small_trees_runs_as_the_warp_screen(d2, n, top):
+    """Trees of at most 32 nodes, few objects: the launches and bits of a level
+    with its cold start fixed."""
+    rng = np.random.default_rng(n)
+    objs = bags(rng, rng.integers(2, top + 1, size=700), 6, 3.0)
+    cents = bags(rng, np.full(10, n), 6, 3.0)
+    a = run_level(d2, objs, cents, 5)
+    b = run_level(d2, objs, cents, 5, start_rule=d2.D2_START_RANKED)
+    assert a[2]["kernel_launches"] == b[2]["kernel_launches"]
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("N,seg,n,lo,top", [
+    (900, 900, 16, 2, 40),     # lane rounds, the exact pass by warps for want of bags
+    (1500, 1500, 16, 2, 40),   # lane rounds and exact pass, trees above 32 nodes
+    (7000, 7000, 16, 8, 16),   # lane rounds and exact pass
+    (2000, 500, 32, 2, 40),    # and a merged level, its exact pass by warps
+    (600, 200, 64, 16, 64),    # a merged level by lanes throughout
+])
+def test_level_routes_agree(d2, N, seg, n, lo, top):
+    """Continuous bags have one optimal plan: the routes' labels are equal and
+    the locations differ by FP32 units."""
+    rng = np.random.default_rng(N + n)
+    objs = bags(rng, rng.integers(lo, top + 1, size=N), 6, 3.0)
+    cents = bags(rng, np.full(8, n), 6, 3.0)
+    a = run_level(d2, objs, cents, 4, seg)
+    b = run_level(d2, objs, cents, 4, seg, start_rule=d2.D2_START_RANKED)
+    assert np.array_equal(a[0], b[0])
+    assert np.abs(a[1] - b[1]).max() <= 2.0 ** -22 * np.abs(b[1]).max()
