@@ -106,3 +106,57 @@ def test_level_routes_agree(d2, N, seg, n, lo, top):
     b = run_level(d2, objs, cents, 4, seg, start_rule=d2.D2_START_RANKED)
     assert np.array_equal(a[0], b[0])
     assert np.abs(a[1] - b[1]).max() <= 2.0 ** -22 * np.abs(b[1]).max()
+
+
+# 1 MiB holds a byte a tree node of every pair, not the 3 or 11 of the other
+# stores: the rounds run by lanes, warm, where the level is not pruned.
+# (N, K, most supports, supports of a centroid): N * K * (top + n) bytes
+WARM_LANES = [
+    (1200, 24, 16, 16),   # 32 nodes, from the staircase, exact pass by lanes
+    (400, 40, 32, 16),    # the other shapes start row by row; exact pass by warps
+    (400, 40, 16, 30),
+    (1100, 14, 24, 32),
+    (600, 16, 64, 32),
+    (300, 20, 64, 64),    # exact pass by lanes
+    (300, 20, 32, 60),
+]
+
+
+@pytest.mark.parametrize("kw", [{"no_prune": True}, {"certify": 1}])
+@pytest.mark.parametrize("N,K,top,n", WARM_LANES)
+def test_warm_rounds_of_all_pairs_by_lanes(d2, oracle_mod, N, K, top, n, kw):
+    """Every round's labels are nearest centroids of the locations the round
+    before left (read from a run of one round less), by the oracle."""
+    assert 3 * N * K * (top + n) > 2 ** 20 >= N * K * (top + n)
+    rng = np.random.default_rng(N + top + n)
+    sizes = rng.integers(max(1, top // 4), top + 1, size=N)
+    sizes[:3] = top, 1, top
+    objs = bags(rng, sizes, 5, 1.0)
+    cents = bags(rng, np.full(K, n), 5, 1.0)
+    cents = Bags(cents.loc, np.full(K * n, 1.0 / n, np.float32), cents.off, "f32", "f32")
+    runs = [run_level(d2, objs, cents, t, warm_budget_mib=1, **kw) for t in (2, 3, 4)]
+    whole = run_level(d2, objs, cents, 4, **kw)  # room for full bases: a warp per pair
+    # another screen: other launches, or other pivots from another start
+    screen = lambda r: (r[2]["kernel_launches"], r[2]["pivots_screened"])
+    assert screen(whole) != screen(runs[2])
+    for s in (whole[2], runs[2][2]):
+        assert s["pairs_screened"] == 4 * N * K
+        if kw.get("certify"):
+            assert s["pairs_certified"] >= 0.99 * 4 * N * K
+    for before, after in ((runs[0], runs[1]), (runs[1], runs[2])):
+        at = Bags(before[1].astype(np.float32), cents.w, cents.off, "f32", "f32")
+        _, _, ref = oracle_mod.assign(objs, at, nthreads=8, return_all=True)
+        got = ref[np.arange(N), after[0]]
+        assert np.all(got <= ref.min(axis=1) * (1 + 1e-7) + 1e-9)
+
+
+def test_pruned_rounds_by_lanes_with_little_memory(d2):
+    """Where only the byte store fits, and where none does, a pruned level has
+    the labels and locations of one with room."""
+    rng = np.random.default_rng(77)
+    objs = bags(rng, rng.integers(2, 33, size=1500), 5, 4.0)
+    cents = bags(rng, np.full(12, 30), 5, 4.0)  # 62 nodes: 1.1 MB of bytes
+    out = [run_level(d2, objs, cents, 4, warm_budget_mib=b) for b in (0, 2, 1)]
+    for o in out[1:]:
+        assert np.array_equal(o[0], out[0][0])
+        assert np.abs(o[1] - out[0][1]).max() <= 2.0 ** -22 * np.abs(out[0][1]).max()
