@@ -93,6 +93,8 @@ struct d2_ctx {
   // cold-start rule (the caller's)
   std::map<std::tuple<int, long long, int, int, int, int>, std::tuple<int, int, int>> tuned;
   int tuning_runs = 0;
+  // pairs of a chunk of the lanes' assignments (grow_cand)
+  long long chunk_pairs = 1LL << 24;
 };
 
 namespace {
@@ -270,7 +272,29 @@ SolveCfg solve_cfg(const d2_ctx* c, int mode, int mmax) {
   s.start = start_default(c);
   s.certify = mode == 1 && c->cfg.certify == D2_CERTIFY_ALL;
   s.lanes = c->cfg.start_rule == D2_START_AUTO;
+  s.max_pairs = c->chunk_pairs;
   return s;
+}
+
+// Scratch of an assignment.  The lanes keep 24 B and a basis a pair for the
+// pairs of a chunk (2^24 of 64 x 64: 2.4 GB); where that is more than half of
+// the free memory this context's chunks are halved, down to 2^18 pairs (a few
+// waves of them), so that a call fits that fitted without the lanes.
+int grow_cand(d2_ctx* c, int slot, long long count, long long K, int mmax, int nmax,
+              d2k::AssignRoute route, int** cand) {
+  const auto bytes = [&] {
+    route.max_pairs = c->chunk_pairs;
+    return (size_t)d2k::assign_scratch_ints(count, K, c->sms, mmax, nmax, route) * 4;
+  };
+  if (route.lanes && bytes() > c->slot[slot].n) {
+    size_t fr = 0, tot = 0;
+    CK(cudaMemGetInfo(&fr, &tot));
+    while (c->chunk_pairs > (1LL << 18) && bytes() > (fr + c->slot[slot].n) / 5 * 2)
+      c->chunk_pairs >>= 1;
+  }
+  int rc = D2_OK;
+  *cand = static_cast<int*>(grow(c, slot, bytes(), &rc));
+  return rc;
 }
 
 // Room for the FP32 bases of a two-launch exact solve (SolveCfg::tree);
@@ -824,9 +848,15 @@ int segment_impl(d2_ctx* c, const ObjView& v, int mmax, const double* om, long l
   double* dd = static_cast<double*>(grow(c, kSgD2, (size_t)N * 8, &rc));
   int* fcell = static_cast<int*>(grow(c, kSgCell, (size_t)(N * stride) * 4, &rc));
   double* fw = static_cast<double*>(grow(c, kSgFw, (size_t)(N * stride) * 8, &rc));
-  int* cand = static_cast<int*>(grow(c, kSgCand, (size_t)d2k::assign_scratch_ints(N, 2, c->sms, mmax, mmax) * 4, &rc));
   if (rc != D2_OK) return rc;
-  SolveCfg cfg = solve_cfg(c, mode_for(c, v.ldt), mmax);
+  const int mode = mode_for(c, v.ldt);
+  int* cand = nullptr;
+  d2k::AssignRoute route;
+  route.lanes = c->cfg.start_rule == D2_START_AUTO;
+  route.own_mass = true;
+  route.trees = mode == 0;
+  if ((rc = grow_cand(c, kSgCand, N, 2, mmax, mmax, route, &cand))) return rc;
+  SolveCfg cfg = solve_cfg(c, mode, mmax);
   cfg.nmax = mmax;  // the split centroids are bags of the data
   // the splits' centroids are FP64 (their FP32 copies are not exact), and
   // only their labels are used: no per-pair certificate
@@ -1374,8 +1404,11 @@ int assign_impl(d2_ctx* c, const d2_bags* objs, const double* omega, int32_t* la
     terms = static_cast<double*>(grow(c, kEpsTerms, (size_t)N * 8, &rc));
     if (rc != D2_OK) return rc;
   }
-  int* cand = static_cast<int*>(grow(c, kCand, (size_t)d2k::assign_scratch_ints(N, c->K, c->sms, mmax, c->nmax) * 4, &rc));
-  if (rc != D2_OK) return rc;
+  int* cand = nullptr;
+  d2k::AssignRoute route;
+  route.lanes = c->cfg.start_rule == D2_START_AUTO;
+  route.trees = true;
+  if ((rc = grow_cand(c, kCand, N, c->K, mmax, c->nmax, route, &cand))) return rc;
   if ((rc = check_bag_symbols(c, v))) return rc;
   const int mode = mode_for(c, objs->loc_dtype);
   Bins bins;
@@ -1746,10 +1779,14 @@ int d2_assign_multi(d2_ctx* const* ctxs, int32_t B, const d2_bags* objs, int32_t
     if ((rc = stage_bags(cb, &objs[b], kObjOff, kObjLoc, kObjW, &v[b]))) return rc;
     if ((rc = bag_bound(cb, &objs[b], v[b], &mmax[b]))) return rc;
     float* pair = static_cast<float*>(grow(cb, kMbPair, (size_t)N * K * 2 * 4, &rc));
-    int* cand = static_cast<int*>(grow(cb, kCand, (size_t)d2k::assign_scratch_ints(N, K, cb->sms, mmax[b], cb->nmax) * 4, &rc));
     int* tl = static_cast<int*>(grow(cb, kMbTmpLab, (size_t)N * 4, &rc));
     double* td = static_cast<double*>(grow(cb, kMbTmpD2, (size_t)N * 8, &rc));
     if (rc != D2_OK) return rc;
+    int* cand = nullptr;
+    d2k::AssignRoute route;
+    route.lanes = cb->cfg.start_rule == D2_START_AUTO;
+    route.own_mass = true;
+    if ((rc = grow_cand(cb, kCand, N, K, mmax[b], cb->nmax, route, &cand))) return rc;
     if ((rc = check_bag_symbols(cb, v[b]))) return rc;
     SolveCfg cfg = solve_cfg(cb, 1, mmax[b]);  // the FP32 screen, whatever the data type
     cfg.certify = false;  // the summed bounds decide; candidates are solved exactly below
@@ -1911,7 +1948,6 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     void* scr = grow(c, kUpd, d2k::update_scratch_bytes(n_l, KT), &rc);
     const size_t lpart_n = d2k::update_part_bytes(n_l, KT, d);
     double* lpart = static_cast<double*>(grow(c, kLvPart, lpart_n, &rc));
-    int* cand = static_cast<int*>(grow(c, kCand, (size_t)d2k::assign_scratch_ints(n_l, K, c->sms, cur_mmax, c->nmax) * 4, &rc));
     if (rc != D2_OK) return rc;
     k_replicate<<<blocks_for(M * Tc), 256, 0, c->stream>>>(c->c_loc32, c->c_loc64, c->c_Q, c->c_w64,
                                                            c->c_off, K, Tc, d, M, l32, l64, lQ, lw,
@@ -2004,6 +2040,11 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
                             0};
       }
     }
+    int* cand = nullptr;
+    d2k::AssignRoute route;
+    route.lanes = cfg.lanes;
+    route.trees = !ws.par8;  // (else the level's store holds them)
+    if ((rc = grow_cand(c, kCand, n_l, K, cur_mmax, c->nmax, route, &cand))) return rc;
     Bins bins;
     if (want_bins(c, cfg, n_l, cur_mmax) && (rc = make_bins(c, cur, &bins)))
       return rc;

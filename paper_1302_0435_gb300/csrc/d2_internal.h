@@ -289,14 +289,16 @@ struct PairJob {
 
 // Scratch of lane_screen behind the merged lists: byte offsets of the object
 // masses, flags and list starts, the pair list and the pair records, for
-// chunks of `objects` objects (about max_pairs pairs).
+// chunks of `objects` objects (about max_pairs pairs).  own_mass: with room for
+// the masses and flags (SolveCfg::mass null); the trees come last, so a screen
+// that saves none (no exact pass by lanes, or a level's own store) ends there.
 struct LaneScratch {
   long long objects;
   size_t mass, bad, start, list, rec, tree, fb, bytes;
   int tstride;
 };
 inline LaneScratch lane_scratch(long long count, long long K, int mmax, int nmax,
-                                long long max_pairs) {
+                                long long max_pairs, bool own_mass) {
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
   LaneScratch s;
   const long long n = count > 0 ? count : 1, k = K > 0 ? K : 1;
@@ -306,9 +308,9 @@ inline LaneScratch lane_scratch(long long count, long long K, int mmax, int nmax
   s.fb = b;        // (in the same place for every bound mmax of a batch)
   b += up((size_t)n * 4);
   s.mass = b;
-  b += up((size_t)n * (size_t)mmax * 8);
+  if (own_mass) b += up((size_t)n * (size_t)mmax * 8);
   s.bad = b;
-  b += up((size_t)n);
+  if (own_mass) b += up((size_t)n);
   s.start = b;
   b += up((size_t)s.objects * 8);
   s.list = b;
@@ -460,11 +462,20 @@ constexpr int kCandCap = 16;
 // count, centroids, lower ends, best upper end, certified FP64 value of that centroid
 constexpr int kItemInts = 2 + 2 * kCandCap + 2;
 constexpr int kMergedInts = 1 + kCandCap + 2;  // count, centroids, certified FP64 value
+// Ints of an assignment's scratch: by lanes (LaneScratch), or the screening
+// items of a warp per pair.
+struct AssignRoute {
+  bool lanes = false;
+  bool own_mass = false;  // lanes: the call brings no masses
+  bool trees = false;     // lanes: bases saved for the exact pass
+  long long max_pairs = 1LL << 24;
+};
 inline long long assign_scratch_ints(long long count, long long K, int sms, int mmax, int nmax,
-                                     long long max_pairs = 1LL << 24) {
-  const long long items = (count + (long long)sms * 256) * kItemInts + 4;
-  const long long lanes = (long long)(lane_scratch(count, K, mmax, nmax, max_pairs).bytes + 256) / 4 + 1;
-  return 4 + ((count * kMergedInts + 3) & ~3LL) + std::max(items, lanes);
+                                     const AssignRoute& r) {
+  const long long merged = 4 + ((count * kMergedInts + 3) & ~3LL);
+  if (!r.lanes) return merged + (count + (long long)sms * 256) * kItemInts + 4;
+  const LaneScratch s = lane_scratch(count, K, mmax, nmax, r.max_pairs, r.own_mass);
+  return merged + (long long)((r.trees ? s.bytes : s.tree) + 256) / 4 + 1;
 }
 cudaError_t cost_matrix(const ObjView& ob, const CentView& cv, long long i, long long j, int mode,
                         double* C, cudaStream_t st);

@@ -232,7 +232,7 @@ cudaError_t lane_screen(const ObjView& ob, const CentView& cv, long long seg_siz
                         const TcWork* tw, const WarmStore* ws, ExactOut X) {
   const long long total_obj = cfg.dev_lo ? ob.count : (cfg.nobj >= 0 ? cfg.nobj : ob.count);
   if (total_obj <= 0) return cudaSuccess;
-  const LaneScratch ls = lane_scratch(ob.count, K, cfg.mmax, cfg.nmax, cfg.max_pairs);
+  const LaneScratch ls = lane_scratch(ob.count, K, cfg.mmax, cfg.nmax, cfg.max_pairs, !cfg.mass);
   int* merged = cand + 4;
   unsigned char* mem = reinterpret_cast<unsigned char*>(cand) + lane_scratch_offset(ob.count);
   LaneArgs A{};
@@ -329,7 +329,7 @@ cudaError_t lane_axes(const ObjView& ob, const SolveCfg& cfg, cudaStream_t st) {
 }
 
 void lane_fallback(const ObjView& ob, int K, int* cand, SolveCfg* cfg) {
-  const LaneScratch ls = lane_scratch(ob.count, K, cfg->mmax, cfg->nmax, cfg->max_pairs);
+  const LaneScratch ls = lane_scratch(ob.count, K, cfg->mmax, cfg->nmax, cfg->max_pairs, !cfg->mass);
   unsigned char* mem = reinterpret_cast<unsigned char*>(cand) + lane_scratch_offset(ob.count);
   const long long* ctr = reinterpret_cast<const long long*>(mem);
   cfg->oidx = reinterpret_cast<const int*>(mem + ls.fb);

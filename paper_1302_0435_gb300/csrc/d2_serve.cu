@@ -145,8 +145,16 @@ struct d2_server {
   long long chunk_objects() const {
     return std::max<long long>(1, kChunkPairs / std::max<long long>(K, 1));
   }
+  bool prunes(const std::shared_ptr<Request>& r) const {
+    return cm.mu && mode == 1 && r->ldt != D2_F64;
+  }
   long long scratch_ints(const std::shared_ptr<Request>& r) const {
-    return d2k::assign_scratch_ints(r->count, K, sms, r->mmax, nmax, chunk_objects() * K);
+    d2k::AssignRoute route;
+    route.lanes = lanes;
+    route.own_mass = !prunes(r);
+    route.trees = true;
+    route.max_pairs = chunk_objects() * K;
+    return d2k::assign_scratch_ints(r->count, K, sms, r->mmax, nmax, route);
   }
   void free_moments() {
     cudaFree(cm.mu); cudaFree(cm.var); cudaFree(cm.muT32); cudaFree(cm.cn);
@@ -174,7 +182,7 @@ bool d2_server::launch(Slot& s, const std::shared_ptr<Request>& r) {
       !grow_dev(&s.d_lab, &s.n_lab, (size_t)N * 4 + 16) ||
       !grow_dev(&s.d_d2, &s.n_d2, (size_t)N * 8 + 16) ||
       !grow_dev(&s.d_cand, &s.n_cand, (size_t)scratch_ints(r) * 4 + 16) ||
-      (cm.mu && (!grow_dev(&s.d_mu, &s.n_mu, (size_t)N * r->dim * 8 + 16) ||
+      (prunes(r) && (!grow_dev(&s.d_mu, &s.n_mu, (size_t)N * r->dim * 8 + 16) ||
                  !grow_dev(&s.d_var, &s.n_var, (size_t)N * 8 + 16) ||
                  !grow_dev(&s.d_mass, &s.n_mass, (size_t)N * r->mmax * 8 + 16) ||
                  !grow_dev(&s.d_bad, &s.n_bad, (size_t)N + 16) ||
@@ -211,7 +219,7 @@ bool d2_server::launch(Slot& s, const std::shared_ptr<Request>& r) {
   cfg.lanes = lanes;
   cfg.max_pairs = chunk_objects() * K;
   d2k::FlowOut fo{nullptr, nullptr, 0};
-  if (cm.mu && cfg.mode == 1) {
+  if (prunes(r)) {
     // skip the pairs that cannot be an object's argmin (d2k::prune_keep)
     const int kw = (int)((K + 31) / 32);
     if (d2k::bag_prep(ob, nullptr, r->mmax, s.d_mass, s.d_bad, r->mmax, s.d_mu, s.d_var, st) !=
