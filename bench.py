@@ -163,11 +163,14 @@ def measured_peaks():
 
 
 def kernel_source_hash():
-    """Hash of the sources of the screening kernel's translation units
-    (k_lane_screen's shapes are instantiated in d2_lane_*.cu from these files)."""
+    """Hash of the sources of the screening kernel: the shapes
+    (k_lane_screen is instantiated in d2_lane_*.cu), their launches and the
+    headers they include."""
     h = hashlib.sha256()
     cs = os.path.join(ROOT, "paper_1302_0435_gb300", "csrc")
-    for f in ("d2_lane.cu", "d2_lane.cuh", "d2_solve.cuh", "d2_solver.cuh", "d2_internal.h"):
+    units = sorted(f for f in os.listdir(cs) if f.startswith("d2_lane") and f.endswith(".cu"))
+    for f in units + ["d2_lane.cuh", "d2_solve.cuh", "d2_solver.cuh", "d2_internal.h"]:
+        h.update(f.encode())
         with open(os.path.join(cs, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
