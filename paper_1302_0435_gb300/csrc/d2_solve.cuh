@@ -231,15 +231,15 @@ __device__ void prefix_in_order(const Grp<G>& g, const long long* pre, const int
 // A projection as the ranks compare it: one that is not a number (a support or
 // a mean that is not finite, squares that overflow) counts as the largest.
 // Unordered values would share rank 0 and leave other ranks without a support,
-// and the staircases take ranks and supports as indices.
+// and the staircases take ranks and supports as indices.  (Made where the
+// projection is stored: in the rank function the 32-node screens came out 2 to
+// 3 % slower, a certified level of 100,000 x 64 264.5 and 270.4 ms.)
 __device__ __forceinline__ float order_value(float x) { return fminf(x, INFINITY); }
 
-// stable ranks of proj[0..cnt) (as order_value makes them; ties to the smaller
-// index): always a permutation
+// stable ranks of proj[0..cnt) (order_value's; ties to the smaller index):
+// always a permutation
 template <int G>
-__device__ void rank_by_proj(const Grp<G>& g, float* proj, int cnt, int* rank, int* id) {
-  for (int a = g.lane; a < cnt; a += G) proj[a] = order_value(proj[a]);
-  g.sync();
+__device__ void rank_by_proj(const Grp<G>& g, const float* proj, int cnt, int* rank, int* id) {
   for (int a = g.lane; a < cnt; a += G) {
     const float v = proj[a];
     int r = 0;
@@ -317,7 +317,7 @@ __device__ void order_rows(const Grp<G>& g, const PairMem<float>& s, const ObjVi
   for (int a = g.lane; a < m; a += G) {
     float dot = 0.f;
     for (int k = 0; k < d; ++k) dot = fmaf(ldx<float>(ob.loc, ob.ldt, (o0 + a) * d + k) - s.mu[k], s.dir[k], dot);
-    s.proj[a] = dot;
+    s.proj[a] = order_value(dot);
   }
   g.sync();
   rank_by_proj<G>(g, s.proj, m, s.rrank, s.rid);
@@ -331,7 +331,7 @@ __device__ void order_cols(const Grp<G>& g, const PairMem<float>& s, const float
   for (int r = g.lane; r < n; r += G) {
     float dot = 0.f;
     for (int k = 0; k < d; ++k) dot = fmaf(y32[(long long)r * d + k] - s.mu[k], s.dir[k], dot);
-    s.proj[r] = dot;
+    s.proj[r] = order_value(dot);
   }
   g.sync();
   rank_by_proj<G>(g, s.proj, n, s.crank, s.cid);
