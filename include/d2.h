@@ -94,10 +94,15 @@ extern "C" {
 /* cold-start basis of the simplex (d2_config.start_rule) */
 #define D2_START_AUTO 0    /* the lane solver (several pairs per warp) with its own
                               start: rows in turn take the cheapest columns left, on
-                              costs less their column's mean.  What it does not take
-                              (short pair lists, d2_update_weights' members, the
-                              rounds of a level without pruning that keeps bases)
-                              starts by Vogel's rule for 64 supports, else RANKED */
+                              costs less their column's mean (in a level that keeps
+                              bases, trees of at most 32 nodes start as RANKED).  A
+                              warp per pair, which starts by Vogel's rule for 64
+                              supports, else RANKED, solves what the lanes do not
+                              take: short pair lists, d2_update_weights' members, and
+                              the rounds of a level that keeps full bases: one that
+                              is not pruned or keeps most of its pairs (then the
+                              faster of both starts, timed on large bins), or one of
+                              few small trees */
 #define D2_START_RANKED 1  /* northwest staircase in principal-direction order, one
                               warp per pair */
 #define D2_START_VOGEL 2   /* Vogel's approximation (largest-penalty line first), one
@@ -161,7 +166,7 @@ typedef struct {
     int32_t precision;          /* D2_PREC_* ; 0 = AUTO */
     int32_t pivot_budget;       /* pivots per pair = pivot_budget*(m+n); 0 = 64 */
     int32_t group_lanes;        /* the warp-per-pair screen (a fixed start_rule, or a
-                                   level without pruning):
+                                   level that keeps full bases):
                                    0 = its launch shape (threads per block, screening
                                    items per SM) is autotuned per support bin on large
                                    batches; 32 = the default shape, no tuning; other
@@ -206,12 +211,13 @@ typedef struct {
                                    every round solves every member from a cold start */
     int32_t warm_budget_mib;    /* device memory d2_cluster_level may take for the bases it
                                    keeps between rounds; 0 = 40% of the free memory.  The
-                                   store is 1 B per tree node and pair (the flows are
-                                   rebuilt on reload); without pruning 11 B where
-                                   that fits; with a fixed start_rule 11 B, or, when
-                                   only its trees fit, 3 B (same results, slower; not
-                                   with D2_CERTIFY_ALL); below that the rounds start
-                                   cold */
+                                   lane solver's store is 1 B per tree node and pair
+                                   (the flows are rebuilt on reload).  A fixed
+                                   start_rule, and in D2_START_AUTO the levels that
+                                   keep a warp per pair, take 11 B, or, when only the
+                                   trees fit, 3 B (same results, slower; not with
+                                   D2_CERTIFY_ALL); AUTO falls back to the lanes'
+                                   store, and below that the rounds start cold */
 } d2_config;
 
 /*

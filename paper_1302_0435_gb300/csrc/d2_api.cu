@@ -532,6 +532,9 @@ int bins_to_host(d2_ctx* c, Bins* b) {
 // long as each of them has several waves of pairs to solve (a launch of one
 // wave costs a pair's latency, 50 to 150 us); small trees of a batch below
 // 2^17 objects go together, and only the mask widths part the larger ones.
+// (2^17 stands for the waves, which follow the pairs kept and are not known
+// here: all cuts at 24,001 x 255 uneven objects 51.5 -> 50.3 ms, at smaller
+// batches slower.)
 // The warp-per-pair kernels change with the nodes per lane only.
 int size_cuts(bool lanes, long long count, int mmax, int nmax, int* cut) {
   static const int steps[] = {4, 8, 12, 16, 24, 32, 48};
@@ -1983,10 +1986,13 @@ int d2_cluster_level_ex(d2_ctx* c, const d2_bags* objs, const double* omega, int
     // image-like level of 200,000 bags 519 ms against 930, Gaussian bags with
     // 42 % of the pairs kept 63 against 68, 10 % kept 126 against 82, 3 % kept
     // 21 against 16.  So with room for the bases such rounds keep a warp per
-    // pair; with centroids of more than 32 supports the lanes win whatever is
-    // kept (587 against 330 ms).  The share that is kept is counted on the
-    // first objects, where the level has enough tree nodes (2^26: 7 ms and more)
-    // to pay for the count's wait.
+    // pair: unpruned levels, whatever their centroids (above 32 supports not
+    // compared), and pruned ones of up to 32 supports a centroid with more than
+    // 0.3 of the pairs kept (a line between the 10 and 42 % measured, no closer).
+    // Pruned with larger centroids, the lanes win at 87 % kept (587 against 330
+    // ms).  The kept share is counted on the first 2,048 objects only, where the
+    // level has enough tree nodes (2^26: 7 ms and more) to pay for the count's
+    // wait.
     const bool store = budget > 0 && (meta_bytes + flow_bytes <= budget ||
                                       (meta_bytes <= budget && !cfg.certify));
     if (cfg.lanes && store && !pruned) cfg.lanes = false;

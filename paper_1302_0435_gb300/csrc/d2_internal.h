@@ -123,7 +123,7 @@ struct SolveCfg {
   const long long* dev_lo = nullptr;
   const long long* dev_hi = nullptr;
   // the screen runs several pairs per warp (lane_screen) unless the caller
-  // fixed a cold-start rule or saved bases are in play; `screened`: it has
+  // fixed a cold-start rule or a level keeps full bases; `screened`: it has
   // run and the merged lists are in place
   bool lanes = false;
   bool screened = false;
@@ -136,7 +136,9 @@ struct SolveCfg {
   const long long* mass = nullptr;
   const unsigned char* bad = nullptr;
   int mstride = 0;
-  bool lane_exact = true;  // the exact pass too (needs centroids whose FP32 copy is exact)
+  // the exact pass too (needs centroids whose FP32 copy is exact; not for a
+  // level's rounds that are shorter with k_exact)
+  bool lane_exact = true;
   long long max_pairs = 1LL << 24;  // pairs of one lane_screen chunk
   int start = 0;              // cold start basis: 0 ranked northwest staircase, 1 Vogel
   // per-pair screen output (optional): pair_out[2*(i*K + j)] = FP32 value,

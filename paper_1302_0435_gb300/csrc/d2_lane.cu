@@ -188,10 +188,12 @@ size_t lane_scratch_offset(long long count) {
 }
 
 // The lanes per pair follow the launch's bounds: enough column lanes for the
-// centroid's blocks of 4 supports, enough lanes that a pair's nodes are 4 to
+// centroid's blocks of 4 supports, enough lanes that a pair's nodes are 3 to
 // 8 per lane, and few enough that the pairs the shared memory holds (about
 // 1.6 KB at 16 x 16, 3.4 KB at 16 x 32, 21 KB at 64 x 64) still give each
-// scheduler several warps.
+// scheduler several warps.  The narrower shapes (a6, a7, b5, b7, c6, e5, f3)
+// are the wide ones of their lanes with fewer row slots, and so less shared
+// memory a pair.
 static cudaError_t lane_dispatch(const ObjView& ob, const CentView& cv, long long seg_size, int K,
                                  const SolveCfg& cfg, const LaneArgs& A, long long total_obj,
                                  long long work, const ExactOut& X, cudaStream_t st) {

@@ -359,13 +359,14 @@ struct Lane {
   // far apart cost nearly f(a) + g(r), and what tells the columns apart is
   // the rest.  The end that runs out (the row on a tie) leaves and hangs from
   // the other; the last line of either kind is the root and takes the rest.
-  // Flows are the int64 masses, so the basis is exactly feasible.  Dantzig
-  // pivots from there, against the other rules on the workload laws (CPU
-  // model, mean per pair): image 8.7 (ranked staircase 22.1, Vogel 13.7, the
-  // same rule on the plain costs 21.1), uneven 5.8 (18.7, 10.4, 18.7), serving
-  // 36 (117, 55, 84), high_dim 52 (217, 55, 76), sequences 11.2 (37, 9.8,
-  // 13.8).  A step reads one row of the tile, where Vogel's rule keeps the two
-  // best of every line.  flow holds the masses, D the singletons.
+  // Flows are the int64 masses, so the basis is exactly feasible.  Pivots a
+  // pair from there, and a warp per pair's from the ranked staircase and from
+  // Vogel's rule (all pairs of some thousand bags of each workload law, by the
+  // library's counters with start_rule 0, 1 and 2): image 8.8 (22.3), uneven
+  // 5.6 (19.8, 12.7), serving 35.7 (126, 69.6), high_dim 56.2 (247, 67.2),
+  // sequences 15.4 (52.9, 14.1).  A step reads one row of the tile, where
+  // Vogel's rule keeps the two best of every line.  flow holds the masses, D
+  // the singletons.
   __device__ __forceinline__ void start_rows(const V4<T>& vm) {
     unsigned long long ra = m >= 64 ? ~0ull : ((1ull << m) - 1ull);
     unsigned long long ca = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
